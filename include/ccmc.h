@@ -252,7 +252,7 @@ ccmc_status ccmc_phase_times(ccmc_ctx *ctx, double *ms, int64_t *launches, int32
 
 /* ---- Batched form: many independent contexts stepped together ----------
  * Every phase of the step is one kernel launch over all replicas that share
- * a determinant word count and precision (a CUDA grid dimension indexes the
+ * a Hamiltonian kind and precision (a CUDA grid dimension indexes the
  * replica), and the whole step is captured once in a CUDA graph and replayed.
  * The cluster sampler, the bulk of the work, is one persistent launch whose
  * blocks take shares of the replicas' samples from a plan written on the

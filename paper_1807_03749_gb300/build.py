@@ -17,7 +17,8 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libccmc.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-UNITS = ["ccmc_step.cu", "ccmc_api.cu", "ccmc_dist.cu"] + [f"ccmc_step_k{k}.cu" for k in range(1, 7)]
+UNITS = ["ccmc_step.cu", "ccmc_api.cu", "ccmc_dist.cu"] + [f"ccmc_step_{kind}_{r}.cu" for kind in ("gas", "generic")
+                                                           for r in ("f64", "f32")]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

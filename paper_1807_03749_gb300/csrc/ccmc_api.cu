@@ -27,8 +27,11 @@ constexpr double PI_D = 3.14159265358979323846;
 struct HostSys {
     int kind = 0, nel = 0, nso = 0, lmax = 0, nw = 0;
     double rs = 0.0, L = 0.0, ecore = 0.0;
-    int npw = 0, nmax = 0, side = 0;
-    std::vector<int> kv, grid;
+    int npw = 0, nmax = 0;
+    std::vector<int> kv, kv4;
+    std::vector<short> lin, grid;   // see SysDev
+    int mid = 0;
+    std::vector<unsigned> pairs;
     std::vector<double> tkin, vtab, h1, eri;
     int norb = 0;
     std::vector<u64> rank_tab;
@@ -40,7 +43,7 @@ struct HostSys {
     double inv_pgen_ueg = 0.0, inv_pgen_single[2] = {0, 0}, inv_pgen_double[3] = {0, 0, 0};
     std::vector<double> fock;     // reference Fock diagonal per spin-orbital
     // FP32 form
-    std::vector<float> tkin_f, vtab_f, h1_f, eri_f, fock_f;
+    std::vector<float> vtab_f, h1_f, eri_f, fock_f;
 };
 
 void fill_binom(HostSys &h)
@@ -145,10 +148,18 @@ bool build_ueg(HostSys &h)
             h.kv[3 * i + c] = v[i][c];
             h.nmax = std::max(h.nmax, std::abs(v[i][c]));
         }
-    h.side = 2 * h.nmax + 1;
-    h.grid.assign((size_t)h.side * h.side * h.side, -1);
-    for (int i = 0; i < h.npw; i++)
-        h.grid[((h.kv[3 * i] + h.nmax) * h.side + (h.kv[3 * i + 1] + h.nmax)) * h.side + (h.kv[3 * i + 2] + h.nmax)] = i;
+    // cube of every k_i + k_j - k_a (components within 3 nmax)
+    const int side = 6 * h.nmax + 1;
+    h.mid = ((3 * h.nmax) * side + 3 * h.nmax) * side + 3 * h.nmax;
+    h.grid.assign((size_t)side * side * side, -1);
+    h.lin.resize(h.npw);
+    h.kv4.resize(h.npw);
+    for (int i = 0; i < h.npw; i++) {
+        const int *k = &h.kv[3 * i];
+        h.lin[i] = (short)((k[0] * side + k[1]) * side + k[2]);
+        h.grid[h.mid + h.lin[i]] = (short)i;
+        h.kv4[i] = (int)((unsigned)(k[0] & 255) | ((unsigned)(k[1] & 255) << 8) | ((unsigned)(k[2] & 255) << 16));
+    }
     h.L = h.rs * std::cbrt((4.0 * PI_D * (double)h.nel) / 3.0);
     h.tkin.resize(h.nso);
     for (int p = 0; p < h.nso; p++) {
@@ -280,7 +291,7 @@ enum : unsigned {
     BAD_COUNT = 1u, BAD_RANGE = 2u, BAD_SZ = 4u, BAD_MOMENTUM = 8u, BAD_LEVEL = 16u, BAD_FIRST = 32u, BAD_ORDER = 64u
 };
 
-// Uploaded list: row-major determinants -> the list's word-major layout,
+// Uploaded list: row-major determinants -> the list's holes and particles,
 // each entry checked (electron count, orbital range, the reference's S_z,
 // zero total momentum for the gas, truncation level, HF first), then its
 // key and diagonal energy.
@@ -297,7 +308,6 @@ __global__ void k_load_list(SysDev s, ListView L, const u64 *rows, i64 i0, i64 i
         for (int w = 0; w < K; w++) {
             const u64 x = rows[i * K + w];
             d.w[w] = x;
-            L.bits[w * L.cap + i] = x;
             pc += __popcll(x);
             na += __popcll(x & alpha);
             holes += __popcll(s.hf[w] & ~x);
@@ -318,13 +328,12 @@ __global__ void k_load_list(SysDev s, ListView L, const u64 *rows, i64 i0, i64 i
         if (kx != 0 || ky != 0 || kz != 0) e |= BAD_MOMENTUM;
         if (holes > s.lmax) e |= BAD_LEVEL;
         if (i == 0 && holes != 0) e |= BAD_FIRST;
-        if (e == 0) {
-            L.key[i] = rank_key(s, d);
-            L.diag[i] = holes == 0 ? 0.0 : diag_rel<K, R>(s, d);
-        } else {
-            L.key[i] = 0;
-            L.diag[i] = 0.0;
-        }
+        Exc x = {0, 0, 0};
+        if (e == 0) x = exc_from_words(s, d);
+        L.h[i] = pack_h(x);
+        L.p[i] = x.p;
+        L.key[i] = rank_key(s, x);
+        L.diag[i] = x.n == 0 ? 0.0 : s.kind == 0 ? diag_rel<R, true>(s, x) : diag_rel<R, false>(s, x);
         b |= e;
     }
     if (b) atomicOr(bad, b);
@@ -341,11 +350,13 @@ __global__ void k_check_order(const u64 *key, i64 n, unsigned *bad)
 
 // the list in row-major order for download
 template <int K>
-__global__ void k_store_list(ListView L, u64 *rows, i64 n)
+__global__ void k_store_list(SysDev s, ListView L, u64 *rows, i64 n)
 {
-    for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (i64)gridDim.x * blockDim.x)
+    for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (i64)gridDim.x * blockDim.x) {
+        const Det<K> d = words_from_exc<K>(s, exc_of(L.h[i], L.p[i]));
 #pragma unroll
-        for (int w = 0; w < K; w++) rows[i * K + w] = L.bits[w * L.cap + i];
+        for (int w = 0; w < K; w++) rows[i * K + w] = d.w[w];
+    }
 }
 
 // the device check of entries [i0, i1) of an upload (key and Delta E computed)
@@ -380,12 +391,12 @@ cudaError_t store_list(ccmc_ctx *ctx, const ListView &L, i64 n)
 {
     const int g = (int)std::min<i64>(4096, (n + 255) / 256 + 1);
     switch (ctx->sc.K) {
-    case 1: k_store_list<1><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
-    case 2: k_store_list<2><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
-    case 3: k_store_list<3><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
-    case 4: k_store_list<4><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
-    case 5: k_store_list<5><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
-    default: k_store_list<6><<<g, 256, 0, ctx->stream>>>(L, ctx->io, n); break;
+    case 1: k_store_list<1><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
+    case 2: k_store_list<2><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
+    case 3: k_store_list<3><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
+    case 4: k_store_list<4><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
+    case 5: k_store_list<5><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
+    default: k_store_list<6><<<g, 256, 0, ctx->stream>>>(ctx->sc.sys, L, ctx->io, n); break;
     }
     return cudaGetLastError();
 }
@@ -455,7 +466,6 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     h.ehf_rel = host_diag(h, hfocc);
     host_fock(h);
     // FP32 tables: rounded from the FP64 ones
-    h.tkin_f.assign(h.tkin.begin(), h.tkin.end());
     h.vtab_f.assign(h.vtab.begin(), h.vtab.end());
     h.h1_f.assign(h.h1.begin(), h.h1.end());
     h.eri_f.assign(h.eri.begin(), h.eri.end());
@@ -479,6 +489,14 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
             h.inv_pgen_double[c] = ((double)(h.npairs * h.ndcase[c]) * (double)(h.ns + h.nd)) / (double)h.nd;
     }
 
+    {
+        // pairs x < y by index y (y - 1) / 2 + x: of electrons, and of the
+        // empty spin-orbitals of one spin
+        const u64 np = std::max(h.npairs, std::max(h.ndcase[0], h.ndcase[1]));
+        for (unsigned y = 1; h.pairs.size() < np; y++)
+            for (unsigned x = 0; x < y; x++) h.pairs.push_back(x | (y << 16));
+    }
+
     // capacities
     double tgt = std::max(params->target_pop, params->d0_init);
     u64 key_bound = h.nvranks * h.cocc;
@@ -487,11 +505,10 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     // spawned records per step: about one per attempt; multi-spawn makes several attempts per cluster
     const double per = params->multispawn ? 8.0 : (params->fnc ? 3.0 : 2.0);
     ctx->spawn_cap = params->spawn_capacity ? (i64)params->spawn_capacity : (i64)(per * tgt + 65536.0);
-    // the original sampler on a generic Hamiltonian queues its clusters for
-    // the attempts kernel (their attempts are long and divergent); the
-    // trajectory is the same either way
-    const bool buffered = !params->multispawn && ham->kind == CCMC_GENERIC;
-    ctx->cl_cap = params->multispawn ? (i64)(3.0 * tgt + 65536.0) : (buffered ? (i64)(4.0 * tgt + 65536.0) : 1);
+    // multi-spawn buffers its clusters; a generic Hamiltonian's other samplers
+    // count them and are bounded by a capacity as well
+    const bool count_clusters = !params->multispawn && ham->kind == CCMC_GENERIC;
+    ctx->cl_cap = params->multispawn ? (i64)(3.0 * tgt + 65536.0) : (count_clusters ? (i64)(4.0 * tgt + 65536.0) : 1);
     if (ctx->list_cap < 2 || ctx->spawn_cap < 1 || ctx->spawn_cap >= (i64)0xFFFFFFFFLL) {
         delete ctx;
         return CCMC_ERR_ARG;
@@ -530,10 +547,11 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     };
     if (h.kind == CCMC_UEG) {
         s.nmax = h.nmax;
-        s.side = h.side;
-        s.grid = (const int *)upload(h.grid.data(), h.grid.size() * sizeof(int));
+        s.mid = h.mid;
+        s.lin = (const short *)upload(h.lin.data(), h.lin.size() * sizeof(short));
+        s.grid = (const short *)upload(h.grid.data(), h.grid.size() * sizeof(short));
+        s.kv4 = (const int *)upload(h.kv4.data(), h.kv4.size() * sizeof(int));
         s.kv = (const int *)upload(h.kv.data(), h.kv.size() * sizeof(int));
-        s.tkin = (const double *)upload(h.tkin.data(), h.tkin.size() * sizeof(double));
         s.vtab = (const double *)upload(h.vtab.data(), h.vtab.size() * sizeof(double));
         s.inv_pgen_ueg = h.inv_pgen_ueg;
     } else {
@@ -552,10 +570,10 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
         s.inv_pgen_single[1] = h.inv_pgen_single[1];
     }
     s.npairs = h.npairs;
+    s.pairs = (const unsigned *)upload(h.pairs.data(), h.pairs.size() * sizeof(unsigned));
     s.nvirt = h.nvirt;
     s.rank_tab = (const u64 *)upload(h.rank_tab.data(), h.rank_tab.size() * sizeof(u64));
     if (h.kind == CCMC_UEG) {
-        s.tkin_f = (const float *)upload(h.tkin_f.data(), h.tkin_f.size() * sizeof(float));
         s.vtab_f = (const float *)upload(h.vtab_f.data(), h.vtab_f.size() * sizeof(float));
     } else {
         s.h1_f = (const float *)upload(h.h1_f.data(), h.h1_f.size() * sizeof(float));
@@ -579,7 +597,7 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     rp.replica = params->replica;
     rp.fnc = params->fnc ? 1 : 0;
     rp.multispawn = params->multispawn ? 1 : 0;
-    rp.buffered = buffered ? 1 : 0;
+    rp.count_clusters = count_clusters ? 1 : 0;
     rp.a_thresh_one = params->a_thresh == 1.0 ? 1 : 0;
     rp.direct = (params->flags & CCMC_SORT_ALL) ? 0 : 1;
     rp.nranks = params->n_ranks > 1 ? params->n_ranks : 1;
@@ -615,13 +633,14 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     Shapes &sh = ctx->sc.sh;
     sh.scan_grid = std::min(1024, 2 * nsm);
-    sh.work_grid = 4 * nsm;   // one wave of the sampler and attempt kernels (four blocks per SM)
+    sh.work_grid = SAMPLE_BLOCKS_PER_SM * nsm;   // one wave of the sampler and attempt kernels
     sh.sort_grid = 2 * nsm;
     sh.key_bits = bits_for(key_bound);
     sh.digit_bits = params->radix_bits ? params->radix_bits : MAX_DIGIT_BITS;
     sh.enum_slots = sh.scan_grid + sh.work_grid;
     sh.nranks = rp.nranks;
     ctx->sc.K = h.nw;
+    ctx->sc.gas = h.kind == CCMC_UEG;
     ctx->sc.fp32 = params->precision == CCMC_FP32;
 
     // lists
@@ -629,7 +648,8 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     for (int b = 0; b < 2; b++) {
         ListView &L = ctx->sc.list[b];
         L.cap = ctx->list_cap;
-        L.bits = al.arr<u64>((size_t)K * L.cap);
+        L.h = al.arr<u64>(L.cap);
+        L.p = al.arr<u64>(L.cap);
         L.key = al.arr<u64>(L.cap);
         L.pop = al.arr<i64>(L.cap);
         L.diag = al.arr<double>(L.cap);
@@ -642,14 +662,17 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     }
     ClusterBuf &cl = ctx->sc.cl;
     cl.cap = ctx->cl_cap;
-    cl.bits = al.arr<u64>((size_t)K * cl.cap);
-    cl.catt = al.arr<double>(cl.cap);
-    cl.index = al.arr<u64>(cl.cap);
-    cl.end = al.arr<i64>(cl.cap);
+    const i64 cl_rows = params->multispawn ? cl.cap : 1;   // only multi-spawn stores clusters
+    cl.h = al.arr<u64>(cl_rows);
+    cl.p = al.arr<u64>(cl_rows);
+    cl.catt = al.arr<double>(cl_rows);
+    cl.index = al.arr<u64>(cl_rows);
+    cl.end = al.arr<i64>(cl_rows);
     WorkArrays &wa = ctx->sc.wa;
     const i64 lc = ctx->list_cap;
     wa.picks = al.arr<PickEntry>(lc);
-    wa.bucket_bits = 10;
+    wa.href = al.arr<double>(lc);
+    wa.bucket_bits = 18;
     while (wa.bucket_bits < 24 && (1LL << wa.bucket_bits) < lc / 2) wa.bucket_bits++;
     wa.bucket = al.arr<int>(((size_t)1 << wa.bucket_bits) + 1);
     wa.att_end = al.arr<i64>(lc);
@@ -1176,8 +1199,8 @@ __global__ void k_batch_shift(const StepArgs *A, int n, const double *shift)
 }
 
 struct BatchGroup {
-    int K = 1;
-    bool fp32 = false, multi = false;
+    int K = 0;                      // words per determinant (simulated distribution only, else 0)
+    bool gas = true, fp32 = false, multi = false;
     std::vector<int> members;
     StepArgs *d_args = nullptr;
     int key_bits = 1;
@@ -1274,7 +1297,7 @@ cudaError_t batch_launch(ccmc_batch *b, const Shapes &base)
         plan.wmax = b->lim.work_grid;
         plan.grid = b->flat_grid;
         const cudaEvent_t *ev = b->profile ? &b->events[8 * gi] : nullptr;
-        cudaError_t e = launch_group(g.d_args, (int)g.members.size(), g.K, g.fp32, sh, g.multi, b->stream,
+        cudaError_t e = launch_group(g.d_args, (int)g.members.size(), g.K, g.gas, g.fp32, sh, g.multi, b->stream,
                                      b->launches, ev, &plan);
         if (e != cudaSuccess) return e;
     }
@@ -1380,15 +1403,19 @@ ccmc_status ccmc_batch_create(ccmc_ctx **ctxs, int32_t n, void *cuda_stream, ccm
             delete b;
             return CCMC_ERR_CUDA;
         }
-        bool multi = c->prm.fnc || c->prm.multispawn || c->sc.prm.buffered;
+        bool multi = c->prm.fnc || c->prm.multispawn;
         bool fp32 = c->sc.fp32;
+        // the kernels differ by kind and precision; the owner hash of the
+        // simulated distribution also by the word count
+        const int K = c->sc.prm.nranks > 1 ? c->sc.K : 0;
         BatchGroup *g = nullptr;
         for (BatchGroup &x : b->groups)
-            if (x.K == c->sc.K && x.fp32 == fp32) g = &x;
+            if (x.K == K && x.gas == c->sc.gas && x.fp32 == fp32) g = &x;
         if (!g) {
             b->groups.emplace_back();
             g = &b->groups.back();
-            g->K = c->sc.K;
+            g->K = K;
+            g->gas = c->sc.gas;
             g->fp32 = fp32;
         }
         g->multi = g->multi || multi;

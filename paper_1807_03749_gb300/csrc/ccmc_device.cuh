@@ -20,6 +20,7 @@ typedef long long i64;
 
 constexpr int MAXK = 6;            // words per determinant (M <= 384)
 constexpr int RANK_STRIDE = 384;   // row stride of the rank tables (positions < M)
+constexpr int MAX_EXC = 6;         // largest excitation level of a collapsed cluster (lmax + 2)
 constexpr double FIX_ONE = 65536.0;
 
 // Philox counter tags (bits 56..63 of counter word 1).
@@ -49,13 +50,19 @@ struct SysDev {
     u64 valid[MAXK];     // bits < nso
     u64 virt[MAXK];      // bits in [nel, nso)
     // UEG
-    int nmax, side;
-    const int *grid;     // (2 nmax + 1)^3 -> spatial orbital or -1
+    int nmax;
+    // k_i + k_j - k_a has components within 3 nmax, so a cube of side
+    // 6 nmax + 1 holds every sum: lin[] is a wave's linear offset in it and
+    // grid[mid + lin_i + lin_j - lin_a] the spatial orbital there, or -1
+    int mid;
+    const short *lin;    // per spatial orbital
+    const short *grid;
     const int *kv;       // 3 ints per spatial orbital
-    const double *tkin;  // per spin-orbital
+    const int *kv4;      // the same packed as signed bytes (x, y, z, 0)
     const double *vtab;  // Coulomb by integer |n|^2
     double inv_pgen_ueg;
     u64 npairs, nvirt;
+    const unsigned *pairs;   // pair index -> x | y << 16 (x < y, index = y (y - 1) / 2 + x)
     // generic integrals
     int norb;
     const double *h1;
@@ -71,7 +78,7 @@ struct SysDev {
     int lmin_exc;        // smallest excitation level of any non-reference list entry
     const double *fock;  // reference Fock diagonal per spin-orbital
     // FP32 form: tables rounded from the FP64 ones
-    const float *tkin_f, *vtab_f, *h1_f, *eri_f;
+    const float *vtab_f, *h1_f, *eri_f;
     const float *fock_f;
     float inv_pgen_ueg_f;
     float inv_pgen_single_f[2];
@@ -81,14 +88,12 @@ struct SysDev {
 // table selection by real type
 template <typename R> struct Tab;
 template <> struct Tab<double> {
-    static __device__ __forceinline__ const double *tkin(const SysDev &s) { return s.tkin; }
     static __device__ __forceinline__ const double *vtab(const SysDev &s) { return s.vtab; }
     static __device__ __forceinline__ const double *h1(const SysDev &s) { return s.h1; }
     static __device__ __forceinline__ const double *eri(const SysDev &s) { return s.eri; }
     static __device__ __forceinline__ const double *fock(const SysDev &s) { return s.fock; }
 };
 template <> struct Tab<float> {
-    static __device__ __forceinline__ const float *tkin(const SysDev &s) { return s.tkin_f; }
     static __device__ __forceinline__ const float *vtab(const SysDev &s) { return s.vtab_f; }
     static __device__ __forceinline__ const float *h1(const SysDev &s) { return s.h1_f; }
     static __device__ __forceinline__ const float *eri(const SysDev &s) { return s.eri_f; }
@@ -159,6 +164,71 @@ __host__ __device__ __forceinline__ R4 draw(u64 k0, u64 k1, u64 it, u64 tag, u64
     return philox(it, (tag << 56) | index, block, 0, k0, k1);
 }
 
+// The draws of one step: the counter's first word (the iteration), its last
+// (zero) and the key are the same for every draw, so the products of the first
+// round, one product of the second and all round keys are computed once per
+// block and kept in shared memory.  A draw is then one product plus eight full
+// rounds.  Bound by the integer multiplier (a 64 x 64 -> 128-bit product is
+// four 32-bit wide multiplies of about four issue slots each): 371 issue slots
+// per draw at full warps against 504 of the plain loop (148 M draws, 367 and
+// 498 us on one GB300; limb and carry-chain forms of the product were slower).
+struct PhiloxStep {
+    u64 k0;          // key word 0
+    u64 u_hi, u_lo;  // second round's product of the third word, key xor-ed into its high half
+    u64 v;           // second round: low half of the iteration's product xor key
+    ulonglong2 rk[8];   // round keys of rounds 3-10
+};
+
+// every thread of the block calls; the caller synchronises
+__device__ __forceinline__ void philox_step_init(PhiloxStep &ps, u64 it, u64 k0, u64 k1)
+{
+    const u64 m0 = 0xD2E7470EE14C6C93ULL, m1 = 0xCA5A826395121157ULL;
+    const u64 w0 = 0x9E3779B97F4A7C15ULL, w1 = 0xBB67AE8584CAA73BULL;
+    const int t = threadIdx.x;
+    if (t < 8) ps.rk[t] = make_ulonglong2(k0 + (u64)(t + 2) * w0, k1 + (u64)(t + 2) * w1);
+    if (t == 8) {
+        const u64 n2 = __umul64hi(it, m0) ^ k1;   // third word after the first round
+        ps.k0 = k0;
+        ps.u_hi = __umul64hi(n2, m1) ^ (k0 + w0);
+        ps.u_lo = n2 * m1;
+        ps.v = (it * m0) ^ (k1 + w1);
+    }
+}
+
+// draw(k0, k1, it, tag, index, block) with the block's first-round product
+// (hi1, lo1) = block * m1 given
+__device__ __forceinline__ R4 step_draw_at(const PhiloxStep &ps, u64 tag, u64 index, u64 hi1, u64 lo1)
+{
+    const u64 m0 = 0xD2E7470EE14C6C93ULL, m1 = 0xCA5A826395121157ULL;
+    u64 hi, lo;
+    mulhilo64(((tag << 56) | index) ^ ps.k0 ^ hi1, m0, hi, lo);
+    u64 c0 = ps.u_hi ^ lo1, c1 = ps.u_lo, c2 = hi ^ ps.v, c3 = lo;
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+        const ulonglong2 k = ps.rk[r];
+        u64 hi0, lo0, hi1r, lo1r;
+        mulhilo64(c0, m0, hi0, lo0);
+        mulhilo64(c2, m1, hi1r, lo1r);
+        c0 = hi1r ^ c1 ^ k.x;
+        c2 = hi0 ^ c3 ^ k.y;
+        c1 = lo1r;
+        c3 = lo0;
+    }
+    R4 o;
+    o.v[0] = c0;
+    o.v[1] = c1;
+    o.v[2] = c2;
+    o.v[3] = c3;
+    return o;
+}
+
+__device__ __forceinline__ R4 step_draw(const PhiloxStep &ps, u64 tag, u64 index, u64 block)
+{
+    u64 hi1, lo1;
+    mulhilo64(block, 0xCA5A826395121157ULL, hi1, lo1);
+    return step_draw_at(ps, tag, index, hi1, lo1);
+}
+
 // ---------------------------------------------------------------------------
 // The paper's distribution of excitors over N_p processors (Sec. III, Eq.
 // ccmc_dist), simulated on one GPU: a determinant hash (Philox-4x64-10 under
@@ -195,192 +265,198 @@ __device__ __forceinline__ double unif(u64 r) { return (double)(r >> 11) * 0x1p-
 __device__ __forceinline__ u64 below(u64 r, u64 n) { return __umul64hi(r, n); }
 
 // ---------------------------------------------------------------------------
-// Bit strings
+// Determinants as excitation lists
+//
+// The kernels hold a determinant as its difference from HF: the holes (empty
+// spin-orbitals below N) and the particles (occupied ones from N), each an
+// ascending list of 10-bit fields in one 64-bit word (positions < 384, at
+// most six of each); unused fields are zero, and bits 60-63 of the hole word
+// are the level n, the number of fields in either list.  Everything the step
+// asks of a determinant -- the k-th occupied or empty orbital, parities,
+// levels, rank keys, matrix elements -- costs a few integer operations per
+// hole and particle in registers.  The bit-string form needs population
+// counts (8 issue slots each on sm_103a; an attempt used about 40) and
+// indexes its words by position, which put them in local memory.  The lists
+// also make every kernel independent of the number of words.  Their loops are
+// short and kept rolled: the sampler's loop is bound by instruction fetch
+// when it is unrolled.
 // ---------------------------------------------------------------------------
 
-template <int K>
-__device__ __forceinline__ int bit(const Det<K> &d, int p) { return (int)((d.w[p >> 6] >> (p & 63)) & 1ULL); }
+constexpr int FB = 10;                            // bits per field
+constexpr u64 FIELDS = (1ULL << 60) - 1ULL;       // the six fields of a word
+constexpr u64 FIELD_LSB = 0x0004010040100401ULL;  // lowest bit of every field
 
-template <int K>
-__device__ __forceinline__ void flip(Det<K> &d, int p) { d.w[p >> 6] ^= 1ULL << (p & 63); }
+struct Exc {
+    u64 h, p;   // fields only
+    int n;
+};
 
-// number of set bits strictly below position p
-template <int K>
-__device__ __forceinline__ int count_below(const Det<K> &d, int p)
-{
-    int c = 0, wp = p >> 6;
-#pragma unroll
-    for (int i = 0; i < K; i++) {
-        if (i < wp) c += __popcll(d.w[i]);
-        else if (i == wp) c += __popcll(d.w[i] & ((1ULL << (p & 63)) - 1ULL));
-    }
-    return c;
-}
+__host__ __device__ __forceinline__ int field(u64 x, int m) { return (int)(x >> (FB * m)) & 1023; }
 
-// position of the k-th (0-based) set bit of x; x must have more than k bits
-__device__ __forceinline__ int kth_bit64(u64 x, int k)
-{
-    int pos = 0, c;
-    c = __popc((unsigned)x);
-    if (k >= c) { k -= c; x >>= 32; pos += 32; }
-    c = __popc((unsigned)(x & 0xFFFFULL));
-    if (k >= c) { k -= c; x >>= 16; pos += 16; }
-    c = __popc((unsigned)(x & 0xFFULL));
-    if (k >= c) { k -= c; x >>= 8; pos += 8; }
-    c = __popc((unsigned)(x & 0xFULL));
-    if (k >= c) { k -= c; x >>= 4; pos += 4; }
-    c = __popc((unsigned)(x & 0x3ULL));
-    if (k >= c) { k -= c; x >>= 2; pos += 2; }
-    if (k >= (int)(x & 1ULL)) pos += 1;
-    return pos;
-}
-
-__device__ __forceinline__ u64 spin_mask(int spin)
-{
-    return spin < 0 ? ~0ULL : (spin == 0 ? 0x5555555555555555ULL : 0xAAAAAAAAAAAAAAAAULL);
-}
-
-// k-th occupied spin-orbital (ascending)
-template <int K>
-__device__ __forceinline__ int kth_occupied(const Det<K> &d, int k)
-{
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        int c = __popcll(d.w[w]);
-        if (k < c) return 64 * w + kth_bit64(d.w[w], k);
-        k -= c;
-    }
-    return -1;
-}
-
-// k-th empty spin-orbital (ascending), optionally of one spin
-template <int K>
-__device__ __forceinline__ int kth_empty(const SysDev &s, const Det<K> &d, u64 k, int spin)
-{
-    u64 sm = spin_mask(spin);
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 m = ~d.w[w] & s.valid[w] & sm;
-        u64 c = (u64)__popcll(m);
-        if (k < c) return 64 * w + kth_bit64(m, (int)k);
-        k -= c;
-    }
-    return -1;
-}
-
-// excitation level relative to HF = number of holes
-template <int K>
-__device__ __forceinline__ int level_of(const SysDev &s, const Det<K> &d)
+// number of the first cnt fields below v
+__device__ __forceinline__ int fields_below(u64 x, int cnt, int v)
 {
     int c = 0;
-#pragma unroll
-    for (int w = 0; w < K; w++) c += __popcll(s.hf[w] & ~d.w[w]);
+#pragma unroll 1
+    for (int m = 0; m < cnt; m++, x >>= FB) c += ((int)x & 1023) < v ? 1 : 0;
     return c;
 }
 
-template <int K>
-__device__ __forceinline__ bool is_hf(const SysDev &s, const Det<K> &d)
+__device__ __forceinline__ bool has_field(u64 x, int cnt, int v)
 {
-    bool e = true;
-#pragma unroll
-    for (int w = 0; w < K; w++) e = e && (d.w[w] == s.hf[w]);
+    bool e = false;
+#pragma unroll 1
+    for (int m = 0; m < cnt; m++, x >>= FB) e = e || ((int)x & 1023) == v;
     return e;
+}
+
+// v inserted before field c
+__device__ __forceinline__ u64 insert_at(u64 x, int c, int v)
+{
+    const u64 low = (1ULL << (FB * c)) - 1ULL;
+    return (x & low) | ((u64)v << (FB * c)) | ((x & ~low) << FB);
+}
+
+// field c taken out
+__device__ __forceinline__ u64 remove_at(u64 x, int c)
+{
+    const u64 low = (1ULL << (FB * c)) - 1ULL;
+    return (x & low) | ((x >> FB) & ~low);
+}
+
+// parity of the sum of the fields
+__device__ __forceinline__ int sum_parity(u64 x)
+{
+    u64 y = x & FIELD_LSB;
+    unsigned z = (unsigned)(y ^ (y >> 30));   // fields 3-5 onto 0-2
+    z ^= (z >> FB) ^ (z >> (2 * FB));
+    return (int)(z & 1u);
+}
+
+__device__ __forceinline__ u64 pack_h(const Exc &e) { return e.h | ((u64)e.n << 60); }
+
+__device__ __forceinline__ Exc exc_of(u64 hn, u64 p)
+{
+    Exc e;
+    e.h = hn & FIELDS;
+    e.p = p & FIELDS;
+    e.n = (int)(hn >> 60);
+    return e;
+}
+
+// bit string -> lists (level at most MAX_EXC; fields beyond are dropped)
+template <int K>
+__device__ __forceinline__ Exc exc_from_words(const SysDev &s, const Det<K> &d)
+{
+    Exc e = {0, 0, 0};
+    int np = 0;
+#pragma unroll
+    for (int w = 0; w < K; w++) {
+        for (u64 m = s.hf[w] & ~d.w[w]; m; m &= m - 1) {
+            if (e.n < MAX_EXC) e.h |= (u64)(64 * w + __ffsll((long long)m) - 1) << (FB * e.n);
+            e.n++;
+        }
+        for (u64 m = d.w[w] & s.virt[w]; m; m &= m - 1) {
+            if (np < MAX_EXC) e.p |= (u64)(64 * w + __ffsll((long long)m) - 1) << (FB * np);
+            np++;
+        }
+    }
+    return e;
+}
+
+template <int K>
+__device__ __forceinline__ Det<K> words_from_exc(const SysDev &s, const Exc &e)
+{
+    Det<K> d;
+#pragma unroll
+    for (int w = 0; w < K; w++) d.w[w] = s.hf[w];
+    u64 h = e.h, p = e.p;
+    for (int m = 0; m < e.n; m++, h >>= FB, p >>= FB) {
+        const int a = (int)h & 1023, b = (int)p & 1023;
+#pragma unroll
+        for (int w = 0; w < K; w++) {
+            if ((a >> 6) == w) d.w[w] &= ~(1ULL << (a & 63));
+            if ((b >> 6) == w) d.w[w] |= 1ULL << (b & 63);
+        }
+    }
+    return d;
+}
+
+// parity of the number of occupied spin-orbitals below x: the core below x
+// without the holes there, or the whole core without the holes and the
+// particles below x
+__device__ __forceinline__ int occ_below_parity(const SysDev &s, const Exc &e, int x)
+{
+    const bool core = x < s.nel;
+    return (core ? x : s.nel + e.n) + fields_below(core ? e.h : e.p, e.n, x);
 }
 
 // s_D = <D|c_D|HF>: annihilating the holes h_1 < ... < h_n of HF in ascending
 // order meets h_m - (m-1) occupied orbitals below h_m; creating the particles
 // in descending order meets the N - n remaining electrons each time.  The sign
-// is therefore (-1)^(sum h_m - n(n-1)/2 + n(N-n)).
-template <int K>
-__device__ __forceinline__ int excitor_sign(const SysDev &s, const Det<K> &d)
+// is therefore (-1)^(sum h_m - n(n-1)/2 + n(N-n)); this is its parity bit.
+__device__ __forceinline__ int sign_parity(const SysDev &s, int hsum_parity, int n)
 {
-    int n = 0, hsum = 0;
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 m = s.hf[w] & ~d.w[w];
-        while (m) {
-            int b = __ffsll((long long)m) - 1;
-            hsum += 64 * w + b;
-            n++;
-            m &= m - 1;
-        }
-    }
-    int par = hsum - n * (n - 1) / 2 + n * (s.nel - n);
-    return (par & 1) ? -1 : 1;
+    return (hsum_parity + n * (n - 1) / 2 + n * (s.nel - n)) & 1;
 }
 
-// Applies excitor c_e (given by its determinant) to cur: annihilators of its
-// holes in ascending order, then creators of its particles in descending
-// order, accumulating the parity of the occupied orbitals passed.  Returns
-// false if the product vanishes.
-template <int K>
-__device__ __forceinline__ bool apply_excitor(const SysDev &s, const Det<K> &e, Det<K> &cur, int &parity)
+__device__ __forceinline__ int sign_parity(const SysDev &s, const Exc &e)
 {
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 m = s.hf[w] & ~e.w[w];
-        while (m) {
-            int p = 64 * w + (__ffsll((long long)m) - 1);
-            if (!bit(cur, p)) return false;
-            parity += count_below(cur, p);
-            flip(cur, p);
-            m &= m - 1;
+    return sign_parity(s, sum_parity(e.h), e.n);
+}
+
+// Applies excitor e to cur: annihilators of its holes in ascending order,
+// then creators of its particles in descending order, accumulating the parity
+// of the occupied orbitals passed.  Returns false if the product vanishes (an
+// orbital emptied or filled twice; so does a repeated excitor).
+__device__ __forceinline__ bool apply_excitor(const SysDev &s, const Exc &e, Exc &cur, int &parity)
+{
+    bool ok = true;
+    // x - c core orbitals below a hole x with c holes below it; N - n + c
+    // orbitals below a particle with c particles below it (n: all holes of the
+    // product), the larger ones of e being created first
+    const int ntot = cur.n + e.n;
+#pragma unroll 1
+    for (int m = 0; m < 2 * e.n; m++) {
+        const bool hole = m < e.n;
+        const int x = hole ? field(e.h, m) : field(e.p, 2 * e.n - 1 - m);
+        const u64 list = hole ? cur.h : cur.p;
+        u64 f = list;
+        int c = 0;
+#pragma unroll 1
+        for (int q = cur.n + (hole ? m : m - e.n); q > 0; q--, f >>= FB) {
+            const int y = (int)f & 1023;
+            c += y < x ? 1 : 0;
+            ok = ok && y != x;
         }
+        const u64 with = insert_at(list, c, x);
+        if (hole) cur.h = with;
+        else cur.p = with;
+        parity += c + (hole ? x : s.nel - ntot);
     }
-#pragma unroll
-    for (int w = K - 1; w >= 0; w--) {
-        u64 m = e.w[w] & s.virt[w];
-        while (m) {
-            int b = 63 - __clzll((long long)m);
-            int p = 64 * w + b;
-            if (bit(cur, p)) return false;
-            parity += count_below(cur, p);
-            flip(cur, p);
-            m &= ~(1ULL << b);
-        }
-    }
-    return true;
+    cur.n = ntot;
+    return ok;
 }
 
 // ---------------------------------------------------------------------------
 // Rank key: key = rank_V * C_O - rank_H (order-preserving on level <= l)
 // ---------------------------------------------------------------------------
 
-template <int K>
-__device__ __forceinline__ u64 rank_key(const SysDev &s, const Det<K> &d)
+__device__ __forceinline__ u64 rank_key(const SysDev &s, const Exc &e)
 {
     u64 rv = 0, rh = 0;
-    int c = 0;
-#pragma unroll
-    for (int w = K - 1; w >= 0; w--) {
-        u64 m = d.w[w] & s.virt[w];
-        while (m) {
-            int b = 63 - __clzll((long long)m);
-            rv += __ldg(&s.rank_tab[c * RANK_STRIDE + (64 * w + b - s.nel)]);
-            c++;
-            m &= ~(1ULL << b);
-        }
-    }
-    c = 0;
-#pragma unroll
-    for (int w = K - 1; w >= 0; w--) {
-        u64 m = s.hf[w] & ~d.w[w];
-        while (m) {
-            int b = 63 - __clzll((long long)m);
-            rh += __ldg(&s.rank_tab[c * RANK_STRIDE + (64 * w + b)]);
-            c++;
-            m &= ~(1ULL << b);
-        }
+#pragma unroll 1
+    for (int c = 0; c < e.n; c++) {
+        const int m = e.n - 1 - c;   // digits from the top
+        rv += __ldg(&s.rank_tab[c * RANK_STRIDE + (field(e.p, m) - s.nel)]);
+        rh += __ldg(&s.rank_tab[c * RANK_STRIDE + field(e.h, m)]);
     }
     return rv * s.cocc - rh;
 }
 
-template <int K>
-__device__ __forceinline__ Det<K> unrank_key(const SysDev &s, u64 key)
+__device__ __forceinline__ Exc unrank_key(const SysDev &s, u64 key)
 {
-    Det<K> d;
-#pragma unroll
-    for (int w = 0; w < K; w++) d.w[w] = s.hf[w];
+    Exc e = {0, 0, 0};
     u64 rv = (key + s.cocc - 1) / s.cocc;
     u64 rh = rv * s.cocc - key;
     // digit c of a rank: the largest position q below the previous digit with
@@ -396,7 +472,8 @@ __device__ __forceinline__ Det<K> unrank_key(const SysDev &s, u64 key)
             else hi = mid - 1;
         }
         rv -= __ldg(&t[lo]);
-        flip(d, lo + s.nel);
+        e.p = (e.p << FB) | (u64)(lo + s.nel);   // the digits descend
+        e.n++;
         top = lo;
     }
     top = s.nel;
@@ -409,21 +486,24 @@ __device__ __forceinline__ Det<K> unrank_key(const SysDev &s, u64 key)
             else hi = mid - 1;
         }
         rh -= __ldg(&t[lo]);
-        flip(d, lo);
+        e.h = (e.h << FB) | (u64)lo;
         top = lo;
     }
-    return d;
+    return e;
 }
 
 // ---------------------------------------------------------------------------
-// Matrix elements (Slater-Condon rules)
+// Matrix elements (Slater-Condon rules).  GAS selects the Hamiltonian kind at
+// compile time: the two kinds' element and generator code is never both in
+// one kernel's loop.
 // ---------------------------------------------------------------------------
 
+// |k_p - k_q|^2 of two spin-orbitals' plane waves
 __device__ __forceinline__ int ueg_n2(const SysDev &s, int p, int q)
 {
-    const int *a = s.kv + 3 * (p >> 1), *b = s.kv + 3 * (q >> 1);
-    int dx = __ldg(a) - __ldg(b), dy = __ldg(a + 1) - __ldg(b + 1), dz = __ldg(a + 2) - __ldg(b + 2);
-    return dx * dx + dy * dy + dz * dz;
+    const int a = __ldg(&s.kv4[p >> 1]), b = __ldg(&s.kv4[q >> 1]);
+    const int d = (int)__vsub4((unsigned)a, (unsigned)b);   // each |component| <= 2 nmax < 128
+    return __dp4a(d, d, 0);
 }
 
 template <typename R>
@@ -434,158 +514,131 @@ __device__ __forceinline__ R eri_at(const SysDev &s, int p, int q, int r, int t)
 }
 
 // physicists' <pq|rs> for a momentum-conserving (UEG) or any (generic) quadruple
-template <typename R>
+template <typename R, bool GAS>
 __device__ __forceinline__ R g2(const SysDev &s, int p, int q, int r, int t)
 {
     if (((p ^ r) & 1) || ((q ^ t) & 1)) return R(0);
-    if (s.kind == 0) return __ldg(&Tab<R>::vtab(s)[ueg_n2(s, p, r)]);
+    if (GAS) return __ldg(&Tab<R>::vtab(s)[ueg_n2(s, p, r)]);
     return eri_at<R>(s, p >> 1, r >> 1, q >> 1, t >> 1);
 }
 
 // <pq||pq> for p != q in the precision R: gas, minus the exchange Coulomb
 // term (callers skip opposite spins, whose pair term is the omitted q = 0
 // Coulomb term); molecule, (pp|qq) minus (pq|qp) for equal spins.
-template <typename R>
+template <typename R, bool GAS>
 __device__ __forceinline__ R pair_ex(const SysDev &s, int p, int q)
 {
-    if (s.kind == 0) return -__ldg(&Tab<R>::vtab(s)[ueg_n2(s, p, q)]);
+    if (GAS) return -__ldg(&Tab<R>::vtab(s)[ueg_n2(s, p, q)]);
     const int P = p >> 1, Q = q >> 1;
     R t = eri_at<R>(s, P, P, Q, Q);
     if (((p ^ q) & 1) == 0) t = t - eri_at<R>(s, P, Q, Q, P);
     return t;
 }
 
-__device__ __forceinline__ bool pair_zero(const SysDev &s, int p, int q)
+template <bool GAS>
+__device__ __forceinline__ bool pair_zero(int p, int q)
 {
-    return s.kind == 0 && ((p ^ q) & 1);
+    return GAS && ((p ^ q) & 1);
 }
 
 // H_DD - E_HF from the excitation of D relative to HF: holes H and particles
 // P ascending, sum_P F_a - sum_H F_i + sum_{i<j in H} <ij||ij>
 // + sum_{a<b in P} <ab||ab> - sum_{a in P, i in H} <ai||ai>, in this order,
-// in the precision R and promoted to double.  D is within the truncation
-// (at most 8 holes are read).
-template <int K, typename R>
-__device__ __forceinline__ double diag_rel(const SysDev &s, const Det<K> &d)
+// in the precision R and promoted to double.
+template <typename R, bool GAS>
+__device__ __noinline__ double diag_rel(const SysDev &s, const Exc d)
 {
-    int hol[8], par[8], nh = 0, np = 0;
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 hm = s.hf[w] & ~d.w[w];
-        u64 pm = d.w[w] & ~s.hf[w];
-        while (hm) {
-            if (nh < 8) hol[nh++] = 64 * w + (__ffsll((long long)hm) - 1);
-            hm &= hm - 1;
-        }
-        while (pm) {
-            if (np < 8) par[np++] = 64 * w + (__ffsll((long long)pm) - 1);
-            pm &= pm - 1;
-        }
-    }
     const R *f = Tab<R>::fock(s);
+    const int n = d.n;
     R e = R(0);
-    for (int x = 0; x < np; x++) e = e + __ldg(&f[par[x]]);
-    for (int x = 0; x < nh; x++) e = e - __ldg(&f[hol[x]]);
-    for (int x = 0; x < nh; x++)
-        for (int y = x + 1; y < nh; y++)
-            if (!pair_zero(s, hol[x], hol[y])) e = e + pair_ex<R>(s, hol[x], hol[y]);
-    for (int x = 0; x < np; x++)
-        for (int y = x + 1; y < np; y++)
-            if (!pair_zero(s, par[x], par[y])) e = e + pair_ex<R>(s, par[x], par[y]);
-    for (int x = 0; x < np; x++)
-        for (int y = 0; y < nh; y++)
-            if (!pair_zero(s, par[x], hol[y])) e = e - pair_ex<R>(s, par[x], hol[y]);
+#pragma unroll 1
+    for (int x = 0; x < 2 * n; x++) {
+        const R t = __ldg(&f[x < n ? field(d.p, x) : field(d.h, x - n)]);
+        e = x < n ? e + t : e - t;
+    }
+    // pairs of holes, pairs of particles, particle-hole pairs
+#pragma unroll 1
+    for (int k = 0; k < 3; k++) {
+        const u64 u = k == 0 ? d.h : d.p, v = k == 1 ? d.p : d.h;
+#pragma unroll 1
+        for (int x = 0; x < n; x++)
+#pragma unroll 1
+            for (int y = k == 2 ? 0 : x + 1; y < n; y++) {
+                const int a = field(u, x), b = field(v, y);
+                if (pair_zero<GAS>(a, b)) continue;
+                const R t = pair_ex<R, GAS>(s, a, b);
+                e = k == 2 ? e - t : e + t;
+            }
+    }
     return (double)e;
 }
 
 // <bra|H|ket> for determinants differing by one or two spin-orbitals.
 // holes i<j are in ket only, particles a<b in bra only; gamma is the phase of
 // a+_a a+_b a_j a_i |ket> = gamma |bra>.  Computed in R, returned as double.
-template <int K, typename R>
-__device__ double h_offdiag(const SysDev &s, const Det<K> &ket, int nh, int i, int j, int a, int b)
+template <typename R, bool GAS>
+__device__ __forceinline__ double h_offdiag(const SysDev &s, const Exc &ket, int nh, int i, int j, int a, int b)
 {
-    Det<K> cur = ket;
-    int par = count_below(cur, i);
-    flip(cur, i);
-    if (nh == 2) {
-        par += count_below(cur, j);
-        flip(cur, j);
-        par += count_below(cur, b);
-        flip(cur, b);
+    const bool dbl = GAS || nh == 2;
+    // i removed below j; i and j removed below b and a, b added above a
+    int par = i < a ? 1 : 0;
+    u64 at = (u64)i | ((u64)a << FB);
+    if (dbl) {
+        par += 1 + (j < a ? 1 : 0) + (i < b ? 1 : 0) + (j < b ? 1 : 0);
+        at |= ((u64)j << (2 * FB)) | ((u64)b << (3 * FB));
     }
-    par += count_below(cur, a);
-    if (nh == 2) {
-        R v1 = g2<R>(s, a, b, i, j);
-        R v2 = g2<R>(s, a, b, j, i);
+#pragma unroll 1
+    for (int m = dbl ? 4 : 2; m > 0; m--, at >>= FB) par += occ_below_parity(s, ket, (int)at & 1023);
+    if (dbl) {
+        R v1 = g2<R, GAS>(s, a, b, i, j);
+        R v2 = g2<R, GAS>(s, a, b, j, i);
         R d = v1 - v2;
         return (double)((par & 1) ? -d : d);
     }
-    if (s.kind == 0 || ((i ^ a) & 1)) return 0.0;
-    int A = a >> 1, I = i >> 1;
+    if ((i ^ a) & 1) return 0.0;
+    const int A = a >> 1, I = i >> 1;
     R acc = __ldg(&Tab<R>::h1(s)[A * s.norb + I]);
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 m = ket.w[w];
-        while (m) {
-            int k = 64 * w + (__ffsll((long long)m) - 1);
-            m &= m - 1;
-            if (k == i) continue;
-            int Kk = k >> 1;
-            R t = eri_at<R>(s, A, I, Kk, Kk);
-            if (((a ^ k) & 1) == 0) t = t - eri_at<R>(s, A, Kk, Kk, I);
-            acc = acc + t;
+    // the other occupied spin-orbitals, ascending: the core without the holes, then the particles
+    u64 holes = ket.h, parts = ket.p;
+    int left = ket.n;
+#pragma unroll 1
+    for (int k = 0; k < s.nel + ket.n; k++) {
+        int o = k;
+        if (k >= s.nel) {
+            o = (int)parts & 1023;
+            parts >>= FB;
+        } else if (left > 0 && ((int)holes & 1023) == k) {
+            holes >>= FB;
+            left--;
+            continue;
         }
+        if (o == i) continue;
+        const int Kk = o >> 1;
+        R t = eri_at<R>(s, A, I, Kk, Kk);
+        if (((a ^ o) & 1) == 0) t = t - eri_at<R>(s, A, Kk, Kk, I);
+        acc = acc + t;
     }
     return (double)((par & 1) ? -acc : acc);
 }
 
-// <bra|H|ket> for bra != ket by at most two spin-orbitals (else 0)
-template <int K, typename R>
-__device__ double h_between(const SysDev &s, const Det<K> &bra, const Det<K> &ket)
+// <HF|H|D> for D at level 1 or 2 (the gas has no level 1)
+template <typename R, bool GAS>
+__device__ __forceinline__ double h_ref(const SysDev &s, const Exc &d)
 {
-    int hol[2], par[2], nh = 0, np = 0;
-#pragma unroll
-    for (int w = 0; w < K; w++) {
-        u64 hm = ket.w[w] & ~bra.w[w];
-        u64 pm = bra.w[w] & ~ket.w[w];
-        while (hm) {
-            if (nh < 2) hol[nh] = 64 * w + (__ffsll((long long)hm) - 1);
-            nh++;
-            hm &= hm - 1;
-        }
-        while (pm) {
-            if (np < 2) par[np] = 64 * w + (__ffsll((long long)pm) - 1);
-            np++;
-            pm &= pm - 1;
-        }
-    }
-    if (nh != np || nh == 0 || nh > 2) return 0.0;
-    return h_offdiag<K, R>(s, ket, nh, hol[0], nh == 2 ? hol[1] : 0, par[0], nh == 2 ? par[1] : 0);
-}
-
-// <HF|H|D> for D at level 1 or 2
-template <int K, typename R>
-__device__ __forceinline__ double h_ref(const SysDev &s, const Det<K> &d)
-{
-    Det<K> hf;
-#pragma unroll
-    for (int w = 0; w < K; w++) hf.w[w] = s.hf[w];
-    return h_between<K, R>(s, hf, d);
+    return h_offdiag<R, GAS>(s, d, d.n, field(d.p, 0), field(d.p, 1), field(d.h, 0), field(d.h, 1));
 }
 
 // ---------------------------------------------------------------------------
 // Excitation generators
 // ---------------------------------------------------------------------------
 
-// pair index -> (x < y) with index = y(y-1)/2 + x
-__device__ __forceinline__ void pair_of(u64 idx, int &x, int &y)
+// pair index -> (x < y) with index = y(y-1)/2 + x, from a table: two square
+// roots' worth of arithmetic per draw otherwise
+__device__ __forceinline__ void pair_of(const SysDev &s, u64 idx, int &x, int &y)
 {
-    int yy = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)idx)) * 0.5f);
-    if (yy < 1) yy = 1;
-    while ((u64)yy * (yy - 1) / 2 > idx) yy--;
-    while ((u64)(yy + 1) * yy / 2 <= idx) yy++;
-    y = yy;
-    x = (int)(idx - (u64)yy * (yy - 1) / 2);
+    const unsigned v = __ldg(&s.pairs[idx]);
+    x = (int)(v & 0xFFFFu);
+    y = (int)(v >> 16);
 }
 
 // 1/p_gen of a generator case (0: gas double; 1, 2: molecule single of spin
@@ -601,78 +654,151 @@ __device__ __forceinline__ double inv_pgen_of(const SysDev &s, int gc)
     return gc == 0 ? s.inv_pgen_ueg : (gc < 3 ? s.inv_pgen_single[gc - 1] : s.inv_pgen_double[gc - 3]);
 }
 
-// One draw of the excitation generator from dj.  Returns false for a null
-// draw; otherwise di, the holes (i<j) and particles (a<b) relative to dj, the
-// number of holes nh and the generator case gc (see inv_pgen_of).
-template <int K>
-__device__ bool excite(const SysDev &s, const Det<K> &dj, const R4 &r, Det<K> &di, int &nh, int &i, int &j,
-                       int &a, int &b, int &gc)
+// k-th occupied spin-orbital (ascending): the core without the holes, then
+// the particles
+__device__ __forceinline__ int kth_occupied(const SysDev &s, const Exc &e, int k)
 {
-    if (s.kind == 0) {
-        int x, y;
-        pair_of(below(r.v[1], s.npairs), x, y);
-        i = kth_occupied(dj, x);
-        j = kth_occupied(dj, y);
-        int aa = kth_empty(s, dj, below(r.v[2], s.nvirt), -1);
-        if (aa < 0) return false;
-        int sb = (i & 1) + (j & 1) - (aa & 1);
-        if (sb < 0 || sb > 1) return false;
-        const int *ki = s.kv + 3 * (i >> 1), *kj = s.kv + 3 * (j >> 1), *ka = s.kv + 3 * (aa >> 1);
-        int nb0 = __ldg(ki) + __ldg(kj) - __ldg(ka);
-        int nb1 = __ldg(ki + 1) + __ldg(kj + 1) - __ldg(ka + 1);
-        int nb2 = __ldg(ki + 2) + __ldg(kj + 2) - __ldg(ka + 2);
-        int nm = s.nmax;
-        if (nb0 < -nm || nb0 > nm || nb1 < -nm || nb1 > nm || nb2 < -nm || nb2 > nm) return false;
-        int bs = __ldg(&s.grid[((nb0 + nm) * s.side + (nb1 + nm)) * s.side + (nb2 + nm)]);
-        if (bs < 0) return false;
-        int bb = 2 * bs + sb;
-        if (bb == aa || bit(dj, bb)) return false;
-        a = aa < bb ? aa : bb;
-        b = aa < bb ? bb : aa;
-        nh = 2;
-        gc = 0;
-    } else if (below(r.v[0], s.ns_nd) < s.ns) {
-        i = kth_occupied(dj, (int)below(r.v[1], (u64)s.nel));
-        int sg = i & 1;
-        if (s.nv[sg] == 0) return false;
-        a = kth_empty(s, dj, below(r.v[2], (u64)s.nv[sg]), sg);
-        if (a < 0) return false;
-        j = b = 0;
-        nh = 1;
-        gc = 1 + sg;
-    } else {
-        int x, y;
-        pair_of(below(r.v[1], s.npairs), x, y);
-        i = kth_occupied(dj, x);
-        j = kth_occupied(dj, y);
-        int aa, bb, c;
-        if (((i ^ j) & 1) == 0) {
-            int sg = i & 1;
-            c = sg;
-            if (s.ndcase[c] == 0) return false;
-            int xa, ya;
-            pair_of(below(r.v[2], s.ndcase[c]), xa, ya);
-            aa = kth_empty(s, dj, (u64)xa, sg);
-            bb = kth_empty(s, dj, (u64)ya, sg);
-        } else {
-            c = 2;
-            if (s.ndcase[c] == 0) return false;
-            u64 q = below(r.v[2], s.ndcase[c]);
-            aa = kth_empty(s, dj, q / (u64)s.nv[1], 0);
-            bb = kth_empty(s, dj, q % (u64)s.nv[1], 1);
-        }
-        if (aa < 0 || bb < 0) return false;
-        a = aa < bb ? aa : bb;
-        b = aa < bb ? bb : aa;
-        nh = 2;
-        gc = 3 + c;
+    const int core = s.nel - e.n;
+    if (k >= core) return field(e.p, k - core);
+    u64 t = e.h;
+#pragma unroll 1
+    for (int m = 0; m < e.n; m++, t >>= FB)
+        if (((int)t & 1023) <= k) k++;
+    return k;
+}
+
+// k-th empty spin-orbital (ascending): the holes, then the virtuals without
+// the particles
+__device__ __forceinline__ int kth_empty(const SysDev &s, const Exc &e, int k)
+{
+    if (k < e.n) return field(e.h, k);
+    int q = s.nel + k - e.n;
+    u64 t = e.p;
+#pragma unroll 1
+    for (int m = 0; m < e.n; m++, t >>= FB)
+        if (((int)t & 1023) <= q) q++;
+    return q;
+}
+
+// k-th empty spin-orbital of one spin (ascending), -1 if there are fewer
+__device__ __forceinline__ int kth_empty_spin(const SysDev &s, const Exc &e, int k, int spin)
+{
+    u64 t = e.h;
+    int c = 0, q = -1;
+#pragma unroll 1
+    for (int m = 0; m < e.n; m++, t >>= FB) {
+        const int x = (int)t & 1023;
+        if ((x & 1) != spin) continue;
+        if (c == k) q = x;
+        c++;
     }
-    di = dj;
-    flip(di, i);
-    if (nh == 2) flip(di, j);
-    flip(di, a);
-    if (nh == 2) flip(di, b);
+    if (k < c) return q;
+    q = s.nel + ((s.nel ^ spin) & 1) + 2 * (k - c);
+    t = e.p;
+#pragma unroll 1
+    for (int m = 0; m < e.n; m++, t >>= FB) {
+        const int x = (int)t & 1023;
+        if ((x & 1) == spin && x <= q) q += 2;
+    }
+    return q < s.nso ? q : -1;
+}
+
+// One draw of the excitation generator from dj.  Returns false for a null
+// draw or one that leaves the truncation; otherwise code = i | j << 10 |
+// a << 20 | b << 30 | gc << 40 with the holes i<j and particles a<b relative
+// to dj (j = b = 0 for a single) and the generator case gc (see inv_pgen_of).
+template <bool GAS>
+__device__ __forceinline__ bool excite(const SysDev &s, const Exc &dj, const R4 &r, u64 &code)
+{
+    int i, j = 0, a, b = 0, gc;
+    if (GAS) {
+        int x, y;
+        pair_of(s, below(r.v[1], s.npairs), x, y);
+        const int aa = kth_empty(s, dj, (int)below(r.v[2], s.nvirt));
+        i = kth_occupied(s, dj, x);
+        j = kth_occupied(s, dj, y);
+        const int sb = (i & 1) + (j & 1) - (aa & 1);
+        if (sb < 0 || sb > 1) return false;
+        const int bs = __ldg(&s.grid[s.mid + __ldg(&s.lin[i >> 1]) + __ldg(&s.lin[j >> 1]) - __ldg(&s.lin[aa >> 1])]);
+        const int bb = 2 * bs + sb;
+        if (bs < 0 || bb == aa) return false;
+        // occupied already?
+        if (bb < s.nel ? !has_field(dj.h, dj.n, bb) : has_field(dj.p, dj.n, bb)) return false;
+        a = min(aa, bb);
+        b = max(aa, bb);
+        gc = 0;
+    } else {
+        const bool dbl = !(below(r.v[0], s.ns_nd) < s.ns);
+        int x, y = 0;
+        if (dbl) pair_of(s, below(r.v[1], s.npairs), x, y);
+        else x = (int)below(r.v[1], (u64)s.nel);
+        i = kth_occupied(s, dj, x);
+        if (dbl) j = kth_occupied(s, dj, y);
+        // the empty orbitals: one of i's spin; or two of the pair's spin, or one of each
+        const int c = dbl && ((i ^ j) & 1) ? 2 : (i & 1);
+        const u64 many = dbl ? s.ndcase[c] : (u64)s.nv[c];
+        if (many == 0) return false;
+        const u64 q = below(r.v[2], many);
+        int ka = (int)q, kb = 0;
+        if (dbl && c < 2) pair_of(s, q, ka, kb);
+        if (c == 2) {
+            ka = (int)((unsigned)q / (unsigned)s.nv[1]);
+            kb = (int)((unsigned)q - (unsigned)ka * (unsigned)s.nv[1]);
+        }
+        a = kth_empty_spin(s, dj, ka, c == 2 ? 0 : c);
+        if (a < 0) return false;
+        if (dbl) {
+            const int bb = kth_empty_spin(s, dj, kb, c == 2 ? 1 : c);
+            if (bb < 0) return false;
+            b = max(a, bb);
+            a = min(a, bb);
+        }
+        gc = (dbl ? 3 : 1) + c;
+    }
+    // the level changes by the core orbitals emptied and filled
+    const int N = s.nel;
+    int lev = dj.n + (i < N ? 1 : 0) - (a < N ? 1 : 0);
+    if (GAS || gc >= 3) lev += (j < N ? 1 : 0) - (b < N ? 1 : 0);
+    if (lev > s.lmax) return false;
+    code = (u64)i | ((u64)j << 10) | ((u64)a << 20) | ((u64)b << 30) | ((u64)gc << 40);
     return true;
+}
+
+// dj with the drawn excitation applied (its level is within the truncation):
+// each of i, j, a, b enters the list it is not in and leaves the one it is in,
+// those that leave first, so that no list ever grows past six fields
+__device__ __forceinline__ Exc excited(const SysDev &s, const Exc &dj, u64 code, bool dbl)
+{
+    const u64 ij = code & 0xFFFFF, ab = (code >> 20) & 0xFFFFF;
+    u64 list = dj.h, h = 0;
+    u64 seq = ab | (ij << 20) | (ij << 40);   // holes: a, b filled, i, j emptied; particles: i, j, then a, b
+    int n = dj.n, nh = 0;
+#pragma unroll 1
+    for (int q = 0; q < 8; q++) {
+        if (q == 4) {
+            h = list;
+            nh = n;
+            list = dj.p;
+            n = dj.n;
+        }
+        if (q == 6) seq = ab;
+        const int v = (int)seq & 1023;
+        seq >>= FB;
+        if ((!dbl && (q & 1)) || (v < s.nel) != (q < 4)) continue;
+        const int c = fields_below(list, n, v);
+        if (c < n && field(list, c) == v) {
+            list = remove_at(list, c);
+            n--;
+        } else {
+            list = insert_at(list, c, v);
+            n++;
+        }
+    }
+    Exc e;
+    e.h = h;
+    e.p = list;
+    e.n = nh;
+    return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -705,21 +831,13 @@ __device__ __forceinline__ bool stoch_round(double x, double u, double cutoff, i
 // u * cutoff -- so comparing the exact values as scaled integers reproduces
 // it bit for bit without using the (narrow) FP64 pipe.
 
-// a * 2^sa < b * 2^sb for unsigned a, b
-__host__ __device__ __forceinline__ bool lt_scaled(u64 a, int sa, u64 b, int sb)
+// m < v 2^d for an integer m < 2^53 is m < this threshold (the ceiling of v 2^d;
+// v 2^d is below 2^53 where d > 0)
+__host__ __device__ __forceinline__ u64 scaled_threshold(u64 v, int d)
 {
-    int d = sa - sb;
-    if (d >= 0) {                       // a * 2^d < b
-        if (a == 0) return b != 0;
-        if (d >= 64) return false;
-        if (d > 0 && (a >> (64 - d)) != 0) return false;
-        return (a << d) < b;
-    }
-    int e = -d;                         // a < b * 2^e
-    if (b == 0) return false;
-    if (e >= 64) return true;
-    if ((b >> (64 - e)) != 0) return true;
-    return a < (b << e);
+    if (d >= 0) return v << (d & 63);
+    if (d <= -64) return v != 0 ? 1 : 0;
+    return (v >> -d) + ((v & ((1ULL << -d) - 1ULL)) != 0 ? 1 : 0);
 }
 
 // |x| = M * 2^E exactly (M < 2^53)
@@ -742,34 +860,49 @@ struct RoundSpec {
     i64 cutoff_fixed;  // cutoff in fixed point
 };
 
-__host__ __device__ __forceinline__ bool stoch_round_bits(u64 xbits, u64 r, const RoundSpec &rs, i64 &out)
+// |x| -> base, or base + inc when the uniform's integer mu = r >> 11 (u = mu 2^-53)
+// is below thr; false when |x| leaves the fixed-point range
+struct RoundCut {
+    u64 thr;
+    i64 base, inc;
+};
+
+__host__ __device__ __forceinline__ bool round_cut(u64 xbits, const RoundSpec &rs, RoundCut &c)
 {
-    const bool neg = (xbits >> 63) != 0;
     const u64 ab = xbits & 0x7FFFFFFFFFFFFFFFULL;
-    if (!(ab < 0x42D0000000000000ULL)) {   // |x| < 2^46 (also rejects inf and NaN)
-        out = 0;
-        return false;
-    }
-    const u64 mu = r >> 11;                // u = mu * 2^-53
+    c.thr = 0;
+    c.base = c.inc = 0;
+    if (!(ab < 0x42D0000000000000ULL)) return false;   // |x| < 2^46 (also rejects inf and NaN)
     u64 M;
     int E;
     split_double(ab, M, E);
-    i64 n;
-    if (ab < rs.cutoff_bits) {             // |x| < cutoff
-        n = lt_scaled(mu, rs.cutoff_e, M, E) ? rs.cutoff_fixed : 0;
-    } else {
-        int e = E + 16;                    // q = |x| 2^16 = M 2^e
+    u64 v = M;
+    int d = E - rs.cutoff_e;               // |x| < cutoff: u cutoff < |x|
+    c.inc = rs.cutoff_fixed;
+    if (ab >= rs.cutoff_bits) {
+        const int e = E + 16;              // q = |x| 2^16 = M 2^e; u < q - floor(q)
+        c.inc = 1;
+        d = 53 + e;
         if (e >= 0) {
-            n = (i64)(M << e);
-        } else {
-            int t = -e;
-            u64 f = t >= 64 ? 0 : (M >> t);
-            u64 fr = t >= 64 ? M : (M & ((1ULL << t) - 1ULL));
-            n = (i64)f + (lt_scaled(mu, -53, fr, -t) ? 1 : 0);
+            c.base = (i64)(M << e);
+            v = 0;
+            d = 0;
+        } else if (e > -64) {
+            c.base = (i64)(M >> -e);
+            v = M & ((1ULL << -e) - 1ULL);
         }
     }
-    out = neg ? -n : n;
+    c.thr = scaled_threshold(v, d);
     return true;
+}
+
+__host__ __device__ __forceinline__ bool stoch_round_bits(u64 xbits, u64 r, const RoundSpec &rs, i64 &out)
+{
+    RoundCut c;
+    const bool ok = round_cut(xbits, rs, c);
+    const i64 n = c.base + ((r >> 11) < c.thr ? c.inc : 0);
+    out = (xbits >> 63) ? -n : n;
+    return ok;
 }
 
 // ---------------------------------------------------------------------------

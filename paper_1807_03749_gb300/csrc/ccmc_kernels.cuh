@@ -1,10 +1,10 @@
 // ccmc_kernels.cuh -- device code of one CCMC time step (Spencer et al.,
 // arXiv:1807.03749, Sec. II and Sec. IV.B-C): the building blocks a1-a10,
-// the kernels templated on the determinant word count K and the precision R
-// of the matrix elements, and the template that issues a whole step.  Each
-// (K, R) pair is instantiated in its own translation unit
-// (ccmc_step_k<K>.cu) so that the word counts compile in parallel; the
-// kernels that do not depend on K are defined once, in ccmc_step.cu.
+// the kernels templated on the Hamiltonian kind and the precision R of the
+// matrix elements, and the template that issues a whole step.  Each (kind, R)
+// pair is instantiated in its own translation unit (ccmc_step_<kind>_<R>.cu)
+// so that they compile in parallel; the kernels that depend on neither are
+// defined once, in ccmc_step.cu.
 //
 //  a1  k_scan_partial / k_scan_top / k_scan_final : |t_i| prefix, N_total,
 //      t_HF, N_ex, n_sel, cluster amplitudes; full non-composite visits
@@ -208,32 +208,13 @@ __device__ __forceinline__ T block_reserve(T *counter, T count, T *sm, T *sbase)
     return base + incl - count;
 }
 
-template <int K>
-__device__ __forceinline__ Det<K> load_det(const u64 *bits, i64 cap, i64 i)
-{
-    Det<K> d;
-#pragma unroll
-    for (int w = 0; w < K; w++) d.w[w] = bits[w * cap + i];
-    return d;
-}
-
-template <int K>
-__device__ __forceinline__ void store_det(u64 *bits, i64 cap, i64 i, const Det<K> &d)
-{
-#pragma unroll
-    for (int w = 0; w < K; w++) bits[w * cap + i] = d.w[w];
-}
-
-template <int K>
-__device__ __forceinline__ Det<K> hf_det(const SysDev &s)
-{
-    Det<K> d;
-#pragma unroll
-    for (int w = 0; w < K; w++) d.w[w] = s.hf[w];
-    return d;
-}
-
 // n_attempts = max(1, floor(|A| / A_thresh)) with multi-spawn, else 1
+static __device__ __noinline__ i64 attempts_of_thresh(double amp_abs, double a_thresh)
+{
+    double q = floor(amp_abs / a_thresh);
+    return q < 1.0 ? 1 : (i64)q;
+}
+
 __device__ __forceinline__ i64 attempts_of(double amp_abs, const RunParams &p)
 {
     if (!p.multispawn) return 1;
@@ -245,54 +226,82 @@ __device__ __forceinline__ i64 attempts_of(double amp_abs, const RunParams &p)
         u64 q = E >= 0 ? (E >= 10 ? (1ULL << 62) : (M << E)) : (E <= -64 ? 0 : (M >> -E));
         return q < 1 ? 1 : (i64)q;
     }
-    double q = floor(amp_abs / p.a_thresh);
-    return q < 1.0 ? 1 : (i64)q;
+    return attempts_of_thresh(amp_abs, p.a_thresh);
+}
+
+// rounding with a cutoff that is no power of two (FP64 decisions)
+static __device__ __noinline__ bool round_value_fp(double x, u64 r, double cutoff, i64 *out)
+{
+    return stoch_round(x, unif(r), cutoff, *out);
 }
 
 // stochastic rounding of a spawned (with cutoff) or death (without) value
 __device__ __forceinline__ bool round_value(double x, u64 r, const RunParams &p, bool spawn, i64 &out)
 {
     if (p.int_round) return stoch_round_bits((u64)__double_as_longlong(x), r, spawn ? p.spawn_rs : p.death_rs, out);
-    return stoch_round(x, unif(r), spawn ? p.spawn_cutoff : 0.0, out);
+    return round_value_fp(x, r, spawn ? p.spawn_cutoff : 0.0, &out);
 }
 
-// the determinant of a picked entry: from its pick row (one granule with
-// the prefix and population just searched) when it has at most four words
-template <int K>
-__device__ __forceinline__ Det<K> pick_det(const PickEntry *pk, const ListView &L, i64 id)
+// smallest i in [1, n-1] with prefix[i] > x (excitor owning position x); the
+// bucket of x brackets the answer between the owners of its first position
+// and of the next bucket's first position
+__device__ __forceinline__ void pick_bracket(const int *bucket, int shift, i64 nbuckets, i64 n, u64 x, int &lo, int &hi)
 {
-    Det<K> d;
-    if constexpr (K <= 4) {
-#pragma unroll
-        for (int w = 0; w < K; w++) d.w[w] = __ldg(&pk[id].w[w]);
-    } else {
-        d = load_det<K>(L.bits, L.cap, id);
-    }
-    return d;
+    const i64 b = (i64)(x >> shift);
+    lo = __ldg(&bucket[b]);
+    hi = b + 1 < nbuckets ? __ldg(&bucket[b + 1]) : (int)(n - 1);
 }
 
-// smallest i in [1, n-1] with prefix[i] > x (excitor owning position x);
-// the bucket of x brackets the answer between the owners of its first
-// position and of the next bucket's first position
-__device__ __forceinline__ i64 pick_index(const PickEntry *pk, const int *bucket, int shift, i64 nbuckets, i64 n,
-                                          u64 x)
+__device__ __forceinline__ int pick_index(const PickEntry *pk, const int *bucket, int shift, i64 nbuckets, i64 n, u64 x)
 {
-    i64 b = (i64)(x >> shift);
-    i64 lo = __ldg(&bucket[b]);
-    i64 hi = b + 1 < nbuckets ? __ldg(&bucket[b + 1]) : n - 1;
+    int lo, hi;
+    pick_bracket(bucket, shift, nbuckets, n, x, lo, hi);
     while (lo < hi) {
-        i64 mid = lo + (hi - lo) / 2;
+        const int mid = lo + (hi - lo) / 2;
         if ((u64)__ldg(&pk[mid].prefix) > x) hi = mid;
         else lo = mid + 1;
     }
     return lo;
 }
 
+// two picks of one sample, their searches in step so that both loads of a
+// round are in flight together
+__device__ __forceinline__ void pick_two(const PickEntry *pk, const int *bucket, int shift, i64 nbuckets, i64 n, u64 x0,
+                                         u64 x1, bool two, int &i0, int &i1)
+{
+    int lo0, hi0, lo1 = 1, hi1 = 1;
+    pick_bracket(bucket, shift, nbuckets, n, x0, lo0, hi0);
+    if (two) pick_bracket(bucket, shift, nbuckets, n, x1, lo1, hi1);
+    while (lo0 < hi0 || lo1 < hi1) {
+        const int m0 = lo0 + (hi0 - lo0) / 2, m1 = lo1 + (hi1 - lo1) / 2;
+        const u64 p0 = lo0 < hi0 ? (u64)__ldg(&pk[m0].prefix) : 0;
+        const u64 p1 = lo1 < hi1 ? (u64)__ldg(&pk[m1].prefix) : 0;
+        if (lo0 < hi0) {
+            if (p0 > x0) hi0 = m0;
+            else lo0 = m0 + 1;
+        }
+        if (lo1 < hi1) {
+            if (p1 > x1) hi1 = m1;
+            else lo1 = m1 + 1;
+        }
+    }
+    i0 = lo0;
+    i1 = lo1;
+}
+
+// the excitor of a pick row
+__device__ __forceinline__ Exc row_exc(const PickEntry *pk, i64 id, u64 &flags)
+{
+    const u64 h = __ldg(&pk[id].h), p = __ldg(&pk[id].p);
+    flags = p;
+    return exc_of(h, p);
+}
+
 // Simulated distribution (Sec. III): the excitor of processor q holding
 // position x in [0, N_q) of that processor's entries in list order -- the
 // chunk whose processor-q prefix brackets x, then a walk over the chunk;
 // -1 only if the tables were inconsistent
-__device__ __forceinline__ i64 local_pick(const WorkArrays &wa, const PickEntry *pk, i64 n, int lcs, i64 nlc, u64 q,
+__device__ __forceinline__ i64 local_pick(const WorkArrays &wa, const i64 *pop, i64 n, int lcs, i64 nlc, u64 q,
                                           u64 x)
 {
     const i64 *row = wa.lcp + (i64)q * nlc;
@@ -306,7 +315,7 @@ __device__ __forceinline__ i64 local_pick(const WorkArrays &wa, const PickEntry 
     const i64 b = lo << lcs, e = b + (1LL << lcs) < n ? b + (1LL << lcs) : n;
     for (i64 i = b > 1 ? b : 1; i < e; i++) {
         if (__ldg(&wa.owner[i]) != q) continue;
-        const i64 v = __ldg(&pk[i].pop);
+        const i64 v = __ldg(&pop[i]);
         acc += (u64)(v < 0 ? -v : v);
         if (acc > x) return i;
     }
@@ -383,41 +392,24 @@ __device__ __forceinline__ i64 lower_bound_key(const u64 *keys, i64 n, u64 k)
 }
 
 // One spawning attempt from dj carrying coefficient c_att (Sec. II):
-// value -dtau H_ij c_att s_D(i) / p_gen, stochastically rounded.
-// A spawning attempt in two halves.  attempt_draw runs the excitation
-// generator and the truncation check (about nine draws in ten end here for
-// the gas); attempt_finish computes the matrix element, the value, its
-// stochastic rounding and the rank key.  The expanded-attempt kernel queues
-// the surviving draws and finishes them 32 at a time, so the second half
-// runs on full warps.
-// the drawn excitation (holes i, j and particles a, b: 16 bits each, M <= 384)
-template <int K>
-__device__ __forceinline__ bool attempt_draw(const SysDev &s, const Det<K> &dj, const R4 &r, u64 &code, int &gc)
+// value -dtau H_ij c_att s_D(i) / p_gen, stochastically rounded, in two
+// halves.  excite() runs the excitation generator and the truncation check
+// (about nine draws in ten end there for the gas); attempt_finish computes the
+// matrix element, the value, its stochastic rounding and the rank key.  The
+// surviving draws are queued per warp and finished 32 at a time, so the second
+// half runs on full warps.
+template <typename R, bool GAS>
+__device__ __forceinline__ bool attempt_finish(const SysDev &s, const RunParams &p, const Exc &dj, double c_att,
+                                               u64 r3, u64 code, u64 &key, i64 &val, unsigned &err)
 {
-    Det<K> di;
-    int nh, i, j, a, b;
-    if (!excite(s, dj, r, di, nh, i, j, a, b, gc)) return false;
-    if (level_of(s, di) > s.lmax) return false;
-    code = (u64)i | ((u64)j << 16) | ((u64)a << 32) | ((u64)b << 48);
-    return true;
-}
-
-template <int K, typename R>
-__device__ __forceinline__ bool attempt_finish(const SysDev &s, const RunParams &p, const Det<K> &dj, double c_att,
-                                               u64 r3, u64 code, int gc, u64 &key, i64 &val, unsigned &err)
-{
-    const int i = (int)(code & 0xFFFF), j = (int)((code >> 16) & 0xFFFF), a = (int)((code >> 32) & 0xFFFF),
-              b = (int)(code >> 48);
-    const int nh = (gc == 1 || gc == 2) ? 1 : 2;
-    Det<K> di = dj;
-    flip(di, i);
-    if (nh == 2) flip(di, j);
-    flip(di, a);
-    if (nh == 2) flip(di, b);
+    const int i = (int)code & 1023, j = (int)(code >> 10) & 1023, a = (int)(code >> 20) & 1023,
+              b = (int)(code >> 30) & 1023, gc = (int)(code >> 40) & 7;
+    const bool dbl = GAS || gc == 0 || gc >= 3;
+    const Exc di = excited(s, dj, code, dbl);
     // matrix element and 1/p_gen in the precision R; the value itself in FP64
-    double h = h_offdiag<K, R>(s, dj, nh, i, j, a, b);
+    double h = h_offdiag<R, GAS>(s, dj, dbl ? 2 : 1, i, j, a, b);
     double x = ((p.tau * h) * inv_pgen_of<R>(s, gc)) * c_att;
-    if (excitor_sign(s, di) > 0) x = -x;
+    if (!sign_parity(s, di)) x = -x;
     i64 v;
     if (!round_value(x, r3, p, true, v)) {
         err |= ERRB_NUMERIC;
@@ -430,30 +422,25 @@ __device__ __forceinline__ bool attempt_finish(const SysDev &s, const RunParams 
 }
 
 // Per-warp queue of drawn attempts waiting for attempt_finish.
-template <int K>
 struct AttQueue {
-    u64 det[K][64];
+    u64 h[64], p[64];
     double c[64];
     u64 r[64];
     u64 code[64];
-    unsigned char gc[64];
 };
 
 // All 32 lanes call; lanes with ok append their attempt (qn < 32 on entry).
-template <int K>
-__device__ __forceinline__ void q_push(AttQueue<K> &q, int &qn, bool ok, const Det<K> &dj, double c, u64 r3, u64 code,
-                                       int gc)
+__device__ __forceinline__ void q_push(AttQueue &q, int &qn, bool ok, const Exc &dj, double c, u64 r3, u64 code)
 {
     const int lane = threadIdx.x & 31;
     const unsigned m = __ballot_sync(FULLMASK, ok);
     if (ok) {
         const int e = qn + __popc(m & ((1u << lane) - 1u));
-#pragma unroll
-        for (int w = 0; w < K; w++) q.det[w][e] = dj.w[w];
+        q.h[e] = pack_h(dj);
+        q.p[e] = dj.p;
         q.c[e] = c;
         q.r[e] = r3;
         q.code[e] = code;
-        q.gc[e] = (unsigned char)gc;
     }
     qn += __popc(m);
     __syncwarp();
@@ -523,78 +510,67 @@ __device__ __forceinline__ i64 find_key(const DirectView &d, u64 k)
     return (lo < d.n && __ldg(&d.key[lo]) == k) ? lo : -1;
 }
 
-// All 32 lanes call: takes the newest 32 staged records while 32 or more are
-// waiting (with all, every staged record); records onto listed determinants
-// are added to them directly, the others appended to the spawn buffer with
-// one atomic per warp.
-__device__ __forceinline__ void rec_flush(RecStage &rs, int &rn, bool all, DevStep *st, const SpawnBuf &sp,
-                                          const DirectView &dv, i64 &ndirect, unsigned &err)
+// All 32 lanes call: takes the newest (at most 32) staged records; records
+// onto listed determinants are added to them directly, the others appended to
+// the spawn buffer with one atomic per warp.
+__device__ __forceinline__ void rec_flush_once(RecStage &rs, int &rn, DevStep *st, const SpawnBuf &sp,
+                                               const DirectView &dv, i64 &ndirect, unsigned &err)
 {
     const int lane = threadIdx.x & 31;
-    while (rn >= 32 || (all && rn > 0)) {
-        const int take = rn >= 32 ? 32 : rn;
-        const bool have = lane < take;
-        u64 k = 0;
-        i64 v = 0;
-        if (have) {
-            const int e = rn - take + lane;
-            k = rs.key[e];
-            v = rs.val[e];
+    const int take = rn >= 32 ? 32 : rn;
+    bool app = lane < take;
+    u64 k = 0;
+    i64 v = 0;
+    if (app) {
+        const int e = rn - take + lane;
+        k = rs.key[e];
+        v = rs.val[e];
+    }
+    __syncwarp();   // the stage is read before later pushes reuse it
+    rn -= take;
+    if (app && dv.nkb > 0) {
+        const i64 pos = find_key(dv, k);
+        if (pos >= 0) {
+            atomicAdd((unsigned long long *)&dv.acc[pos], (unsigned long long)v);
+            dv.hit[pos] = 1;
+            ndirect++;
+            app = false;
         }
-        __syncwarp();   // the stage is read before later pushes reuse it
-        rn -= take;
-        bool app = have;
-        if (have && dv.nkb > 0) {
-            const i64 pos = find_key(dv, k);
-            if (pos >= 0) {
-                atomicAdd((unsigned long long *)&dv.acc[pos], (unsigned long long)v);
-                dv.hit[pos] = 1;
-                ndirect++;
-                app = false;
-            }
-        }
-        const unsigned m = __ballot_sync(FULLMASK, app);
-        if (m == 0) continue;
-        i64 base = 0;
-        if (lane == 0) base = (i64)atomicAdd((unsigned long long *)&st->n_sp, (unsigned long long)__popc(m));
-        base = __shfl_sync(FULLMASK, base, 0);
-        if (app) {
-            const i64 off = base + __popc(m & ((1u << lane) - 1u));
-            if (off < sp.cap) {
-                sp.key[0][off] = k;
-                sp.pop[0][off] = v;
-            } else {
-                err |= ERRB_SPAWN_OVERFLOW;
-            }
+    }
+    const unsigned m = __ballot_sync(FULLMASK, app);
+    if (m == 0) return;
+    i64 base = 0;
+    if (lane == 0) base = (i64)atomicAdd((unsigned long long *)&st->n_sp, (unsigned long long)__popc(m));
+    base = __shfl_sync(FULLMASK, base, 0);
+    if (app) {
+        const i64 off = base + __popc(m & ((1u << lane) - 1u));
+        if (off < sp.cap) {
+            sp.key[0][off] = k;
+            sp.pop[0][off] = v;
+        } else {
+            err |= ERRB_SPAWN_OVERFLOW;
         }
     }
 }
 
-// All 32 lanes call: finishes the newest 32 queued attempts while 32 or more
-// are waiting (with all, every waiting attempt) into the record stage.
-template <int K, typename R>
-__device__ __forceinline__ void q_drain_staged(AttQueue<K> &q, int &qn, bool all, RecStage &rs, int &rn,
-                                               const SysDev &s, const RunParams &p, DevStep *st, const SpawnBuf &sp,
-                                               const DirectView &dv, i64 &ndirect, unsigned &err)
+// All 32 lanes call: finishes the newest (at most 32) queued attempts into
+// the record stage (rn < 32 on entry).
+template <typename R, bool GAS>
+__device__ __forceinline__ void q_finish(AttQueue &q, int &qn, RecStage &rs, int &rn, const SysDev &s,
+                                         const RunParams &p, unsigned &err)
 {
     const int lane = threadIdx.x & 31;
-    while (qn >= 32 || (all && qn > 0)) {
-        const int take = qn >= 32 ? 32 : qn;
-        bool has = false;
-        u64 k = 0;
-        i64 v = 0;
-        if (lane < take) {
-            const int e = qn - take + lane;
-            Det<K> dj;
-#pragma unroll
-            for (int w = 0; w < K; w++) dj.w[w] = q.det[w][e];
-            has = attempt_finish<K, R>(s, p, dj, q.c[e], q.r[e], q.code[e], q.gc[e], k, v, err);
-        }
-        __syncwarp();   // the entries are read before later pushes reuse them
-        qn -= take;
-        rec_push(rs, rn, has, k, v);
-        rec_flush(rs, rn, false, st, sp, dv, ndirect, err);
+    const int take = qn >= 32 ? 32 : qn;
+    bool has = false;
+    u64 k = 0;
+    i64 v = 0;
+    if (lane < take) {
+        const int e = qn - take + lane;
+        has = attempt_finish<R, GAS>(s, p, exc_of(q.h[e], q.p[e]), q.c[e], q.r[e], q.code[e], k, v, err);
     }
+    __syncwarp();   // the entries are read before later pushes reuse them
+    qn -= take;
+    rec_push(rs, rn, has, k, v);
 }
 
 // occupation threshold: 0 < |v| < 1 becomes +-1 with probability |v|, else 0
@@ -691,9 +667,14 @@ __device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const
         st->ntot = ntot;
         st->nex = tw;
         // selection buckets: the smallest power of two 2^k with N_ex <= 2^(k + bucket_bits)
-        // about two buckets per list entry (bounded by the bucket array)
+        // about two buckets per list entry
+        // (bounded by the bucket array), and for a short list sampled often up to one
+        // per 32 samples: its populations span decades, so that equal ranges
+        // of positions hold from none to hundreds of its entries
+        i64 nb_want = n_sel >> 5 < (1LL << 18) ? n_sel >> 5 : (1LL << 18);
+        if (nb_want < 2 * st->n_occ) nb_want = 2 * st->n_occ;
         int bb = 4;
-        while (bb < wa.bucket_bits && (1LL << bb) < 2 * st->n_occ) bb++;
+        while (bb < wa.bucket_bits && (1LL << bb) < nb_want) bb++;
         int k = 0;
         while (k < 62 && ((u64)tw >> (k + bb)) != 0) k++;
         st->bucket_shift = k;
@@ -701,7 +682,8 @@ __device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const
         st->n_sel = n_sel;
         st->fnc_attempts = p.fnc ? ta : 0;
         // key buckets for direct accumulation: about two per list entry over
-        // the list's key range, within the table's capacity
+        // the list's key range (up to eight for a short list: the keys
+        // cluster), within the table's capacity
         st->n_direct = 0;
         st->n_hit = 0;
         // direct accumulation pays once the step spawns more than about one
@@ -710,7 +692,8 @@ __device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const
         // step and does not change any result
         if (p.direct && st->n_occ > 0 && 10 * st->prev_spawned > st->n_occ) {
             const u64 kmax = L.key[st->n_occ - 1];
-            i64 want = 2 * st->n_occ;
+            i64 want = 8 * st->n_occ < (1LL << 18) ? 8 * st->n_occ : (1LL << 18);
+            if (want < 2 * st->n_occ) want = 2 * st->n_occ;
             if (want > (1LL << wa.kbucket_bits)) want = 1LL << wa.kbucket_bits;
             int ks = 0;
             while (ks < 63 && (i64)(kmax >> ks) + 1 > want) ks++;
@@ -777,9 +760,29 @@ __device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const
     }
 }
 
+// All 32 lanes call: each lane's run [b0, b1) of t (empty if b1 <= b0) is set
+// to v.  Runs of up to 8 are written by their lane; longer ones (an excitor
+// holding many particles, a gap in the keys) by the whole warp, one after
+// another.
+__device__ __forceinline__ void fill_run(int *t, i64 b0, i64 b1, int v)
+{
+    const int lane = threadIdx.x & 31;
+    const bool lng = b1 - b0 > 8;
+    if (!lng)
+        for (i64 b = b0; b < b1; b++) t[b] = v;
+    unsigned m = __ballot_sync(FULLMASK, lng);
+    while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        const i64 s0 = __shfl_sync(FULLMASK, b0, src), s1 = __shfl_sync(FULLMASK, b1, src);
+        const int sv = __shfl_sync(FULLMASK, v, src);
+        for (i64 b = s0 + lane; b < s1; b += 32) t[b] = sv;
+    }
+}
+
 // prefix arrays; with full non-composite sampling also every visit's death,
 // estimator contribution and attempt coefficient (Sec. IV.B)
-template <int K, typename R>
+template <typename R, bool GAS>
 __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa)
 {
     __shared__ u64 smf[64];
@@ -791,6 +794,7 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
     Fix128 es = {0, 0};
     unsigned err = 0;
     const bool kb = st->nkb > 0;
+    const int bsh = st->bucket_shift, ksh = st->kshift;
     // each warp scans its own chunk 32 entries at a time (no block barrier)
     for (i64 base = lo; base < hi; base += 32) {
         i64 i = base + (threadIdx.x & 31);
@@ -800,8 +804,7 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
         i64 v = ok ? L.pop[i] : 0, av = v < 0 ? -v : v;
         const u64 key_i = ok && kb ? L.key[i] : 0, key_p = ok && kb && i > 0 ? L.key[i - 1] : 0;
         const double diag_i = ok && i > 0 ? L.diag[i] : 0.0;
-        Det<K> d;
-        if (ok) d = load_det<K>(L.bits, L.cap, i);
+        const Exc d = ok ? exc_of(L.h[i], L.p[i]) : Exc{0, 0, 0};
         i64 w = (ok && i > 0) ? av : 0;
         double amp = (double)v / FIX_ONE;
         i64 na = (ok && p.fnc) ? attempts_of(fabs(amp), p) : 0;
@@ -812,49 +815,40 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
             ia = warp_incl_scan(na);
             ta = __shfl_sync(FULLMASK, ia, 31);
         }
+        {
+            // buckets whose first position falls in [prefix[i-1], prefix[i]) start at entry i
+            const u64 p0 = (u64)(cw + iw - w), p1 = (u64)(cw + iw), half = (1ULL << bsh) - 1;
+            fill_run(wa.bucket, (i64)((p0 + half) >> bsh), w > 0 ? (i64)((p1 + half) >> bsh) : 0, (int)i);
+            // buckets whose first key falls in (key[i-1], key[i]] start at entry i
+            if (kb) fill_run(wa.kbucket, i == 0 ? 0 : (i64)(key_p >> ksh) + 1, ok ? (i64)(key_i >> ksh) + 1 : 0, (int)i);
+        }
         if (ok) {
             PickEntry pe;
             pe.prefix = cw + iw;
-            pe.pop = v;
-            pe.href = 0.0;
-            if (i > 0 && w > 0) {
-                // buckets whose first position falls in [prefix[i-1], prefix[i]) start at entry i
-                const int k = st->bucket_shift;
-                u64 p0 = (u64)(cw + iw - w), p1 = (u64)(cw + iw);
-                u64 b0 = (p0 + (1ULL << k) - 1) >> k, b1 = (p1 + (1ULL << k) - 1) >> k;
-                for (u64 b = b0; b < b1; b++) wa.bucket[b] = (int)i;
-            }
             wa.acc[i] = 0;
             wa.before[i] = 0;
             if (kb) {
-                // buckets whose first key falls in (key[i-1], key[i]] start at entry i
-                const int ks = st->kshift;
-                const u64 b0 = i == 0 ? 0 : (key_p >> ks) + 1, b1 = key_i >> ks;
-                for (u64 b = b0; b <= b1; b++) wa.kbucket[b] = (int)i;
                 wa.hit[i] = 0;
             }
             const double td = p.tau * ((i == 0 ? 0.0 : diag_i) - S);
+            const int odd = sign_parity(s, d);
             pe.tdeath = td;
+            pe.h = pack_h(d);
+            pe.p = d.p | (odd ? PICK_ODD : 0) | (v < 0 ? PICK_NEG : 0);
             i64 dv = 0;
             if (p.fnc) {
                 wa.att_end[i] = ca + ia;
-                int sd = excitor_sign(s, d);
-                double coef = sd > 0 ? amp : -amp;
-                int lev = level_of(s, d);
-                if (lev == 1 || lev == 2) es.add(to_fix(h_ref<K, R>(s, d) * coef));
+                double coef = odd ? -amp : amp;
+                if (d.n == 1 || d.n == 2) es.add(to_fix(h_ref<R, GAS>(s, d) * coef));
                 R4 r = draw(p.seed, p.replica, it, TAG_VISIT, (u64)i, 0);
                 double x = td * coef;
-                if (sd > 0) x = -x;
+                if (!odd) x = -x;
                 if (!round_value(x, r.v[0], p, false, dv)) err |= ERRB_NUMERIC;
                 wa.catt[i] = na > 1 ? coef / (double)na : coef;
             } else {
                 // <HF|H|D_i> for the single-excitor clusters of the sampler
-                const int lev = level_of(s, d);
-                pe.href = (lev == 1 || lev == 2) ? h_ref<K, R>(s, d) : 0.0;
+                wa.href[i] = (d.n == 1 || d.n == 2) ? h_ref<R, GAS>(s, d) : 0.0;
             }
-            // the words ride in the row a pick reads anyway (up to four)
-#pragma unroll
-            for (int q = 0; q < 4; q++) pe.w[q] = q < K ? d.w[q < K ? q : 0] : 0;
             wa.picks[i] = pe;
             wa.death[i] = dv;
         }
@@ -874,7 +868,7 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
 // each processor holds in it; one warp per chunk, which clears its column of
 // the table first (integer sums: the table does not depend on the order)
 template <int K>
-__device__ __forceinline__ void d_local_table(const ListView &L, const DevStep *st, const RunParams &p, const WorkArrays &wa)
+__device__ __forceinline__ void d_local_table(const SysDev &s, const ListView &L, const DevStep *st, const RunParams &p, const WorkArrays &wa)
 {
     if (p.nranks <= 1) return;
     const i64 n = st->n_occ, nlc = st->nlc;
@@ -887,7 +881,7 @@ __device__ __forceinline__ void d_local_table(const ListView &L, const DevStep *
         const i64 b = c << lcs, e = b + (1LL << lcs) < n ? b + (1LL << lcs) : n;
         for (i64 i = b + lane; i < e; i += 32) {
             if (i == 0) continue;   // the reference is not an excitor
-            const Det<K> d = load_det<K>(L.bits, L.cap, i);
+            const Det<K> d = words_from_exc<K>(s, exc_of(L.h[i], L.p[i]));
             const u64 q = words_owner(d.w, K, it, p.nu_move, (u64)p.nranks);
             wa.owner[i] = (unsigned short)q;
             const i64 v = L.pop[i];
@@ -923,239 +917,323 @@ __device__ __forceinline__ void d_local_scan(const DevStep *st, const RunParams 
 // a2-a5: cluster sampling (Sec. II; composites only with FNC, Sec. IV.B)
 // ---------------------------------------------------------------------------
 
+// Per-warp shared memory of the sampler: samples waiting for their picks,
+// samples of the bare reference, drawn attempts and spawned records.
+struct SampWarp {
+    u64 g[64], v1[64], v2[64], v3[64];   // sample index and the selection draw's words 1-3
+    u64 hg[64];                          // sample indices of reference clusters
+    unsigned char sz[64];                // cluster sizes of the waiting samples
+    AttQueue q;
+    RecStage rs;
+};
+
+// Each warp runs its samples in two stages on full warps.  Stage 1 draws 32
+// samples' selection words and sorts them by cost into two queues: the bare
+// reference (half of the original sampler's samples: no picks, a constant
+// amplitude and death value) and the clusters that need picks; sizes that
+// cannot stay within l + 2 end there.  Whenever a queue holds 32, stage 2 takes
+// them: picks, collapse, death and estimator for the clusters, then one
+// spawning attempt each (or the append to the multi-spawn buffer).  Both
+// kinds share the attempt's code, so that it is fetched once.
+//
+// What bounds it: instruction issue (55 % of the slots, 24 of 32 lanes; the
+// two Philox draws of a sample are a third of it).  With every size handled
+// where it was drawn and bit-string determinants, 15.7 (gas) and 8.7
+// (molecule) lanes of 32 were active, 320 bytes of local memory per thread.
+// 1.5e8 samples of the 162-orbital FP32 gas: 18.7 -> 7.6 ms; 2e7 of the
+// molecule: 5.5 ms (with the attempts of its clusters, which then went through
+// a buffer) -> 3.6 ms; 64 gas replicas: 3.2 -> 1.65 ms.
 // DIST: the simulated distribution's restricted composite draw is compiled
 // in (a separate instantiation keeps it out of the plain sampler's loop)
-template <int K, typename R, bool DIST>
+template <typename R, bool GAS, bool DIST>
 __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa,
                                                          const SpawnBuf &sp, const ClusterBuf &cl, int enum_base,
-                                                         int vb, int vg)
+                                                         int vb, int vg, SampWarp &sw)
 {
     __shared__ double smag[8], scmag[8], smden[8];
     __shared__ i64 snatt[8];
     __shared__ u64 smf[64];
     __shared__ i64 sm[32];
-    // per-warp queues: drawn spawning attempts waiting for attempt_finish,
-    // and spawned records waiting to be written 32 at a time
-    __shared__ AttQueue<K> aq[WORK_THREADS / 32];
-    __shared__ RecStage rsb[WORK_THREADS / 32];
+    __shared__ PhiloxStep ps;
     if (threadIdx.x < 8) {
         smag[threadIdx.x] = st->mag[threadIdx.x];
         scmag[threadIdx.x] = st->cmag[threadIdx.x];
         snatt[threadIdx.x] = st->natt_s[threadIdx.x];
         smden[threadIdx.x] = st->mden[threadIdx.x];
     }
+    philox_step_init(ps, st->iter, p.seed, p.replica);
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    AttQueue<K> &q = aq[wid];
-    RecStage &rb = rsb[wid];
-    int qn = 0, rn = 0;   // warp-uniform queue fills
+    const unsigned below_me = (1u << lane) - 1u;
+    AttQueue &q = sw.q;
+    RecStage &rb = sw.rs;
+    int wn = 0, hn = 0, qn = 0, rn = 0;   // warp-uniform queue fills
     const i64 n_sel = st->n_sel, n = st->n_occ, nex = st->nex, n0 = st->n0;
     const int bshift = st->bucket_shift;
     const i64 nbk = st->nbuckets;
-    const int lcs = st->lcs;
-    const i64 nlc = st->nlc;
-    const u64 it = st->iter;
-    const double S = st->shift;
     Fix128 es = {0, 0};
     unsigned err = 0;
-    i64 inline_att = 0;
-    u64 cl_att = 0;        // attempts of the clusters this thread buffers
+    unsigned n_valid = 0;  // valid clusters of this thread
+    double cl_att = 0.0;   // attempts of the clusters this thread buffers (exact below 2^53)
     i64 death_hf = 0;      // reference-cluster deaths, summed per block at the end
     i64 ndirect = 0;       // records added directly to listed determinants
     const DirectView dv = direct_view(L, wa, st);
     const PickEntry *pk = wa.picks;
-    // each warp runs its 32 samples of every block tile on its own: the
-    // appends are staged per warp, so no block barrier is needed in the loop
-    for (i64 g0 = (i64)vb * blockDim.x + 32 * wid; g0 < n_sel; g0 += (i64)vg * blockDim.x) {
-        const i64 g = g0 + lane;
-        bool rec = false;       // a composite death record
-        u64 rk = 0;
-        i64 rv = 0;
-        bool valid_cl = false;  // a cluster that makes spawning attempts
-        Det<K> dj;
-        double coef = 0.0, catt = 0.0;
-        i64 natt = 0;
-        if (g < n_sel) {
-            R4 r0 = draw(p.seed, p.replica, it, TAG_SAMPLE, (u64)g, 0);
-            u64 nr = ~r0.v[0];
-            int lz = nr ? __clzll((long long)nr) : 64;
-            int sz = p.fnc ? 2 + min(lz, s.lmax) : min(lz, s.lmax + 2);
-            bool valid = true;
-            int par = 0;
-            i64 idx0 = 0;
-            double amp = 0.0;
-            dj = hf_det<K>(s);
-            if (sz == 0) {
-                amp = n0 < 0 ? -smag[0] : smag[0];
-            } else if (nex == 0 || (sz >= 2 && n0 == 0) || sz * s.lmin_exc > s.lmax + 2) {
-                // the last test: a valid cluster's level is the sum of its
-                // excitors' levels, so this size cannot stay within l + 2
-                // and the sample contributes nothing (its picks are skipped)
-                valid = false;
-            } else {
-                R4 r1;
-                if (sz > 2) r1 = draw(p.seed, p.replica, it, TAG_SAMPLE, (u64)g, 1);
-                i64 idx[6];
-                int neg = 0;
-                // simulated distribution: a composite's later excitors come
-                // from the first one's processor q (Sec. III)
-                const bool local = DIST && p.nranks > 1 && sz >= 2;
-                i64 nq = 0;
-                if (!local) {
-                    // the picks are independent: issue all searches before using them
-                    for (int e = 0; e < sz; e++) {
-                        u64 rr = e < 2 ? r0.v[2 + e] : r1.v[e - 2];
-                        idx[e] = pick_index(pk, wa.bucket, bshift, nbk, n, below(rr, (u64)nex));
-                    }
-                } else {
-                    idx[0] = pick_index(pk, wa.bucket, bshift, nbk, n, below(r0.v[2], (u64)nex));
-                    const u64 q = __ldg(&wa.owner[idx[0]]);
-                    nq = __ldg(&wa.nq[q]);
-                    for (int e = 1; e < sz; e++) {
-                        u64 rr = e < 2 ? r0.v[2 + e] : r1.v[e - 2];
-                        idx[e] = local_pick(wa, pk, n, lcs, nlc, q, below(rr, (u64)nq));
-                        if (idx[e] < 0) {   // tables inconsistent (cannot happen): a sticky error, not a guess
-                            valid = false;
-                            err |= ERRB_NUMERIC;
+    const double coef_hf = n0 < 0 ? -smag[0] : smag[0];
+    // every reference cluster's death value is the same: its rounding once per block
+    const double death_x = -(pk[0].tdeath * coef_hf);   // the reference's sign s_D is +1
+    RoundCut hf_cut = {0, 0, 0};
+    const bool hf_ok = !p.int_round || round_cut((u64)__double_as_longlong(death_x), p.death_rs, hf_cut);
+    i64 g0 = (i64)vb * blockDim.x + 32 * wid;
+    const i64 stride = (i64)vg * blockDim.x;
+    for (;;) {
+        // one action per pass, so that each piece of code is fetched from one
+        // place (the loop is bound by instruction fetch when it grows):
+        // finish what is waiting 32 at a time, else take 32 queued samples,
+        // else draw 32 new ones; at the end whatever is left
+        const bool more = g0 < n_sel;
+        const bool last = !more && wn + hn == 0;
+        if (rn >= 32 || (last && qn == 0 && rn > 0)) {
+            rec_flush_once(rb, rn, st, sp, dv, ndirect, err);
+            continue;
+        }
+        if (qn >= 32 || (last && qn > 0)) {
+            q_finish<R, GAS>(q, qn, rb, rn, s, p, err);
+            continue;
+        }
+        if (last) break;
+        int tw = 0, th = 0;   // samples taken from either queue
+        if (wn >= 32) {
+            tw = 32;
+        } else if (hn >= 32) {
+            th = 32;
+        } else if (!more) {
+            tw = wn;
+            th = min(hn, 32 - tw);
+        }
+        const bool sel = tw + th == 0;   // draw new samples
+        u64 g = (u64)g0 + lane;
+        bool valid = true;
+        Exc dj = {0, 0, 0};
+        double coef = coef_hf;
+        if (!sel) {
+            const bool is_w = lane < tw;
+            valid = is_w || lane < tw + th;
+            int sz = 0;
+            i64 natt = 1;
+            bool local = false;
+            if (valid) g = is_w ? sw.g[wn - tw + lane] : sw.hg[hn - th + lane - tw];
+            if (tw > 0) {
+                // stage 2: picks, collapse, estimator and death of the clusters
+                bool rec = false;   // a composite death record
+                u64 rk = 0;
+                i64 rv = 0;
+                if (is_w) {
+                    const int we = wn - tw + lane;
+                    const u64 v1 = sw.v1[we], v2 = sw.v2[we], v3 = sw.v3[we];
+                    sz = sw.sz[we];
+                    local = DIST && p.nranks > 1 && sz >= 2;
+                    i64 nq = 0;
+                    u64 lq = 0, xa = v2, xb = v3, xc = 0, xd = 0;
+                    int i0 = 0, neg = 0, par = 0;
+                    // two picks a round: the selection draw's words 2-3, then its second block
+#pragma unroll 1
+                    for (int e = 0; e < sz && valid; e += 2) {
+                        if (e == 2) {
+                            const R4 r1 = step_draw_at(ps, TAG_SAMPLE, g, 0, 0xCA5A826395121157ULL);
+                            xa = r1.v[0];
+                            xb = r1.v[1];
+                            xc = r1.v[2];
+                            xd = r1.v[3];
+                        } else if (e == 4) {
+                            xa = xc;
+                            xb = xd;
+                        }
+                        const bool two = e + 1 < sz;
+                        int ia, ib = 0;
+                        if (!local) {
+                            pick_two(pk, wa.bucket, bshift, nbk, n, below(xa, (u64)nex), below(xb, (u64)nex), two, ia, ib);
+                        } else {
+                            // simulated distribution: a composite's later
+                            // excitors come from the first one's processor
+                            if (e == 0) {
+                                ia = pick_index(pk, wa.bucket, bshift, nbk, n, below(xa, (u64)nex));
+                                lq = __ldg(&wa.owner[ia]);
+                                nq = __ldg(&wa.nq[lq]);
+                            } else {
+                                ia = (int)local_pick(wa, L.pop, n, st->lcs, st->nlc, lq, below(xa, (u64)nq));
+                            }
+                            if (two) ib = (int)local_pick(wa, L.pop, n, st->lcs, st->nlc, lq, below(xb, (u64)nq));
+                            if (ia < 0 || ib < 0) {   // tables inconsistent (cannot happen): a sticky error, not a guess
+                                valid = false;
+                                err |= ERRB_NUMERIC;
+                                break;
+                            }
+                        }
+                        if (e == 0) i0 = ia;
+#pragma unroll 1
+                        for (int k = 0; k <= (two ? 1 : 0) && valid; k++) {
+                            u64 f;
+                            const Exc x = row_exc(pk, k ? ib : ia, f);
+                            if (f & PICK_NEG) neg ^= 1;
+                            if (e + k == 0) {
+                                dj = x;
+                                par = (f & PICK_ODD) ? 1 : 0;
+                            } else {
+                                // within l + 2 (the levels add up) and
+                                // sharing no orbital, else the product vanishes
+                                valid = dj.n + x.n <= s.lmax + 2 && apply_excitor(s, x, dj, par);
+                            }
                         }
                     }
-                }
-                for (int e = 1; e < sz; e++)
-                    for (int f = 0; f < e; f++)
-                        if (idx[f] == idx[e]) valid = false;   // repeated excitor: discarded
-                if (sz == 1) {
-                    // one excitor: its own determinant, with the sign s_D of
-                    // applying it to HF (the closed form of the same product)
-                    const i64 id = idx[0];
-                    if (__ldg(&pk[id].pop) < 0) neg ^= 1;
-                    dj = pick_det<K>(pk, L, id);
-                    par = excitor_sign(s, dj) < 0 ? 1 : 0;
-                } else {
-                    for (int e = 0; e < sz && valid; e++) {
-                        const i64 id = idx[e];
-                        if (__ldg(&pk[id].pop) < 0) neg ^= 1;
-                        const Det<K> de = pick_det<K>(pk, L, id);
-                        if (!apply_excitor(s, de, dj, par)) valid = false;   // shared orbital
+                    if (dj.n > s.lmax + 2) valid = false;
+                    if (valid) {
+                        if (n0 < 0 && ((sz - 1) & 1)) neg ^= 1;
+                        double a = smag[sz];
+                        if (local) {
+                            // |A| = N_ex (N_q N_p)^(s-1) / (|t_HF|^(s-1) n_sel p(s) s!):
+                            // selection within q times co-location N_p^-(s-1)
+                            const double f = ((double)nq / FIX_ONE) * (double)p.nranks;
+                            double num = (double)nex / FIX_ONE;
+    #pragma unroll 1
+                            for (int e = 1; e < sz; e++) num = num * f;
+                            a = num / smden[sz];
+                        }
+                        const double amp = neg ? -a : a;
+                        coef = (par & 1) ? -amp : amp;
+                        const int lev = dj.n;
+                        // one excitor: its own determinant with s_D = its collapse sign, <HF|H|D> and death factor per entry
+                        if (lev == 1 || lev == 2) {
+                            if (sz == 1) es.add(to_fix(__ldg(&wa.href[i0]) * coef));
+                            else if (!GAS) es.add(to_fix(h_ref<R, GAS>(s, dj) * coef));   // a gas composite has level 4 or more
+                        }
+                        // death: tau (Delta E - S) C, of a composite within the truncation only
+                        if (sz == 1 || lev <= s.lmax) {
+                            double x = (sz == 1 ? __ldg(&pk[i0].tdeath) : p.tau * (diag_rel<R, GAS>(s, dj) - st->shift)) * coef;
+                            if (!(sz == 1 ? (par & 1) : sign_parity(s, dj))) x = -x;
+                            i64 d;
+                            if (!round_value(x, v1, p, false, d)) err |= ERRB_NUMERIC;
+                            if (d != 0) {
+                                if (sz == 1) {
+                                    atomicAdd((unsigned long long *)&wa.death[i0], (unsigned long long)d);
+                                } else {
+                                    rk = rank_key(s, dj);
+                                    rv = d;
+                                    rec = true;
+                                }
+                            }
+                        }
+                        // = attempts_of(|amp|): |amp| = mag[sz] for every cluster of
+                        // size sz, unless its processor's population sets it
+                        if (p.multispawn) natt = local ? attempts_of(fabs(amp), p) : snatt[sz];
                     }
                 }
-                if (valid) {
-                    if (n0 < 0 && ((sz - 1) & 1)) neg ^= 1;
-                    double a = smag[sz];
-                    if (local) {
-                        // |A| = N_ex (N_q N_p)^(s-1) / (|t_HF|^(s-1) n_sel p(s) s!):
-                        // selection within q times co-location N_p^-(s-1)
-                        const double f = ((double)nq / FIX_ONE) * (double)p.nranks;
-                        double num = (double)nex / FIX_ONE;
-                        for (int e = 1; e < sz; e++) num = num * f;
-                        a = num / smden[sz];
-                    }
-                    amp = neg ? -a : a;
-                    idx0 = idx[0];
-                }
+                rec_push(rb, rn, rec, rk, rv);
             }
-            int lev = valid ? level_of(s, dj) : 0;
-            if (valid && lev <= s.lmax + 2) {
-                coef = (par & 1) ? -amp : amp;
-                // a single excitor collapses to its own determinant: <HF|H|D> cached per entry
-                if (lev == 1 || lev == 2)
-                    es.add(to_fix((sz == 1 && !p.fnc ? __ldg(&pk[idx0].href) : h_ref<K, R>(s, dj)) * coef));
-                // s_D of the collapsed determinant (HF: +1; one excitor: known)
-                const int sdj = sz == 0 ? 1 : (sz == 1 ? ((par & 1) ? -1 : 1) : excitor_sign(s, dj));
-                if (sz <= 1) {
-                    double x = __ldg(&pk[idx0].tdeath) * coef;   // tau (Delta E - S) C (idx0 = 0 for the reference)
-                    if (sdj > 0) x = -x;
-                    i64 dv;
-                    if (!round_value(x, r0.v[1], p, false, dv)) err |= ERRB_NUMERIC;
-                    if (dv != 0) {
-                        if (idx0 == 0) death_hf += dv;   // hot entry: one atomic per block below
-                        else atomicAdd((unsigned long long *)&wa.death[idx0], (unsigned long long)dv);
-                    }
-                } else if (lev <= s.lmax) {
-                    double x = (p.tau * (diag_rel<K, R>(s, dj) - S)) * coef;
-                    if (sdj > 0) x = -x;
-                    i64 dv;
-                    if (!round_value(x, r0.v[1], p, false, dv)) err |= ERRB_NUMERIC;
-                    if (dv != 0) {
-                        rk = rank_key(s, dj);
-                        rv = dv;
-                        rec = true;
-                    }
-                }
-                // = attempts_of(|amp|): |amp| = mag[sz] for every cluster of
-                // size sz, unless its processor's population sets it
-                const bool local_amp = DIST && p.nranks > 1 && sz >= 2;
-                natt = local_amp ? attempts_of(fabs(amp), p) : snatt[sz];
-                valid_cl = true;
-                if (p.buffered) {
-                    catt = coef;    // the original sampler's one attempt
-                    cl_att += 1;
-                } else if (p.multispawn) {
+            if (p.multispawn && !is_w) natt = snatt[0];
+            __syncwarp();   // the entries are read before later pushes reuse them
+            wn -= tw;
+            hn -= th;
+            n_valid += valid ? 1u : 0u;
+            if (p.multispawn) {
+                // queued for the attempts kernel: one counter packs
+                // (clusters << CL_SHIFT | attempts)
+                double catt = coef;
+                if (valid) {
                     // coef / natt: the same division, done once per size
-                    if (local_amp) catt = natt > 1 ? coef / (double)natt : coef;
-                    else catt = natt > 1 ? (coef < 0.0 ? -scmag[sz] : scmag[sz]) : coef;
+                    if (natt > 1) catt = local ? coef / (double)natt : (coef < 0.0 ? -scmag[sz] : scmag[sz]);
                     if (natt > p.work_cap) {   // runaway: the attempts kernel will not run them
                         err |= ERRB_RUNAWAY;
                         natt = p.work_cap + 1;
                     }
-                    cl_att += (u64)natt;
+                    cl_att += (double)natt;
                 }
+                const u64 o = warp_reserve_u64(&st->cl_packed, valid ? ((1ULL << CL_SHIFT) | (u64)natt) : 0ULL);
+                if (valid) {
+                    const i64 c = (i64)(o >> CL_SHIFT);
+                    if (c < cl.cap) {
+                        cl.h[c] = pack_h(dj);
+                        cl.p[c] = dj.p;
+                        cl.catt[c] = catt;
+                        cl.index[c] = g;
+                        cl.end[c] = (i64)(o & CL_MASK) + natt;
+                    } else {
+                        err |= ERRB_CLUSTER_OVERFLOW;
+                    }
+                }
+                continue;
             }
         }
-        rec_push(rb, rn, rec, rk, rv);
-        rec_flush(rb, rn, false, st, sp, dv, ndirect, err);   // the stage holds fewer than 32 again
-        if (p.multispawn || p.buffered) {
-            // the cluster is queued for the attempts kernel: multi-spawn
-            // packs (clusters << CL_SHIFT | attempts) into one counter; the
-            // original sampler's one attempt per cluster counts clusters only
-            u64 mine = valid_cl ? (p.buffered ? 1ULL : ((1ULL << CL_SHIFT) | (u64)natt)) : 0ULL;
-            u64 o = warp_reserve_u64(&st->cl_packed, mine);
-            if (valid_cl) {
-                const i64 c = p.buffered ? (i64)o : (i64)(o >> CL_SHIFT);
-                if (c < cl.cap) {
-                    store_det<K>(cl.bits, cl.cap, c, dj);
-                    cl.catt[c] = catt;
-                    cl.index[c] = (u64)g;
-                    cl.end[c] = p.buffered ? c + 1 : (i64)(o & CL_MASK) + natt;
-                } else {
-                    err |= ERRB_CLUSTER_OVERFLOW;
-                }
+        // the selection draw of new samples, or one attempt per valid cluster
+        const R4 r = step_draw_at(ps, sel ? TAG_SAMPLE : TAG_SAMPLE_ATT, g, 0, 0);
+        if (sel) {
+            // the cluster size
+            g0 += stride;
+            valid = (i64)g < n_sel;
+            const u64 nr = ~r.v[0];
+            const int lz = nr ? __clzll((long long)nr) : 64;
+            const int sz = p.fnc ? 2 + min(lz, s.lmax) : min(lz, s.lmax + 2);
+            const bool hf = valid && sz == 0;
+            // a valid cluster's level is the sum of its excitors' levels: a
+            // size beyond (l + 2) / (smallest level) contributes nothing
+            const bool work = valid && sz > 0 && nex != 0 && (sz < 2 || n0 != 0) && sz * s.lmin_exc <= s.lmax + 2;
+            const unsigned mh = __ballot_sync(FULLMASK, hf), mw = __ballot_sync(FULLMASK, work);
+            if (hf) {
+                sw.hg[hn + __popc(mh & below_me)] = g;
+                i64 d = hf_cut.base + ((r.v[1] >> 11) < hf_cut.thr ? hf_cut.inc : 0);
+                bool in_range = hf_ok;
+                if (!p.int_round) in_range = round_value_fp(fabs(death_x), r.v[1], 0.0, &d);
+                if (!in_range) err |= ERRB_NUMERIC;
+                death_hf += death_x < 0.0 ? -d : d;
             }
+            if (work) {
+                const int e = wn + __popc(mw & below_me);
+                sw.g[e] = g;
+                sw.v1[e] = r.v[1];
+                sw.v2[e] = r.v[2];
+                sw.v3[e] = r.v[3];
+                sw.sz[e] = (unsigned char)sz;
+            }
+            hn += __popc(mh);
+            wn += __popc(mw);
+            __syncwarp();
         } else {
-            // one attempt per valid cluster, drawn and generated with the
-            // valid lanes together; the few that survive the generator and
-            // the truncation wait in the queue and are finished 32 at a time
-            bool ok = false;
+            // the draws that survive the generator and the truncation are finished 32 at a time
             u64 code = 0;
-            int gc = 0;
-            u64 r3 = 0;
-            if (valid_cl) {
-                inline_att++;
-                R4 ra = draw(p.seed, p.replica, it, TAG_SAMPLE_ATT, (u64)g, 0);
-                ok = attempt_draw<K>(s, dj, ra, code, gc);
-                r3 = ra.v[3];
-            }
-            q_push<K>(q, qn, ok, dj, coef, r3, code, gc);
-            q_drain_staged<K, R>(q, qn, false, rb, rn, s, p, st, sp, dv, ndirect, err);
+            const bool ok = valid && excite<GAS>(s, dj, r, code);
+            q_push(q, qn, ok, dj, coef, r.v[3], code);
         }
-        rec_flush(rb, rn, false, st, sp, dv, ndirect, err);
     }
-    q_drain_staged<K, R>(q, qn, true, rb, rn, s, p, st, sp, dv, ndirect, err);
-    rec_flush(rb, rn, true, st, sp, dv, ndirect, err);
-    es = block_fix(es, smf);
-    inline_att = block_sum(inline_att, sm);
-    death_hf = block_sum(death_hf, sm);
-    ndirect = block_sum(ndirect, sm);
-    if (p.multispawn || p.buffered) {
-        __shared__ double smd[32];
-        double ca = block_sum((double)cl_att, smd);
-        if (threadIdx.x == 0 && ca != 0.0) atomicAdd(&st->cl_att, ca);
+    // the block's sums: E_num, reference deaths, valid clusters, direct records, attempts
+    es = warp_fix(es);
+    death_hf = warp_sum(death_hf);
+    const unsigned nv = __reduce_add_sync(FULLMASK, n_valid), nd = __reduce_add_sync(FULLMASK, (unsigned)ndirect);
+    if (p.multispawn) cl_att = warp_sum(cl_att);
+    if (lane == 0) {
+        smf[2 * wid] = es.lo;
+        smf[2 * wid + 1] = es.hi;
+        sm[2 * wid] = death_hf;
+        sm[2 * wid + 1] = (i64)nv | ((i64)nd << 32);
+        if (p.multispawn && cl_att != 0.0) atomicAdd(&st->cl_att, cl_att);
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (death_hf) atomicAdd((unsigned long long *)&wa.death[0], (unsigned long long)death_hf);
-        wa.enum_part[2 * (enum_base + vb)] = es.lo;
-        wa.enum_part[2 * (enum_base + vb) + 1] = es.hi;
-        if (inline_att) atomicAdd((unsigned long long *)&st->n_attempts, (unsigned long long)inline_att);
-        if (ndirect) atomicAdd((unsigned long long *)&st->n_direct, (unsigned long long)ndirect);
+        Fix128 e = {0, 0};
+        i64 d = 0, v = 0, dr = 0;
+        for (int w = 0; w < WORK_THREADS / 32; w++) {
+            e.add(Fix128{smf[2 * w], smf[2 * w + 1]});
+            d += sm[2 * w];
+            v += sm[2 * w + 1] & 0xFFFFFFFFLL;
+            dr += sm[2 * w + 1] >> 32;
+        }
+        if (d) atomicAdd((unsigned long long *)&wa.death[0], (unsigned long long)d);
+        wa.enum_part[2 * (enum_base + vb)] = e.lo;
+        wa.enum_part[2 * (enum_base + vb) + 1] = e.hi;
+        if (v && !p.multispawn) {
+            atomicAdd((unsigned long long *)&st->n_attempts, (unsigned long long)v);
+            if (p.count_clusters) atomicAdd((unsigned long long *)&st->cl_packed, (unsigned long long)v);
+        }
+        if (dr) atomicAdd((unsigned long long *)&st->n_direct, (unsigned long long)dr);
     }
     if (err) atomicOr(&st->err, err);   // every thread reports its own bits
 }
@@ -1165,7 +1243,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
 // buffered composite clusters (Sec. IV.B-C)
 // ---------------------------------------------------------------------------
 
-template <int K, typename R>
+template <typename R, bool GAS>
 __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, DevStep *st, const RunParams &p,
                                                               const WorkArrays &wa, const SpawnBuf &sp, const ClusterBuf &cl)
 {
@@ -1176,64 +1254,76 @@ __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, D
         return;
     }
     const i64 n = st->n_occ, tf = st->fnc_attempts;
-    i64 ncl = p.buffered ? (i64)st->cl_packed : (i64)(st->cl_packed >> CL_SHIFT);
+    i64 ncl = p.multispawn ? (i64)(st->cl_packed >> CL_SHIFT) : 0;
     if (ncl > cl.cap) ncl = cl.cap;
     const i64 tc = ncl > 0 ? cl.end[ncl - 1] : 0;
-    const u64 it = st->iter;
     const int lane = threadIdx.x & 31;
     const i64 nwarps = (i64)gridDim.x * blockDim.x / 32;
     const i64 wglob = ((i64)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     unsigned err = 0;
-    __shared__ AttQueue<K> aq[WORK_THREADS / 32];
+    __shared__ AttQueue aq[WORK_THREADS / 32];
     __shared__ RecStage rsb[WORK_THREADS / 32];
     __shared__ i64 sm[32];
-    AttQueue<K> &q = aq[threadIdx.x >> 5];
+    __shared__ PhiloxStep ps;
+    philox_step_init(ps, st->iter, p.seed, p.replica);
+    __syncthreads();
+    AttQueue &q = aq[threadIdx.x >> 5];
     RecStage &rb = rsb[threadIdx.x >> 5];
     int qn = 0, rn = 0;   // drawn attempts and staged records of this warp (warp-uniform)
     i64 ndirect = 0;
     const DirectView dv = direct_view(L, wa, st);
-    for (int part = 0; part < 2; part++) {
-        // part 0: full non-composite attempts (owners: list entries);
-        // part 1: attempts of the composite clusters queued by k_sample
-        const i64 total = part == 0 ? tf : tc;
-        const i64 *end = part == 0 ? wa.att_end : cl.end;
-        const i64 nown = part == 0 ? n : ncl;
-        const i64 per = ((total + nwarps - 1) / nwarps + 31) & ~31LL;
-        const i64 a0 = wglob * per, a1 = a0 + per < total ? a0 + per : total;
-        if (a0 >= a1) continue;
-        AttemptWindow w = window_start(end, nown, a0);
-        for (i64 t0 = a0; t0 < a1; t0 += 32) {
-            i64 o, m;
-            window_step(end, nown, t0, w, o, m);
-            bool ok = false;
-            Det<K> dj;
-            double ca = 0.0;
-            u64 r3 = 0;
-            u64 code = 0;
-            int gc = 0;
-            if (t0 + lane < a1) {
-                u64 tag, idx;
-                if (part == 0) {
-                    dj = load_det<K>(L.bits, L.cap, o);
-                    ca = wa.catt[o];
-                    tag = TAG_VISIT_ATT;
-                    idx = (u64)o;
-                } else {
-                    dj = load_det<K>(cl.bits, cl.cap, o);
-                    ca = cl.catt[o];
-                    tag = TAG_SAMPLE_ATT;
-                    idx = cl.index[o];
-                }
-                R4 r = draw(p.seed, p.replica, it, tag, idx, (u64)m);
-                ok = attempt_draw<K>(s, dj, r, code, gc);
-                r3 = r.v[3];
-            }
-            q_push<K>(q, qn, ok, dj, ca, r3, code, gc);
-            q_drain_staged<K, R>(q, qn, false, rb, rn, s, p, st, sp, dv, ndirect, err);
+    // part 0: full non-composite attempts (owners: list entries); part 1:
+    // attempts of the composite clusters queued by k_sample; part 2: what is
+    // still queued.  One action per pass, as in the sampler.
+    int part = -1;
+    const i64 *end = nullptr;
+    i64 nown = 0, t0 = 0, a1 = 0;
+    AttemptWindow w = {0, 0};
+    for (;;) {
+        if (rn >= 32 || (part == 2 && qn == 0 && rn > 0)) {
+            rec_flush_once(rb, rn, st, sp, dv, ndirect, err);
+            continue;
         }
+        if (qn >= 32 || (part == 2 && qn > 0)) {
+            q_finish<R, GAS>(q, qn, rb, rn, s, p, err);
+            continue;
+        }
+        if (part == 2) break;
+        if (t0 >= a1) {
+            if (++part == 2) continue;
+            const i64 total = part == 0 ? tf : tc;
+            end = part == 0 ? wa.att_end : cl.end;
+            nown = part == 0 ? n : ncl;
+            const i64 per = ((total + nwarps - 1) / nwarps + 31) & ~31LL;
+            t0 = wglob * per;
+            a1 = t0 + per < total ? t0 + per : total;
+            if (t0 < a1) w = window_start(end, nown, t0);
+            continue;
+        }
+        i64 o, m;
+        window_step(end, nown, t0, w, o, m);
+        bool ok = false;
+        Exc dj = {0, 0, 0};
+        double ca = 0.0;
+        u64 r3 = 0, code = 0;
+        if (t0 + lane < a1) {
+            u64 tag = TAG_VISIT_ATT, idx = (u64)o;
+            if (part == 0) {
+                dj = exc_of(L.h[o], L.p[o]);
+                ca = wa.catt[o];
+            } else {
+                dj = exc_of(cl.h[o], cl.p[o]);
+                ca = cl.catt[o];
+                tag = TAG_SAMPLE_ATT;
+                idx = cl.index[o];
+            }
+            const R4 r = step_draw(ps, tag, idx, (u64)m);
+            ok = excite<GAS>(s, dj, r, code);
+            r3 = r.v[3];
+        }
+        q_push(q, qn, ok, dj, ca, r3, code);
+        t0 += 32;
     }
-    q_drain_staged<K, R>(q, qn, true, rb, rn, s, p, st, sp, dv, ndirect, err);
-    rec_flush(rb, rn, true, st, sp, dv, ndirect, err);
     ndirect = block_sum(ndirect, sm);
     if (threadIdx.x == 0 && ndirect) atomicAdd((unsigned long long *)&st->n_direct, (unsigned long long)ndirect);
     if (err) atomicOr(&st->err, err);
@@ -1536,7 +1626,6 @@ __device__ __forceinline__ void d_keep_top(DevStep *st, const WorkArrays &wa, in
 // before their scans; each kept entry goes to e_lo + e_hi + (new keys right
 // before it), and e is stored only where kept new keys are inserted (the
 // new-key scatter reads it there).
-template <int K>
 __device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView &O, DevStep *st, const WorkArrays &wa,
                                                int G)
 {
@@ -1588,10 +1677,13 @@ __device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView
                 err |= ERRB_LIST_OVERFLOW;
                 continue;
             }
-            store_det<K>(O.bits, O.cap, out, load_det<K>(L.bits, L.cap, i));
-            O.key[out] = L.key[i];
+            const u64 eh = L.h[i], ep = L.p[i], ek = L.key[i];
+            const double ed = L.diag[i];
+            O.h[out] = eh;
+            O.p[out] = ep;
+            O.key[out] = ek;
             O.pop[out] = v[r];
-            O.diag[out] = L.diag[i];
+            O.diag[out] = ed;
             asum += v[r] < 0 ? -v[r] : v[r];
         }
     }
@@ -1602,7 +1694,7 @@ __device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView
     if (err) atomicOr(&st->err, err);   // every thread reports its own bits
 }
 
-template <int K, typename R>
+template <typename R, bool GAS>
 __device__ __forceinline__ void d_scatter_new(const SysDev &s, const ListView &O, DevStep *st, const WorkArrays &wa,
                                                                const u64 *rkey, const i64 *rpop)
 {
@@ -1620,11 +1712,12 @@ __device__ __forceinline__ void d_scatter_new(const SysDev &s, const ListView &O
             continue;
         }
         u64 k = rkey[j];
-        Det<K> d = unrank_key<K>(s, k);
-        store_det<K>(O.bits, O.cap, out, d);
+        const Exc d = unrank_key(s, k);
+        O.h[out] = pack_h(d);
+        O.p[out] = d.p;
         O.key[out] = k;
         O.pop[out] = v;
-        O.diag[out] = diag_rel<K, R>(s, d);
+        O.diag[out] = diag_rel<R, GAS>(s, d);
         asum += v < 0 ? -v : v;
     }
     asum = block_sum(asum, sm);
@@ -1649,9 +1742,13 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
     }
     k = block_fix(k, smf);
     if (threadIdx.x == 0) {
-        i64 ncl = p.buffered ? (i64)st->cl_packed : (i64)(st->cl_packed >> CL_SHIFT);
-        if (ncl > cl.cap) ncl = cl.cap;
-        i64 tc = ncl > 0 ? cl.end[ncl - 1] : 0;
+        i64 ncl = p.multispawn ? (i64)(st->cl_packed >> CL_SHIFT) : (i64)st->cl_packed;
+        if (ncl > cl.cap) {
+            // the generic original sampler's clusters are bounded like multi-spawn's buffer
+            if (!p.multispawn) st->err |= ERRB_CLUSTER_OVERFLOW;
+            ncl = cl.cap;
+        }
+        i64 tc = p.multispawn && ncl > 0 ? cl.end[ncl - 1] : 0;
         Record r;
         r.iter = st->iter;
         r.shift = st->shift;
@@ -1717,25 +1814,31 @@ __global__ void __launch_bounds__(WORK_THREADS) k_merge_match(const StepArgs *__
 __global__ void __launch_bounds__(SCAN_THREADS) k_merge_count(const StepArgs *__restrict__ A, int G);
 __global__ void __launch_bounds__(SCAN_THREADS) k_local_scan(const StepArgs *__restrict__ A);
 __global__ void __launch_bounds__(1024) k_keep_top(const StepArgs *__restrict__ A, int G);
+__global__ void __launch_bounds__(SCAN_THREADS) k_keep_scatter(const StepArgs *__restrict__ A, int G);
 __global__ void __launch_bounds__(1024) k_finalize(const StepArgs *__restrict__ A, int slots);
+// owners and position table of the simulated distribution, for K words
+void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm);
 
-template <int K, typename R>
+template <typename R, bool GAS>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_final(const StepArgs *__restrict__ A)
 {
     REPLICA_SMEM;
-    d_scan_final<K, R>(a.s, a.list[cur_], a.st, a.p, a.wa);
+    d_scan_final<R, GAS>(a.s, a.list[cur_], a.st, a.p, a.wa);
 }
 
-template <int K, typename R, bool DIST>
+extern __shared__ __align__(16) unsigned char dyn_smem[];
+
+template <typename R, bool GAS, bool DIST>
 __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_sample(const StepArgs *__restrict__ A, int enum_base)
 {
     REPLICA_SMEM;
-    d_sample<K, R, DIST>(a.s, a.list[cur_], a.st, a.p, a.wa, a.sp, a.cl, enum_base, blockIdx.x, gridDim.x);
+    d_sample<R, GAS, DIST>(a.s, a.list[cur_], a.st, a.p, a.wa, a.sp, a.cl, enum_base, blockIdx.x, gridDim.x,
+                           ((SampWarp *)dyn_smem)[threadIdx.x >> 5]);
 }
 
 // Persistent batch sampler: each block takes the next virtual block of the
 // plan, finds its replica and runs that share of the replica's samples.
-template <int K, typename R, bool DIST>
+template <typename R, bool GAS, bool DIST>
 __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_sample_flat(const StepArgs *__restrict__ A, int nrep, FlatPlan fp,
                                                                  int enum_base)
 {
@@ -1773,37 +1876,23 @@ __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_sample_f
         }
         const StepArgs &a = a_sm;
         const int v0 = fp.vstart[r];
-        d_sample<K, R, DIST>(a.s, a.list[a.st->cur], a.st, a.p, a.wa, a.sp, a.cl, enum_base, v - v0,
-                       fp.vstart[r + 1] - v0);
+        d_sample<R, GAS, DIST>(a.s, a.list[a.st->cur], a.st, a.p, a.wa, a.sp, a.cl, enum_base, v - v0,
+                               fp.vstart[r + 1] - v0, ((SampWarp *)dyn_smem)[threadIdx.x >> 5]);
     }
 }
 
-template <int K, typename R>
-__global__ void __launch_bounds__(WORK_THREADS, 4) k_attempts(const StepArgs *__restrict__ A)
+template <typename R, bool GAS>
+__global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_attempts(const StepArgs *__restrict__ A)
 {
     REPLICA_SMEM;
-    d_attempts<K, R>(a.s, a.list[cur_], a.st, a.p, a.wa, a.sp, a.cl);
+    d_attempts<R, GAS>(a.s, a.list[cur_], a.st, a.p, a.wa, a.sp, a.cl);
 }
 
-template <int K>
-__global__ void __launch_bounds__(WORK_THREADS) k_local_table(const StepArgs *__restrict__ A)
-{
-    REPLICA;
-    d_local_table<K>(a.list[cur_], a.st, a.p, a.wa);
-}
-
-template <int K>
-__global__ void __launch_bounds__(SCAN_THREADS) k_keep_scatter(const StepArgs *__restrict__ A, int G)
-{
-    REPLICA;
-    d_keep_scatter<K>(a.list[cur_], a.list[cur_ ^ 1], a.st, a.wa, G);
-}
-
-template <int K, typename R>
+template <typename R, bool GAS>
 __global__ void __launch_bounds__(WORK_THREADS) k_scatter_new(const StepArgs *__restrict__ A, int src)
 {
     REPLICA;
-    d_scatter_new<K, R>(a.s, a.list[cur_ ^ 1], a.st, a.wa, a.sp.key[src ^ 1], a.sp.pop[src ^ 1]);
+    d_scatter_new<R, GAS>(a.s, a.list[cur_ ^ 1], a.st, a.wa, a.sp.key[src ^ 1], a.sp.pop[src ^ 1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1811,8 +1900,8 @@ __global__ void __launch_bounds__(WORK_THREADS) k_scatter_new(const StepArgs *__
 // every step, so it can be captured once in a CUDA graph.
 // ---------------------------------------------------------------------------
 
-template <int K, typename R>
-cudaError_t launch_phases(const StepArgs *A, int nrep, const Shapes &sh, bool multi_att, cudaStream_t sm,
+template <typename R, bool GAS>
+cudaError_t launch_phases(const StepArgs *A, int nrep, int K, const Shapes &sh, bool multi_att, cudaStream_t sm,
                           i64 *launches, const cudaEvent_t *ev, const FlatPlan *plan)
 {
     auto mark = [&](int phase) {
@@ -1822,28 +1911,32 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, const Shapes &sh, bool mu
     mark(0);
     k_scan_partial<<<gscan, SCAN_THREADS, 0, sm>>>(A);
     k_scan_top<<<gone, 1024, 0, sm>>>(A, sh.scan_grid);
-    k_scan_final<K, R><<<gscan, SCAN_THREADS, 0, sm>>>(A);
+    k_scan_final<R, GAS><<<gscan, SCAN_THREADS, 0, sm>>>(A);
     launches[0] += 3;
     if (sh.nranks > 1) {
         // simulated distribution: owners and per-processor position tables
-        k_local_table<K><<<gwork, WORK_THREADS, 0, sm>>>(A);
+        launch_local_table(A, K, gwork, sm);
         k_local_scan<<<dim3(sh.nranks < 1024 ? sh.nranks : 1024, nrep), SCAN_THREADS, 0, sm>>>(A);
         launches[0] += 2;
     }
     mark(1);
+    const size_t smem = (WORK_THREADS / 32) * sizeof(SampWarp);
+    const bool dist = sh.nranks > 1;
     if (plan) {
+        auto *k = dist ? k_sample_flat<R, GAS, true> : k_sample_flat<R, GAS, false>;
+        if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
         k_sample_plan<<<1, 1024, 0, sm>>>(A, nrep, *plan, sh.scan_grid);
-        if (sh.nranks > 1) k_sample_flat<K, R, true><<<plan->grid, WORK_THREADS, 0, sm>>>(A, nrep, *plan, sh.scan_grid);
-        else k_sample_flat<K, R, false><<<plan->grid, WORK_THREADS, 0, sm>>>(A, nrep, *plan, sh.scan_grid);
+        k<<<plan->grid, WORK_THREADS, smem, sm>>>(A, nrep, *plan, sh.scan_grid);
         launches[1] += 2;
     } else {
-        if (sh.nranks > 1) k_sample<K, R, true><<<gwork, WORK_THREADS, 0, sm>>>(A, sh.scan_grid);
-        else k_sample<K, R, false><<<gwork, WORK_THREADS, 0, sm>>>(A, sh.scan_grid);
+        auto *k = dist ? k_sample<R, GAS, true> : k_sample<R, GAS, false>;
+        if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
+        k<<<gwork, WORK_THREADS, smem, sm>>>(A, sh.scan_grid);
         launches[1] += 1;
     }
     mark(2);
     if (multi_att) {
-        k_attempts<K, R><<<gwork, WORK_THREADS, 0, sm>>>(A);
+        k_attempts<R, GAS><<<gwork, WORK_THREADS, 0, sm>>>(A);
         launches[2] += 1;
     }
     mark(3);
@@ -1865,8 +1958,8 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, const Shapes &sh, bool mu
     k_merge_match<<<gwork, WORK_THREADS, 0, sm>>>(A, src);
     k_merge_count<<<dim3(2 * sh.scan_grid, nrep), SCAN_THREADS, 0, sm>>>(A, sh.scan_grid);
     k_keep_top<<<gone, 1024, 0, sm>>>(A, sh.scan_grid);
-    k_keep_scatter<K><<<dim3(2 * sh.scan_grid, nrep), SCAN_THREADS, 0, sm>>>(A, sh.scan_grid);
-    k_scatter_new<K, R><<<gwork, WORK_THREADS, 0, sm>>>(A, src);
+    k_keep_scatter<<<dim3(2 * sh.scan_grid, nrep), SCAN_THREADS, 0, sm>>>(A, sh.scan_grid);
+    k_scatter_new<R, GAS><<<gwork, WORK_THREADS, 0, sm>>>(A, src);
     launches[5] += 5;
     mark(6);
     k_finalize<<<gone, 1024, 0, sm>>>(A, plan ? sh.scan_grid + plan->wmax : sh.enum_slots);

@@ -16,7 +16,7 @@ constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;
 constexpr int MAX_DIGIT_BITS = 8;
 // resident blocks of the cluster sampler per SM (its register budget)
 #ifndef CCMC_SAMPLE_BLOCKS_PER_SM
-#define CCMC_SAMPLE_BLOCKS_PER_SM 4
+#define CCMC_SAMPLE_BLOCKS_PER_SM 3
 #endif
 constexpr int SAMPLE_BLOCKS_PER_SM = CCMC_SAMPLE_BLOCKS_PER_SM;
 constexpr int RING = 1 << 14;             // per-step records kept on the device
@@ -33,7 +33,7 @@ struct RunParams {
     int int_round;        // rounding decisions from the FP64 bit pattern (cutoff 0 or 2^k)
     int a_thresh_one;     // A_thresh == 1: floor(|A|) without a division
     int direct;           // spawns onto listed determinants are added to them directly (not sorted)
-    int buffered;         // original sampler: each valid cluster's one attempt runs in the attempts kernel
+    int count_clusters;   // generic original sampler: valid clusters are counted (record, capacity check)
     int nranks;           // simulated processors (Sec. III): composite clusters from one processor's excitors
     int nu_move;          // owners move every 2^nu_move iterations (>= 64: never)
     i64 work_cap;         // samples, visit attempts or cluster attempts per step beyond which the step is abandoned
@@ -43,7 +43,7 @@ struct RunParams {
 
 // Excip list, structure of arrays with capacity cap.
 struct ListView {
-    u64 *bits;      // bits[w * cap + i]
+    u64 *h, *p;     // the determinant's holes (and level) and particles, see Exc
     u64 *key;
     i64 *pop;
     double *diag;   // H_DD - E_HF
@@ -107,28 +107,32 @@ struct SpawnBuf {
 
 // Clusters buffered for expanded multi-spawn attempts.
 struct ClusterBuf {
-    u64 *bits;      // bits[w * cap + c]
+    u64 *h, *p;     // holes (and level) and particles of the collapsed determinant
     double *catt;   // coefficient of one attempt
     u64 *index;     // sample index g (Philox counter)
     i64 *end;       // inclusive attempt prefix
-    i64 cap;
+    i64 cap;        // also the bound on the clusters the generic original sampler may form
 };
 
-// The cluster sampler's view of one list entry besides its bit string,
-// written by the scans each step and gathered by a pick as one 32-byte
-// sector: selection prefix, population, death factor and <HF|H|D>.
-struct __align__(64) PickEntry {
+// The cluster sampler's view of one list entry, written by the scans each
+// step: one 32-byte sector per probe of a pick's search, and the last probe
+// brings the whole excitor.  (64-byte rows with the determinant's words made
+// the 1.1e7-entry molecule list's scan write twice as much and its sampler
+// read two sectors per pick.)
+struct __align__(32) PickEntry {
     i64 prefix;     // inclusive |pop| prefix over entries >= 1 (entry 0: 0)
-    i64 pop;
+    u64 h;          // holes and level (Exc)
+    u64 p;          // particles | PICK_ODD | PICK_NEG
     double tdeath;  // tau (Delta E_i - S): the death factor of this step
-    double href;    // <HF|H|D_i> (levels 1-2; 0 otherwise; 0 with full non-composite sampling)
-    u64 w[4];       // the determinant's words (up to four; more are read from the list)
 };
-static_assert(sizeof(PickEntry) == 64, "pick table rows are one 64-byte granule");
+static_assert(sizeof(PickEntry) == 32, "pick table rows are one 32-byte sector");
+constexpr u64 PICK_ODD = 1ULL << 62;   // s_D = -1
+constexpr u64 PICK_NEG = 1ULL << 63;   // negative population
 
 // Per-step work arrays over the list and the merge.
 struct WorkArrays {
     PickEntry *picks; // one row per list entry
+    double *href;     // <HF|H|D_i> (levels 1-2, else 0; not with full non-composite sampling)
     int *bucket;      // owner of the first position of each selection bucket
     int bucket_bits;  // log2 of the bucket capacity
     i64 *att_end;     // inclusive prefix of full non-composite attempts
@@ -181,7 +185,8 @@ struct StepArgs {
 
 // Everything the step launcher needs.
 struct StepCtx {
-    int K;
+    int K;                // words per determinant (host rows and the owner hash)
+    bool gas;
     bool fp32;            // FP32 matrix elements and generation probabilities
     SysDev sys;
     RunParams prm;
@@ -220,11 +225,12 @@ struct FlatPlan {
 // Issues one full time step on ctx.stream.  Returns a CUDA error code.
 cudaError_t launch_step(StepCtx &ctx);
 
-// Issues one step for nrep replicas of the same word count and precision
-// whose arguments are A[0..nrep); launch counts are added to launches[7].
-// With a work plan the sampler runs as one persistent launch over all of
-// them, with blocks shared out in proportion to each replica's samples.
-cudaError_t launch_group(const StepArgs *A, int nrep, int K, bool fp32, const Shapes &sh, bool multi_att,
+// Issues one step for nrep replicas of the same Hamiltonian kind and precision
+// (and, with a simulated distribution, the same word count K) whose arguments
+// are A[0..nrep); launch counts are added to launches[7].  With a work plan
+// the sampler runs as one persistent launch over all of them, with blocks
+// shared out in proportion to each replica's samples.
+cudaError_t launch_group(const StepArgs *A, int nrep, int K, bool gas, bool fp32, const Shapes &sh, bool multi_att,
                          cudaStream_t sm, i64 *launches, const cudaEvent_t *ev, const FlatPlan *plan = nullptr);
 
 // Number of radix passes for the shapes.

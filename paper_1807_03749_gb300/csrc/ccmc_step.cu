@@ -1,12 +1,12 @@
 // ccmc_step.cu -- the kernels of one CCMC time step (Spencer et al.,
 // arXiv:1807.03749, Sec. II and Sec. IV.B-C) that do not depend on the
-// determinant word count, the dispatch of a step to the word count's
-// instantiation (ccmc_step_k<K>.cu) and the allocation-free sort-and-reduce
-// entry point.  The device building blocks are in ccmc_kernels.cuh.
+// Hamiltonian kind or the precision, the dispatch of a step to its
+// instantiation (ccmc_step_<kind>_<precision>.cu) and the allocation-free
+// sort-and-reduce entry point.  The device building blocks are in ccmc_kernels.cuh.
 //
 //  a1  k_scan_partial / k_scan_top           a7  k_sort_hist / scan / scatter
 //  a8  k_seg_count / k_part_scan / k_seg_write
-//  a9  k_merge_match / k_merge_count / k_keep_top (k_keep_scatter, k_scatter_new: per word count)
+//  a9  k_merge_match / k_merge_count / k_keep_top / k_keep_scatter (k_scatter_new: per kind and precision)
 //  a10 k_finalize      batch: k_sample_plan
 //  ccmc_reduce_records_noalloc (end of file): the sort and reduction as a
 //      standalone call on a static scratch array
@@ -134,6 +134,31 @@ __global__ void __launch_bounds__(1024) k_keep_top(const StepArgs *__restrict__ 
     d_keep_top(a.st, a.wa, G);
 }
 
+__global__ void __launch_bounds__(SCAN_THREADS) k_keep_scatter(const StepArgs *__restrict__ A, int G)
+{
+    REPLICA;
+    d_keep_scatter(a.list[cur_], a.list[cur_ ^ 1], a.st, a.wa, G);
+}
+
+template <int K>
+__global__ void __launch_bounds__(WORK_THREADS) k_local_table(const StepArgs *__restrict__ A)
+{
+    REPLICA;
+    d_local_table<K>(a.s, a.list[cur_], a.st, a.p, a.wa);
+}
+
+void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm)
+{
+    switch (K) {
+    case 1: k_local_table<1><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    case 2: k_local_table<2><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    case 3: k_local_table<3><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    case 4: k_local_table<4><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    case 5: k_local_table<5><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    default: k_local_table<6><<<grid, WORK_THREADS, 0, sm>>>(A); break;
+    }
+}
+
 __global__ void __launch_bounds__(1024) k_finalize(const StepArgs *__restrict__ A, int slots)
 {
     REPLICA;
@@ -192,46 +217,29 @@ int sort_passes(const Shapes &sh)
     return (sh.key_bits + sh.digit_bits - 1) / sh.digit_bits;
 }
 
-// instantiated in ccmc_step_k<K>.cu
-#define CCMC_EXTERN_LAUNCH(K, R)                                                                              \
-    extern template cudaError_t launch_phases<K, R>(const StepArgs *, int, const Shapes &, bool, cudaStream_t, \
-                                                    i64 *, const cudaEvent_t *, const FlatPlan *)
-CCMC_EXTERN_LAUNCH(1, double);
-CCMC_EXTERN_LAUNCH(2, double);
-CCMC_EXTERN_LAUNCH(3, double);
-CCMC_EXTERN_LAUNCH(4, double);
-CCMC_EXTERN_LAUNCH(5, double);
-CCMC_EXTERN_LAUNCH(6, double);
-CCMC_EXTERN_LAUNCH(1, float);
-CCMC_EXTERN_LAUNCH(2, float);
-CCMC_EXTERN_LAUNCH(3, float);
+// instantiated in ccmc_step_<kind>_<precision>.cu
+#define CCMC_EXTERN_LAUNCH(R, GAS)                                                                            \
+    extern template cudaError_t launch_phases<R, GAS>(const StepArgs *, int, int, const Shapes &, bool,       \
+                                                      cudaStream_t, i64 *, const cudaEvent_t *, const FlatPlan *)
+CCMC_EXTERN_LAUNCH(double, true);
+CCMC_EXTERN_LAUNCH(double, false);
+CCMC_EXTERN_LAUNCH(float, true);
+CCMC_EXTERN_LAUNCH(float, false);
 
-cudaError_t launch_group(const StepArgs *A, int nrep, int K, bool fp32, const Shapes &sh, bool multi_att,
+cudaError_t launch_group(const StepArgs *A, int nrep, int K, bool gas, bool fp32, const Shapes &sh, bool multi_att,
                          cudaStream_t sm, i64 *launches, const cudaEvent_t *ev, const FlatPlan *plan)
 {
-    if (fp32) {   // the FP32 form: up to three words (M <= 192)
-        switch (K) {
-        case 1: return launch_phases<1, float>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-        case 2: return launch_phases<2, float>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-        case 3: return launch_phases<3, float>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-        default: return cudaErrorInvalidValue;
-        }
-    }
-    switch (K) {
-    case 1: return launch_phases<1, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    case 2: return launch_phases<2, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    case 3: return launch_phases<3, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    case 4: return launch_phases<4, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    case 5: return launch_phases<5, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    case 6: return launch_phases<6, double>(A, nrep, sh, multi_att, sm, launches, ev, plan);
-    default: return cudaErrorInvalidValue;
-    }
+    if (fp32)
+        return gas ? launch_phases<float, true>(A, nrep, K, sh, multi_att, sm, launches, ev, plan)
+                   : launch_phases<float, false>(A, nrep, K, sh, multi_att, sm, launches, ev, plan);
+    return gas ? launch_phases<double, true>(A, nrep, K, sh, multi_att, sm, launches, ev, plan)
+               : launch_phases<double, false>(A, nrep, K, sh, multi_att, sm, launches, ev, plan);
 }
 
 cudaError_t launch_step(StepCtx &c)
 {
-    cudaError_t e = launch_group(c.d_args, 1, c.K, c.fp32, c.sh, c.prm.fnc || c.prm.multispawn || c.prm.buffered, c.stream, c.launches,
-                                 c.profile ? c.events : nullptr);
+    cudaError_t e = launch_group(c.d_args, 1, c.K, c.gas, c.fp32, c.sh, c.prm.fnc || c.prm.multispawn, c.stream,
+                                 c.launches, c.profile ? c.events : nullptr);
     c.sorted_buf = sort_passes(c.sh) & 1;
     c.cur ^= 1;
     return e;
