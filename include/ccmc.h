@@ -317,9 +317,9 @@ void ccmc_batch_free(ccmc_batch *b);
  *   n_out              host pointer; receives the number of distinct keys
  *   cuda_stream        cudaStream_t for the work (NULL = legacy stream); the
  *                      call waits for it before returning
- * Scratch is one fixed device array inside the library of about 2.07 MiB
+ * Scratch is one fixed device array inside the library of about 2.1 MiB
  * (two ping-pong buffers of CCMC_NOALLOC_MAX_RECORDS keys and weights, 2 MiB,
- * plus histograms, block partials and counters), held by every GPU that
+ * plus histograms, block partials and barriers), held by every GPU that
  * loads the library until the process exits.  n above
  * CCMC_NOALLOC_MAX_RECORDS is rejected with CCMC_ERR_ARG before any work.
  * The first call on a device looks up that array's device address (once per

@@ -220,6 +220,7 @@ struct ccmc_ctx {
     double nprev = 0.0;
     u64 records_read = 0;
     bool stepped = false;
+    bool timed_out = false;       // a device wait gave up: the barriers are reset with the next list
     // pinned staging
     DevStep *h_st = nullptr;
     double *h_shift = nullptr;
@@ -279,6 +280,10 @@ ccmc_status status_from_bits(ccmc_ctx *ctx, unsigned bits)
     if (bits & ERRB_RUNAWAY)
         return fail(ctx, CCMC_ERR_RUNAWAY, "population runaway: a step needed more than max(64 x target_pop, 2^24) "
                                            "samples or spawning attempts");
+    if (bits & ERRB_TIMEOUT) {
+        ctx->timed_out = true;
+        return fail(ctx, CCMC_ERR_TIMEOUT, "a wait between the blocks of a step gave up");
+    }
     if (bits & ERRB_SPAWN_OVERFLOW) return fail(ctx, CCMC_ERR_SPAWN_OVERFLOW, "spawned particles exceeded spawn_capacity");
     if (bits & ERRB_CLUSTER_OVERFLOW) return fail(ctx, CCMC_ERR_SPAWN_OVERFLOW, "multi-spawn clusters exceeded capacity");
     if (bits & ERRB_LIST_OVERFLOW) return fail(ctx, CCMC_ERR_LIST_OVERFLOW, "occupied excitors exceeded list_capacity");
@@ -636,7 +641,7 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     sh.work_grid = SAMPLE_BLOCKS_PER_SM * nsm;   // one wave of the sampler and attempt kernels
     sh.sort_grid = 2 * nsm;
     sh.key_bits = bits_for(key_bound);
-    sh.digit_bits = params->radix_bits ? params->radix_bits : MAX_DIGIT_BITS;
+    sh.digit_bits = params->radix_bits ? params->radix_bits : SORT_DIGIT_BITS;
     sh.enum_slots = sh.scan_grid + sh.work_grid;
     sh.nranks = rp.nranks;
     ctx->sc.K = h.nw;
@@ -689,10 +694,9 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     wa.keep_s = al.arr<i64>(sp.cap);
     wa.ins = al.arr<i64>(sp.cap);
     wa.part = al.arr<i64>(4 * 2 * (size_t)std::max(sh.scan_grid, sh.work_grid));
-    wa.wpart = al.arr<i64>(4 * (size_t)sh.scan_grid * (SCAN_THREADS / 32));
+    wa.bar = al.arr<unsigned>(64);
     wa.enum_part = al.arr<u64>(2 * (size_t)sh.enum_slots);
-    wa.hist = al.arr<unsigned>((size_t)(1 << MAX_DIGIT_BITS) * sh.sort_grid);
-    wa.hist_tot = al.arr<unsigned>((size_t)(1 << MAX_DIGIT_BITS));
+    wa.hist = al.arr<unsigned>((size_t)(1 << SORT_DIGIT_BITS) * sh.sort_grid);
     wa.ring = al.arr<Record>(RING);
     wa.owner = nullptr;
     wa.lcp = nullptr;
@@ -751,6 +755,7 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
         }
     }
 
+    ctx->timed_out = true;   // the barriers start at zero with the first list
     // initial state: d0_init on HF
     ctx->iter = 0;
     ctx->shift = 0.0;
@@ -832,6 +837,8 @@ ccmc_status ccmc_set_list(ccmc_ctx *ctx, const uint64_t *bits, const int64_t *po
     st.n_occ = (i64)n;
     st.cur = ctx->sc.cur;
     CK(cudaMemcpy(ctx->sc.st, &st, sizeof(DevStep), cudaMemcpyHostToDevice));
+    if (ctx->timed_out) CK(cudaMemset(ctx->sc.wa.bar, 0, 64 * sizeof(unsigned)));
+    ctx->timed_out = false;
     ctx->stepped = false;
     return CCMC_OK;
 }
@@ -998,8 +1005,12 @@ ccmc_status ccmc_get_records(ccmc_ctx *ctx, ccmc_record *out, size_t cap, size_t
         count = cap;
     }
     static_assert(sizeof(Record) == sizeof(ccmc_record), "record layout");
-    for (u64 k = 0; k < count; k++)
-        CK(cudaMemcpy(out + k, ctx->sc.wa.ring + ((first + k) % RING), sizeof(Record), cudaMemcpyDeviceToHost));
+    // the ring's records in at most two pieces
+    for (u64 k = 0; k < count;) {
+        const u64 at = (first + k) % RING, m = std::min<u64>(count - k, (u64)RING - at);
+        CK(cudaMemcpy(out + k, ctx->sc.wa.ring + at, m * sizeof(Record), cudaMemcpyDeviceToHost));
+        k += m;
+    }
     ctx->records_read = ctx->iter;
     *n = (size_t)count;
     return CCMC_OK;

@@ -38,7 +38,8 @@ enum : unsigned {
     ERRB_NUMERIC = 2u,
     ERRB_LIST_OVERFLOW = 4u,
     ERRB_CLUSTER_OVERFLOW = 8u,
-    ERRB_RUNAWAY = 16u
+    ERRB_RUNAWAY = 16u,
+    ERRB_TIMEOUT = 32u
 };
 
 // Hamiltonian and generator tables as seen by the kernels (passed by value).
@@ -454,7 +455,7 @@ __device__ __forceinline__ u64 rank_key(const SysDev &s, const Exc &e)
     return rv * s.cocc - rh;
 }
 
-__device__ __forceinline__ Exc unrank_key(const SysDev &s, u64 key)
+__device__ __forceinline__ Exc unrank_key(const SysDev &s, const u64 *tab, u64 key)
 {
     Exc e = {0, 0, 0};
     u64 rv = (key + s.cocc - 1) / s.cocc;
@@ -464,28 +465,28 @@ __device__ __forceinline__ Exc unrank_key(const SysDev &s, u64 key)
     // rank has no further digits) -- a binary search per digit
     int top = s.nso - s.nel;
     for (int c = 0; c <= s.lmax && rv > 0 && top > 0; c++) {
-        const u64 *t = s.rank_tab + c * RANK_STRIDE;
+        const u64 *t = tab + c * RANK_STRIDE;
         int lo = 0, hi = top - 1;   // tab[c][0] = 1 <= rv
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(&t[mid]) <= rv) lo = mid;
+            if (t[mid] <= rv) lo = mid;
             else hi = mid - 1;
         }
-        rv -= __ldg(&t[lo]);
+        rv -= t[lo];
         e.p = (e.p << FB) | (u64)(lo + s.nel);   // the digits descend
         e.n++;
         top = lo;
     }
     top = s.nel;
     for (int c = 0; c <= s.lmax && rh > 0 && top > 0; c++) {
-        const u64 *t = s.rank_tab + c * RANK_STRIDE;
+        const u64 *t = tab + c * RANK_STRIDE;
         int lo = 0, hi = top - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(&t[mid]) <= rh) lo = mid;
+            if (t[mid] <= rh) lo = mid;
             else hi = mid - 1;
         }
-        rh -= __ldg(&t[lo]);
+        rh -= t[lo];
         e.h = (e.h << FB) | (u64)lo;
         top = lo;
     }
@@ -963,25 +964,5 @@ __host__ __device__ __forceinline__ double fix_to_double(Fix128 v)
     double d = (double)v.hi + (double)v.lo * 0x1p-64;
     return neg ? -d : d;
 }
-
-// ---------------------------------------------------------------------------
-// Neumaier-compensated accumulation
-// ---------------------------------------------------------------------------
-
-struct KSum {
-    double s, c;
-    __device__ __forceinline__ void add(double x)
-    {
-        double t = s + x;
-        if (fabs(s) >= fabs(x)) c += (s - t) + x;
-        else c += (x - t) + s;
-        s = t;
-    }
-    __device__ __forceinline__ void merge(const KSum &o)
-    {
-        add(o.s);
-        add(o.c);
-    }
-};
 
 }  // namespace ccmc

