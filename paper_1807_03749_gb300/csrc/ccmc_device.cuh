@@ -383,15 +383,6 @@ __device__ __forceinline__ Det<K> words_from_exc(const SysDev &s, const Exc &e)
     return d;
 }
 
-// parity of the number of occupied spin-orbitals below x: the core below x
-// without the holes there, or the whole core without the holes and the
-// particles below x
-__device__ __forceinline__ int occ_below_parity(const SysDev &s, const Exc &e, int x)
-{
-    const bool core = x < s.nel;
-    return (core ? x : s.nel + e.n) + fields_below(core ? e.h : e.p, e.n, x);
-}
-
 // s_D = <D|c_D|HF>: annihilating the holes h_1 < ... < h_n of HF in ascending
 // order meets h_m - (m-1) occupied orbitals below h_m; creating the particles
 // in descending order meets the N - n remaining electrons each time.  The sign
@@ -412,28 +403,35 @@ __device__ __forceinline__ int sign_parity(const SysDev &s, const Exc &e)
 // orbital emptied or filled twice; so does a repeated excitor).
 __device__ __forceinline__ bool apply_excitor(const SysDev &s, const Exc &e, Exc &cur, int &parity)
 {
+    // one pass over cur counts, for each orbital of e (at most four of each),
+    // the fields below it
+    // (the counts packed four bits each: registers decide the sampler's speed)
     bool ok = true;
-    // x - c core orbitals below a hole x with c holes below it; N - n + c
-    // orbitals below a particle with c particles below it (n: all holes of the
-    // product), the larger ones of e being created first
+    unsigned ch = 0, cp = 0;
+    u64 th = cur.h, tp = cur.p;
+#pragma unroll 1
+    for (int q = cur.n; q > 0; q--, th >>= FB, tp >>= FB) {
+        const int h = (int)th & 1023, p = (int)tp & 1023;
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            if (m >= e.n) break;
+            const int x = field(e.h, m), y = field(e.p, m);
+            ok = ok && h != x && p != y;
+            if (h < x) ch += 1u << (4 * m);
+            if (p < y) cp += 1u << (4 * m);
+        }
+    }
+    // x - c core orbitals lie below a hole x with c holes below it (e's
+    // smaller ones among them); N - n + c orbitals below a particle with c
+    // particles below it (n: all holes of the product; e's larger ones are
+    // created first)
     const int ntot = cur.n + e.n;
 #pragma unroll 1
-    for (int m = 0; m < 2 * e.n; m++) {
-        const bool hole = m < e.n;
-        const int x = hole ? field(e.h, m) : field(e.p, 2 * e.n - 1 - m);
-        const u64 list = hole ? cur.h : cur.p;
-        u64 f = list;
-        int c = 0;
-#pragma unroll 1
-        for (int q = cur.n + (hole ? m : m - e.n); q > 0; q--, f >>= FB) {
-            const int y = (int)f & 1023;
-            c += y < x ? 1 : 0;
-            ok = ok && y != x;
-        }
-        const u64 with = insert_at(list, c, x);
-        if (hole) cur.h = with;
-        else cur.p = with;
-        parity += c + (hole ? x : s.nel - ntot);
+    for (int m = 0; m < e.n; m++, ch >>= 4, cp >>= 4) {
+        const int x = field(e.h, m), y = field(e.p, m), cx = (int)(ch & 15u) + m, cy = (int)(cp & 15u);
+        cur.h = insert_at(cur.h, cx, x);
+        cur.p = insert_at(cur.p, cy + m, y);
+        parity += x + cx + s.nel - ntot + cy;
     }
     cur.n = ntot;
     return ok;
@@ -575,26 +573,16 @@ __device__ __noinline__ double diag_rel(const SysDev &s, const Exc d)
 }
 
 // <bra|H|ket> for determinants differing by one or two spin-orbitals.
-// holes i<j are in ket only, particles a<b in bra only; gamma is the phase of
-// a+_a a+_b a_j a_i |ket> = gamma |bra>.  Computed in R, returned as double.
+// holes i<j are in ket only, particles a<b in bra only; par is the parity of
+// a+_a a+_b a_j a_i |ket>.  Computed in R, returned as double.
 template <typename R, bool GAS>
-__device__ __forceinline__ double h_offdiag(const SysDev &s, const Exc &ket, int nh, int i, int j, int a, int b)
+__device__ __forceinline__ double h_offdiag(const SysDev &s, const Exc &ket, bool dbl, int i, int j, int a, int b, int par)
 {
-    const bool dbl = GAS || nh == 2;
-    // i removed below j; i and j removed below b and a, b added above a
-    int par = i < a ? 1 : 0;
-    u64 at = (u64)i | ((u64)a << FB);
-    if (dbl) {
-        par += 1 + (j < a ? 1 : 0) + (i < b ? 1 : 0) + (j < b ? 1 : 0);
-        at |= ((u64)j << (2 * FB)) | ((u64)b << (3 * FB));
-    }
-#pragma unroll 1
-    for (int m = dbl ? 4 : 2; m > 0; m--, at >>= FB) par += occ_below_parity(s, ket, (int)at & 1023);
-    if (dbl) {
+    if (GAS || dbl) {
         R v1 = g2<R, GAS>(s, a, b, i, j);
         R v2 = g2<R, GAS>(s, a, b, j, i);
         R d = v1 - v2;
-        return (double)((par & 1) ? -d : d);
+        return (double)(par ? -d : d);
     }
     if ((i ^ a) & 1) return 0.0;
     const int A = a >> 1, I = i >> 1;
@@ -619,14 +607,19 @@ __device__ __forceinline__ double h_offdiag(const SysDev &s, const Exc &ket, int
         if (((a ^ o) & 1) == 0) t = t - eri_at<R>(s, A, Kk, Kk, I);
         acc = acc + t;
     }
-    return (double)((par & 1) ? -acc : acc);
+    return (double)(par ? -acc : acc);
 }
 
-// <HF|H|D> for D at level 1 or 2 (the gas has no level 1)
+// <HF|H|D> for D at level 1 or 2 (the gas has no level 1): i < j the
+// particles, a < b the holes.  Below a hole lie x - c core orbitals, below a
+// particle N - n + c; every hole lies below every particle.
 template <typename R, bool GAS>
 __device__ __forceinline__ double h_ref(const SysDev &s, const Exc &d)
 {
-    return h_offdiag<R, GAS>(s, d, d.n, field(d.p, 0), field(d.p, 1), field(d.h, 0), field(d.h, 1));
+    const int i = field(d.p, 0), j = field(d.p, 1), a = field(d.h, 0), b = field(d.h, 1);
+    // one hole and particle: N - 1 + a; two: N - 2 + (N - 1 - 1) + a + (b - 1)
+    const int par = GAS || d.n == 2 ? (a + b + 1) & 1 : (s.nel - 1 + a) & 1;
+    return h_offdiag<R, GAS>(s, d, d.n == 2, i, j, a, b, par);
 }
 
 // ---------------------------------------------------------------------------
@@ -765,40 +758,44 @@ __device__ __forceinline__ bool excite(const SysDev &s, const Exc &dj, const R4 
     return true;
 }
 
-// dj with the drawn excitation applied (its level is within the truncation):
-// each of i, j, a, b enters the list it is not in and leaves the one it is in,
-// those that leave first, so that no list ever grows past six fields
-__device__ __forceinline__ Exc excited(const SysDev &s, const Exc &dj, u64 code, bool dbl)
+// dj with the drawn excitation i j -> a b applied (its level is within the
+// truncation) and the parity of a+_a a+_b a_j a_i on dj.  Each orbital is
+// counted once in the list it belongs to, which gives both its parity and its
+// place in the new list; the orbitals that leave a list are taken out first,
+// so that no list ever grows past six fields.
+__device__ __forceinline__ Exc excited(const SysDev &s, const Exc &dj, bool dbl, int i, int j, int a, int b, int &parity)
 {
-    const u64 ij = code & 0xFFFFF, ab = (code >> 20) & 0xFFFFF;
-    u64 list = dj.h, h = 0;
-    u64 seq = ab | (ij << 20) | (ij << 40);   // holes: a, b filled, i, j emptied; particles: i, j, then a, b
-    int n = dj.n, nh = 0;
+    const int N = s.nel;
+    const bool ih = i < N, jh = dbl && j < N, ah = a < N, bh = dbl && b < N;   // the core's
+    int ci = 0, cj = 0, ca = 0, cb = 0;
+    u64 th = dj.h, tp = dj.p;
 #pragma unroll 1
-    for (int q = 0; q < 8; q++) {
-        if (q == 4) {
-            h = list;
-            nh = n;
-            list = dj.p;
-            n = dj.n;
-        }
-        if (q == 6) seq = ab;
-        const int v = (int)seq & 1023;
-        seq >>= FB;
-        if ((!dbl && (q & 1)) || (v < s.nel) != (q < 4)) continue;
-        const int c = fields_below(list, n, v);
-        if (c < n && field(list, c) == v) {
-            list = remove_at(list, c);
-            n--;
-        } else {
-            list = insert_at(list, c, v);
-            n++;
-        }
+    for (int m = dj.n; m > 0; m--, th >>= FB, tp >>= FB) {
+        const int h = (int)th & 1023, p = (int)tp & 1023;
+        ci += (ih ? h : p) < i ? 1 : 0;
+        cj += (jh ? h : p) < j ? 1 : 0;
+        ca += (ah ? h : p) < a ? 1 : 0;
+        cb += (bh ? h : p) < b ? 1 : 0;
     }
-    Exc e;
-    e.h = h;
-    e.p = list;
-    e.n = nh;
+    // occupied below x: x - c in the core, N - n + c above it; i and j are
+    // removed below what follows them, b added above a
+    int par = (ih ? i : N + dj.n) + ci + (ah ? a : N + dj.n) + ca + (i < a ? 1 : 0);
+    if (dbl)
+        par += (jh ? j : N + dj.n) + cj + (bh ? b : N + dj.n) + cb + 1 + (j < a ? 1 : 0) + (i < b ? 1 : 0) + (j < b ? 1 : 0);
+    parity = par & 1;
+    Exc e = dj;
+    // holes: a and b filled, i and j emptied
+    if (ah) e.h = remove_at(e.h, ca);
+    if (bh) e.h = remove_at(e.h, cb - (ah ? 1 : 0));
+    if (ih) e.h = insert_at(e.h, ci - (ah && a < i ? 1 : 0) - (bh && b < i ? 1 : 0), i);
+    if (jh) e.h = insert_at(e.h, cj - (ah && a < j ? 1 : 0) - (bh && b < j ? 1 : 0) + (ih ? 1 : 0), j);
+    // particles: i and j removed, a and b added
+    const bool ip = !ih, jp = dbl && !jh, ap = !ah, bp = dbl && !bh;
+    if (ip) e.p = remove_at(e.p, ci);
+    if (jp) e.p = remove_at(e.p, cj - (ip ? 1 : 0));
+    if (ap) e.p = insert_at(e.p, ca - (ip && i < a ? 1 : 0) - (jp && j < a ? 1 : 0), a);
+    if (bp) e.p = insert_at(e.p, cb - (ip && i < b ? 1 : 0) - (jp && j < b ? 1 : 0) + (ap ? 1 : 0), b);
+    e.n = dj.n + (ih ? 1 : 0) + (jh ? 1 : 0) - (ah ? 1 : 0) - (bh ? 1 : 0);
     return e;
 }
 

@@ -238,6 +238,10 @@ __device__ __forceinline__ u64 warp_reserve_u64(u64 *counter, u64 count)
     return base + incl - count;
 }
 
+// divisions that a step does once or seldom, out of line: each is some
+// hundred instructions
+static __device__ __noinline__ double div_rn(double a, double b) { return a / b; }
+
 // n_attempts = max(1, floor(|A| / A_thresh)) with multi-spawn, else 1
 static __device__ __noinline__ i64 attempts_of_thresh(double amp_abs, double a_thresh)
 {
@@ -275,14 +279,14 @@ __device__ __forceinline__ bool round_value(double x, u64 r, const RunParams &p,
 // smallest i in [1, n-1] with prefix[i] > x (excitor owning position x); the
 // bucket of x brackets the answer between the owners of its first position
 // and of the next bucket's first position
-__device__ __forceinline__ void pick_bracket(const int *bucket, int shift, i64 nbuckets, i64 n, u64 x, int &lo, int &hi)
+__device__ __forceinline__ void pick_bracket(const int *bucket, int shift, int nbuckets, int n, u64 x, int &lo, int &hi)
 {
-    const i64 b = (i64)(x >> shift);
+    const int b = (int)(x >> shift);
     lo = __ldg(&bucket[b]);
-    hi = b + 1 < nbuckets ? __ldg(&bucket[b + 1]) : (int)(n - 1);
+    hi = b + 1 < nbuckets ? __ldg(&bucket[b + 1]) : n - 1;
 }
 
-__device__ __forceinline__ int pick_index(const PickEntry *pk, const int *bucket, int shift, i64 nbuckets, i64 n, u64 x)
+__device__ __forceinline__ int pick_index(const PickEntry *pk, const int *bucket, int shift, int nbuckets, int n, u64 x)
 {
     int lo, hi;
     pick_bracket(bucket, shift, nbuckets, n, x, lo, hi);
@@ -296,7 +300,7 @@ __device__ __forceinline__ int pick_index(const PickEntry *pk, const int *bucket
 
 // two picks of one sample, their searches in step so that both loads of a
 // round are in flight together
-__device__ __forceinline__ void pick_two(const PickEntry *pk, const int *bucket, int shift, i64 nbuckets, i64 n, u64 x0,
+__device__ __forceinline__ void pick_two(const PickEntry *pk, const int *bucket, int shift, int nbuckets, int n, u64 x0,
                                          u64 x1, bool two, int &i0, int &i1)
 {
     int lo0, hi0, lo1 = 1, hi1 = 1;
@@ -423,9 +427,10 @@ __device__ __forceinline__ bool attempt_finish(const SysDev &s, const RunParams 
     const int i = (int)code & 1023, j = (int)(code >> 10) & 1023, a = (int)(code >> 20) & 1023,
               b = (int)(code >> 30) & 1023, gc = (int)(code >> 40) & 7;
     const bool dbl = GAS || gc == 0 || gc >= 3;
-    const Exc di = excited(s, dj, code, dbl);
+    int par;
+    const Exc di = excited(s, dj, dbl, i, j, a, b, par);
     // matrix element and 1/p_gen in the precision R; the value itself in FP64
-    double h = h_offdiag<R, GAS>(s, dj, dbl ? 2 : 1, i, j, a, b);
+    double h = h_offdiag<R, GAS>(s, dj, dbl, i, j, a, b, par);
     double x = ((p.tau * h) * inv_pgen_of<R>(s, gc)) * c_att;
     if (!sign_parity(s, di)) x = -x;
     i64 v;
@@ -532,7 +537,7 @@ __device__ __forceinline__ i64 find_key(const DirectView &d, u64 k)
 // onto listed determinants are added to them directly, the others appended to
 // the spawn buffer with one atomic per warp.
 __device__ __forceinline__ void rec_flush_once(RecStage &rs, int &rn, DevStep *st, const SpawnBuf &sp,
-                                               const DirectView &dv, i64 &ndirect, unsigned &err)
+                                               const DirectView &dv, unsigned &ndirect, unsigned &err)
 {
     const int lane = threadIdx.x & 31;
     const int take = rn >= 32 ? 32 : rn;
@@ -718,10 +723,10 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
         if (s <= smax && n_sel > 0 && !(p.fnc && s < 2)) {
             const double nex_d = (double)tw / FIX_ONE, n0_d = (double)an0 / FIX_ONE;
             double pr;
-            if (p.fnc) pr = s < smax ? ldexp(1.0, -(s - 1)) : ldexp(1.0, -lmax);
-            else pr = s < smax ? ldexp(1.0, -(s + 1)) : ldexp(1.0, -(lmax + 2));
+            const int k = p.fnc ? (s < smax ? s - 1 : lmax) : (s < smax ? s + 1 : lmax + 2);   // p(s) = 2^-k
+            pr = __longlong_as_double((i64)(1023 - k) << 52);
             if (s == 0) {
-                mag = n0_d / ((double)n_sel * pr);
+                mag = div_rn(n0_d, (double)n_sel * pr);
             } else {
                 double num = 1.0, den = 1.0, fact = 1.0;
                 for (int e = 0; e < s; e++) num = num * nex_d;
@@ -730,7 +735,7 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
                 den = den * (double)n_sel;
                 den = den * pr;
                 den = den * fact;
-                mag = num / den;
+                mag = div_rn(num, den);
                 mden = den;
             }
         }
@@ -740,7 +745,7 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
         // the magnitude of one attempt's coefficient, once per step
         const i64 na = attempts_of(mag, p);
         st->natt_s[s] = na;
-        st->cmag[s] = na > 1 ? mag / (double)na : mag;
+        st->cmag[s] = na > 1 ? div_rn(mag, (double)na) : mag;
     }
     if (threadIdx.x == 32) {
         if (runaway) atomicOr(&st->err, (unsigned)ERRB_RUNAWAY);
@@ -786,8 +791,10 @@ __device__ __forceinline__ void fill_run(int *t, i64 b0, i64 b1, int v)
     const int lane = threadIdx.x & 31;
     const bool lng = b1 - b0 > 8;
     if (!lng)
+#pragma unroll 1
         for (i64 b = b0; b < b1; b++) t[b] = v;
     unsigned m = __ballot_sync(FULLMASK, lng);
+#pragma unroll 1
     while (m) {
         const int src = __ffs(m) - 1;
         m &= m - 1;
@@ -813,6 +820,7 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
     const bool kb = sc.nkb > 0;
     const int bsh = sc.bshift, ksh = sc.kshift;
     // each warp scans its own chunk 32 entries at a time (no block barrier)
+#pragma unroll 1
     for (i64 base = lo; base < hi; base += 32) {
         i64 i = base + (threadIdx.x & 31);
         bool ok = i < hi;
@@ -861,7 +869,7 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
                 double x = td * coef;
                 if (!odd) x = -x;
                 if (!round_value(x, r.v[0], p, false, dv)) err |= ERRB_NUMERIC;
-                wa.catt[i] = na > 1 ? coef / (double)na : coef;
+                wa.catt[i] = na > 1 ? div_rn(coef, (double)na) : coef;
             } else {
                 // <HF|H|D_i> for the single-excitor clusters of the sampler
                 wa.href[i] = (d.n == 1 || d.n == 2) ? h_ref<R, GAS>(s, d) : 0.0;
@@ -972,6 +980,17 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
     __shared__ u64 smf[64];
     __shared__ i64 sm[32];
     __shared__ PhiloxStep ps;
+    // what the loop needs of the step: in shared memory, because the registers
+    // it leaves free decide the loop's speed
+    __shared__ struct {
+        DirectView dv;
+        i64 n_sel;
+        u64 nex;
+        double coef_hf, death_x;
+        RoundCut hf_cut;
+        int n, nbk, bshift;
+        bool n0_neg, n0_zero, hf_ok;
+    } ss;
     if (threadIdx.x < 8) {
         smag[threadIdx.x] = st->mag[threadIdx.x];
         scmag[threadIdx.x] = st->cmag[threadIdx.x];
@@ -979,28 +998,35 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         smden[threadIdx.x] = st->mden[threadIdx.x];
     }
     philox_step_init(ps, st->iter, p.seed, p.replica);
-    __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned below_me = (1u << lane) - 1u;
+    const PickEntry *pk = wa.picks;
+    if (threadIdx.x == 32) {
+        const i64 n0 = st->n0;
+        ss.dv = direct_view(L, wa, st);
+        ss.n_sel = st->n_sel;
+        ss.nex = (u64)st->nex;
+        ss.n = (int)st->n_occ;
+        ss.nbk = (int)st->nbuckets;
+        ss.bshift = st->bucket_shift;
+        ss.n0_neg = n0 < 0;
+        ss.n0_zero = n0 == 0;
+        ss.coef_hf = n0 < 0 ? -st->mag[0] : st->mag[0];
+        // every reference cluster's death value is the same (the reference's
+        // sign s_D is +1): its rounding once per block
+        ss.death_x = -(pk[0].tdeath * ss.coef_hf);
+        ss.hf_cut = RoundCut{0, 0, 0};
+        ss.hf_ok = !p.int_round || round_cut((u64)__double_as_longlong(ss.death_x), p.death_rs, ss.hf_cut);
+    }
+    __syncthreads();
     AttQueue &q = sw.q;
     RecStage &rb = sw.rs;
     int wn = 0, hn = 0, qn = 0, rn = 0;   // warp-uniform queue fills
-    const i64 n_sel = st->n_sel, n = st->n_occ, nex = st->nex, n0 = st->n0;
-    const int bshift = st->bucket_shift;
-    const i64 nbk = st->nbuckets;
     Fix128 es = {0, 0};
     unsigned err = 0;
-    unsigned n_valid = 0;  // valid clusters of this thread
+    unsigned n_valid = 0, ndirect = 0;   // valid clusters, records added directly (of this thread)
     double cl_att = 0.0;   // attempts of the clusters this thread buffers (exact below 2^53)
     i64 death_hf = 0;      // reference-cluster deaths, summed per block at the end
-    i64 ndirect = 0;       // records added directly to listed determinants
-    const DirectView dv = direct_view(L, wa, st);
-    const PickEntry *pk = wa.picks;
-    const double coef_hf = n0 < 0 ? -smag[0] : smag[0];
-    // every reference cluster's death value is the same: its rounding once per block
-    const double death_x = -(pk[0].tdeath * coef_hf);   // the reference's sign s_D is +1
-    RoundCut hf_cut = {0, 0, 0};
-    const bool hf_ok = !p.int_round || round_cut((u64)__double_as_longlong(death_x), p.death_rs, hf_cut);
+    const DirectView &dv = ss.dv;
     i64 g0 = (i64)vb * blockDim.x + 32 * wid;
     const i64 stride = (i64)vg * blockDim.x;
     for (;;) {
@@ -1008,7 +1034,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         // place (the loop is bound by instruction fetch when it grows):
         // finish what is waiting 32 at a time, else take 32 queued samples,
         // else draw 32 new ones; at the end whatever is left
-        const bool more = g0 < n_sel;
+        const bool more = g0 < ss.n_sel;
         const bool last = !more && wn + hn == 0;
         if (rn >= 32 || (last && qn == 0 && rn > 0)) {
             rec_flush_once(rb, rn, st, sp, dv, ndirect, err);
@@ -1032,7 +1058,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         u64 g = (u64)g0 + lane;
         bool valid = true;
         Exc dj = {0, 0, 0};
-        double coef = coef_hf;
+        double coef = ss.coef_hf;
         if (!sel) {
             const bool is_w = lane < tw;
             valid = is_w || lane < tw + th;
@@ -1069,18 +1095,18 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
                         const bool two = e + 1 < sz;
                         int ia, ib = 0;
                         if (!local) {
-                            pick_two(pk, wa.bucket, bshift, nbk, n, below(xa, (u64)nex), below(xb, (u64)nex), two, ia, ib);
+                            pick_two(pk, wa.bucket, ss.bshift, ss.nbk, ss.n, below(xa, ss.nex), below(xb, ss.nex), two, ia, ib);
                         } else {
                             // simulated distribution: a composite's later
                             // excitors come from the first one's processor
                             if (e == 0) {
-                                ia = pick_index(pk, wa.bucket, bshift, nbk, n, below(xa, (u64)nex));
+                                ia = pick_index(pk, wa.bucket, ss.bshift, ss.nbk, ss.n, below(xa, ss.nex));
                                 lq = __ldg(&wa.owner[ia]);
                                 nq = __ldg(&wa.nq[lq]);
                             } else {
-                                ia = (int)local_pick(wa, L.pop, n, st->lcs, st->nlc, lq, below(xa, (u64)nq));
+                                ia = (int)local_pick(wa, L.pop, ss.n, st->lcs, st->nlc, lq, below(xa, (u64)nq));
                             }
-                            if (two) ib = (int)local_pick(wa, L.pop, n, st->lcs, st->nlc, lq, below(xb, (u64)nq));
+                            if (two) ib = (int)local_pick(wa, L.pop, ss.n, st->lcs, st->nlc, lq, below(xb, (u64)nq));
                             if (ia < 0 || ib < 0) {   // tables inconsistent (cannot happen): a sticky error, not a guess
                                 valid = false;
                                 err |= ERRB_NUMERIC;
@@ -1105,16 +1131,16 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
                     }
                     if (dj.n > s.lmax + 2) valid = false;
                     if (valid) {
-                        if (n0 < 0 && ((sz - 1) & 1)) neg ^= 1;
+                        if (ss.n0_neg && ((sz - 1) & 1)) neg ^= 1;
                         double a = smag[sz];
                         if (local) {
                             // |A| = N_ex (N_q N_p)^(s-1) / (|t_HF|^(s-1) n_sel p(s) s!):
                             // selection within q times co-location N_p^-(s-1)
                             const double f = ((double)nq / FIX_ONE) * (double)p.nranks;
-                            double num = (double)nex / FIX_ONE;
+                            double num = (double)(i64)ss.nex / FIX_ONE;
     #pragma unroll 1
                             for (int e = 1; e < sz; e++) num = num * f;
-                            a = num / smden[sz];
+                            a = div_rn(num, smden[sz]);
                         }
                         const double amp = neg ? -a : a;
                         coef = (par & 1) ? -amp : amp;
@@ -1158,7 +1184,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
                 double catt = coef;
                 if (valid) {
                     // coef / natt: the same division, done once per size
-                    if (natt > 1) catt = local ? coef / (double)natt : (coef < 0.0 ? -scmag[sz] : scmag[sz]);
+                    if (natt > 1) catt = local ? div_rn(coef, (double)natt) : (coef < 0.0 ? -scmag[sz] : scmag[sz]);
                     if (natt > p.work_cap) {   // runaway: the attempts kernel will not run them
                         err |= ERRB_RUNAWAY;
                         natt = p.work_cap + 1;
@@ -1186,25 +1212,25 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         if (sel) {
             // the cluster size
             g0 += stride;
-            valid = (i64)g < n_sel;
+            valid = (i64)g < ss.n_sel;
             const u64 nr = ~r.v[0];
             const int lz = nr ? __clzll((long long)nr) : 64;
             const int sz = p.fnc ? 2 + min(lz, s.lmax) : min(lz, s.lmax + 2);
             const bool hf = valid && sz == 0;
             // a valid cluster's level is the sum of its excitors' levels: a
             // size beyond (l + 2) / (smallest level) contributes nothing
-            const bool work = valid && sz > 0 && nex != 0 && (sz < 2 || n0 != 0) && sz * s.lmin_exc <= s.lmax + 2;
+            const bool work = valid && sz > 0 && ss.nex != 0 && (sz < 2 || !ss.n0_zero) && sz * s.lmin_exc <= s.lmax + 2;
             const unsigned mh = __ballot_sync(FULLMASK, hf), mw = __ballot_sync(FULLMASK, work);
             if (hf) {
-                sw.hg[hn + __popc(mh & below_me)] = g;
-                i64 d = hf_cut.base + ((r.v[1] >> 11) < hf_cut.thr ? hf_cut.inc : 0);
-                bool in_range = hf_ok;
-                if (!p.int_round) in_range = round_value_fp(fabs(death_x), r.v[1], 0.0, &d);
+                sw.hg[hn + __popc(mh & ((1u << lane) - 1u))] = g;
+                i64 d = ss.hf_cut.base + ((r.v[1] >> 11) < ss.hf_cut.thr ? ss.hf_cut.inc : 0);
+                bool in_range = ss.hf_ok;
+                if (!p.int_round) in_range = round_value_fp(fabs(ss.death_x), r.v[1], 0.0, &d);
                 if (!in_range) err |= ERRB_NUMERIC;
-                death_hf += death_x < 0.0 ? -d : d;
+                death_hf += ss.death_x < 0.0 ? -d : d;
             }
             if (work) {
-                const int e = wn + __popc(mw & below_me);
+                const int e = wn + __popc(mw & ((1u << lane) - 1u));
                 sw.g[e] = g;
                 sw.v1[e] = r.v[1];
                 sw.v2[e] = r.v[2];
@@ -1224,7 +1250,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
     // the block's sums: E_num, reference deaths, valid clusters, direct records, attempts
     es = warp_fix(es);
     death_hf = warp_sum(death_hf);
-    const unsigned nv = __reduce_add_sync(FULLMASK, n_valid), nd = __reduce_add_sync(FULLMASK, (unsigned)ndirect);
+    const unsigned nv = __reduce_add_sync(FULLMASK, n_valid), nd = __reduce_add_sync(FULLMASK, ndirect);
     if (p.multispawn) cl_att = warp_sum(cl_att);
     if (lane == 0) {
         smf[2 * wid] = es.lo;
@@ -1287,7 +1313,7 @@ __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, D
     AttQueue &q = aq[threadIdx.x >> 5];
     RecStage &rb = rsb[threadIdx.x >> 5];
     int qn = 0, rn = 0;   // drawn attempts and staged records of this warp (warp-uniform)
-    i64 ndirect = 0;
+    unsigned ndirect = 0;
     const DirectView dv = direct_view(L, wa, st);
     // part 0: full non-composite attempts (owners: list entries); part 1:
     // attempts of the composite clusters queued by k_sample; part 2: what is
@@ -1341,8 +1367,8 @@ __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, D
         q_push(q, qn, ok, dj, ca, r3, code);
         t0 += 32;
     }
-    ndirect = block_sum(ndirect, sm);
-    if (threadIdx.x == 0 && ndirect) atomicAdd((unsigned long long *)&st->n_direct, (unsigned long long)ndirect);
+    const i64 direct = block_sum((i64)ndirect, sm);
+    if (threadIdx.x == 0 && direct) atomicAdd((unsigned long long *)&st->n_direct, (unsigned long long)direct);
     if (err) atomicOr(&st->err, err);
 }
 
