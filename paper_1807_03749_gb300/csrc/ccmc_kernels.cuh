@@ -741,6 +741,17 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
         }
         st->mag[s] = mag;
         st->mden[s] = mden;
+        if (s == 0) {
+            // every reference cluster has this coefficient and death value
+            // (the reference's sign s_D is +1): its rounding once per step
+            const double coef = n0 < 0 ? -mag : mag;
+            const double x = -((p.tau * (0.0 - st->shift)) * coef);
+            RoundCut cut = {0, 0, 0};
+            st->hf_ok = !p.int_round || round_cut((u64)__double_as_longlong(x), p.death_rs, cut);
+            st->hf_coef = coef;
+            st->hf_death = x;
+            st->hf_cut = cut;
+        }
         // every cluster of size s has |A| = mag[s]: its attempt count and
         // the magnitude of one attempt's coefficient, once per step
         const i64 na = attempts_of(mag, p);
@@ -871,8 +882,8 @@ __device__ __forceinline__ void d_scan_final(const SysDev &s, const ListView &L,
                 if (!round_value(x, r.v[0], p, false, dv)) err |= ERRB_NUMERIC;
                 wa.catt[i] = na > 1 ? div_rn(coef, (double)na) : coef;
             } else {
-                // <HF|H|D_i> for the single-excitor clusters of the sampler
-                wa.href[i] = (d.n == 1 || d.n == 2) ? h_ref<R, GAS>(s, d) : 0.0;
+                // <HF|H|D_i> for the single-excitor clusters of the sampler (read at these levels only)
+                if (d.n == 1 || d.n == 2) wa.href[i] = h_ref<R, GAS>(s, d);
             }
             wa.picks[i] = pe;
             wa.death[i] = dv;
@@ -1010,12 +1021,10 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         ss.bshift = st->bucket_shift;
         ss.n0_neg = n0 < 0;
         ss.n0_zero = n0 == 0;
-        ss.coef_hf = n0 < 0 ? -st->mag[0] : st->mag[0];
-        // every reference cluster's death value is the same (the reference's
-        // sign s_D is +1): its rounding once per block
-        ss.death_x = -(pk[0].tdeath * ss.coef_hf);
-        ss.hf_cut = RoundCut{0, 0, 0};
-        ss.hf_ok = !p.int_round || round_cut((u64)__double_as_longlong(ss.death_x), p.death_rs, ss.hf_cut);
+        ss.coef_hf = st->hf_coef;
+        ss.death_x = st->hf_death;
+        ss.hf_cut = st->hf_cut;
+        ss.hf_ok = st->hf_ok != 0;
     }
     __syncthreads();
     AttQueue &q = sw.q;
@@ -2114,6 +2123,24 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *
     }
 }
 
+// Launches a grid, cooperatively (all blocks resident) if its blocks wait for
+// one another.
+template <typename... P, typename... Q>
+cudaError_t launch_blocks(void (*k)(P...), dim3 grid, bool cooperative, int threads, size_t smem, cudaStream_t sm, Q... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = sm;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cooperative ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // Launches a kernel whose blocks wait for their replica's other blocks: as
 // many per replica as fit on the GPU with every replica's (at most want).
 // One block per replica waits for nobody.
@@ -2129,17 +2156,7 @@ cudaError_t launch_team(void (*k)(P...), int want, int nrep, int threads, size_t
     int g = per * sms / nrep;
     if (g > want) g = want;
     if (g < 1) g = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g, nrep);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = sm;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = g > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+    return launch_blocks(k, dim3(g, nrep), g > 1, threads, smem, sm, args...);
 }
 
 // ---------------------------------------------------------------------------

@@ -95,6 +95,10 @@ struct DevStep {
     // composite's amplitude depends on its processor's population), and the
     // chunks of the per-processor position table
     double mden[8];
+    // bare-reference clusters: coefficient, death value and its rounding
+    double hf_coef, hf_death;
+    RoundCut hf_cut;
+    int hf_ok;
     int lcs;            // chunks cover 2^lcs list entries
     int pad2;
     i64 nlc;            // chunks in use
@@ -134,7 +138,7 @@ constexpr u64 PICK_NEG = 1ULL << 63;   // negative population
 // Per-step work arrays over the list and the merge.
 struct WorkArrays {
     PickEntry *picks; // one row per list entry
-    double *href;     // <HF|H|D_i> (levels 1-2, else 0; not with full non-composite sampling)
+    double *href;     // <HF|H|D_i> (levels 1-2 only; not with full non-composite sampling)
     int *bucket;      // owner of the first position of each selection bucket
     int bucket_bits;  // log2 of the bucket capacity
     i64 *att_end;     // inclusive prefix of full non-composite attempts

@@ -149,6 +149,10 @@ namespace {
 constexpr size_t NOALLOC_MAX = (size_t)1 << 16;   // records per call
 constexpr int NOALLOC_GRID = (int)(NOALLOC_MAX / (2 * SORT_THREADS));   // blocks of the largest call
 
+struct NoAllocResult {
+    i64 n_keys;   // -1: a wait ran out
+};
+
 struct NoAllocScratch {
     u64 key[2][NOALLOC_MAX];
     i64 pop[2][NOALLOC_MAX];
@@ -162,10 +166,29 @@ __device__ __align__(256) NoAllocScratch g_noalloc;
 
 std::mutex g_noalloc_mutex;
 NoAllocScratch *g_noalloc_ptr[256];
+NoAllocResult *g_noalloc_out[256];   // page-locked, mapped: the kernel writes a call's result there
+
+// The whole call (its blocks wait for each other: a cooperative launch when
+// there are several).
+__global__ void __launch_bounds__(SORT_THREADS, 1) k_noalloc(const u64 *keys_in, const i64 *pops_in, i64 n, int key_bits,
+                                                             u64 *keys_out, i64 *pops_out, NoAllocScratch *N,
+                                                             NoAllocResult *res)
+{
+    SortSmem &S = *(SortSmem *)dyn_smem;
+    __shared__ i64 sm[64];
+    const Team t = {(int)blockIdx.x, (int)gridDim.x};
+    u64 *key[2] = {N->key[0], N->key[1]};
+    i64 *pop[2] = {N->pop[0], N->pop[1]};
+    if (!team_sort(keys_in, pops_in, key, pop, n, key_bits, SORT_DIGIT_BITS, N->hist, N->bar, t, &N->st, S)) return;
+    const int src = ((key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS) & 1;
+    const i64 m = team_reduce(key[src], pop[src], n, keys_out, pops_out, N->part, N->bar, t, &N->st, sm);
+    if (t.id == 0 && threadIdx.x == 0) res->n_keys = m;
+}
 
 // Device address of the scratch on the current device, looked up once per
-// device (host code cannot use the symbol itself as a device address).
-cudaError_t noalloc_scratch(NoAllocScratch **out)
+// device (host code cannot use the symbol itself as a device address), with
+// the kernel's shared memory size set and a page-locked word for the result.
+cudaError_t noalloc_scratch(NoAllocScratch **out, NoAllocResult **res)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -176,26 +199,17 @@ cudaError_t noalloc_scratch(NoAllocScratch **out)
         void *p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc);
         if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(k_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+        if (e != cudaSuccess) return e;
+        if (!g_noalloc_out[dev]) {
+            e = cudaHostAlloc((void **)&g_noalloc_out[dev], sizeof(NoAllocResult), cudaHostAllocMapped);
+            if (e != cudaSuccess) return e;
+        }
         g_noalloc_ptr[dev] = (NoAllocScratch *)p;
     }
     *out = g_noalloc_ptr[dev];
+    *res = g_noalloc_out[dev];
     return cudaSuccess;
-}
-
-// The whole call (its blocks wait for each other: a cooperative launch when
-// there are several).
-__global__ void __launch_bounds__(SORT_THREADS, 1) k_noalloc(const u64 *keys_in, const i64 *pops_in, i64 n, int key_bits,
-                                                             u64 *keys_out, i64 *pops_out, NoAllocScratch *N)
-{
-    SortSmem &S = *(SortSmem *)dyn_smem;
-    __shared__ i64 sm[64];
-    const Team t = {(int)blockIdx.x, (int)gridDim.x};
-    u64 *key[2] = {N->key[0], N->key[1]};
-    i64 *pop[2] = {N->pop[0], N->pop[1]};
-    if (!team_sort(keys_in, pops_in, key, pop, n, key_bits, SORT_DIGIT_BITS, N->hist, N->bar, t, &N->st, S)) return;
-    const int src = ((key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS) & 1;
-    const i64 m = team_reduce(key[src], pop[src], n, keys_out, pops_out, N->part, N->bar, t, &N->st, sm);
-    if (t.id == 0 && threadIdx.x == 0) N->st.n_keys = m;
 }
 
 }  // namespace
@@ -214,19 +228,19 @@ extern "C" ccmc_status ccmc_reduce_records_noalloc(const uint64_t *keys_in, cons
     if (!keys_in || !pops_in || !keys_out || !pops_out) return CCMC_ERR_ARG;
     cudaStream_t sm = (cudaStream_t)cuda_stream;
     NoAllocScratch *S = nullptr;
-    if (noalloc_scratch(&S) != cudaSuccess) return CCMC_ERR_CUDA;
-    const int blocks = (int)sort_blocks((i64)n);
-    if (launch_team(k_noalloc, blocks, 1, SORT_THREADS, sizeof(SortSmem), sm, (const u64 *)keys_in, (const i64 *)pops_in,
-                    (i64)n, (int)key_bits, (u64 *)keys_out, (i64 *)pops_out, S) != cudaSuccess)
+    NoAllocResult *res = nullptr;
+    if (noalloc_scratch(&S, &res) != cudaSuccess) return CCMC_ERR_CUDA;
+    res->n_keys = -1;
+    if (launch_blocks(k_noalloc, dim3((unsigned)sort_blocks((i64)n)), n > SORT_TILE, SORT_THREADS, sizeof(SortSmem), sm,
+                      (const u64 *)keys_in, (const i64 *)pops_in, (i64)n, (int)key_bits, (u64 *)keys_out, (i64 *)pops_out,
+                      S, res) != cudaSuccess)
         return CCMC_ERR_CUDA;
-    DevStep st;
-    if (cudaMemcpyAsync(&st, &S->st, sizeof(st), cudaMemcpyDeviceToHost, sm) != cudaSuccess) return CCMC_ERR_CUDA;
     if (cudaStreamSynchronize(sm) != cudaSuccess) return CCMC_ERR_CUDA;
-    if (st.err || st.n_keys < 0) {   // a wait ran out: the next call starts clean
+    const i64 m = *(volatile i64 *)&res->n_keys;
+    if (m < 0) {   // a wait ran out: the next call starts clean
         cudaMemsetAsync(S->bar, 0, sizeof(S->bar) + sizeof(S->st), sm);
         return CCMC_ERR_TIMEOUT;
     }
-    const i64 m = st.n_keys;
     *n_out = (size_t)m;
     return CCMC_OK;
 }
