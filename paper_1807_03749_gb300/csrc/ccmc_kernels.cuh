@@ -205,6 +205,11 @@ __device__ __forceinline__ bool team_sync(unsigned *bar, Team t, DevStep *st)
 // sum of the partials v[stride b] of the blocks before this one, and of all
 __device__ __forceinline__ void team_prefix(const i64 *v, int stride, Team t, i64 *sm, i64 &before, i64 &total)
 {
+    if (t.n == 1) {
+        before = 0;
+        total = __ldcg(v);
+        return;
+    }
     i64 a = 0, b = 0;
     for (int q = threadIdx.x; q < t.n; q += blockDim.x) {
         const i64 x = __ldcg(&v[(size_t)stride * q]);
@@ -695,10 +700,9 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
     // hundreds of its entries
     i64 nb_want = n_sel >> 5 < (1LL << 18) ? n_sel >> 5 : (1LL << 18);
     if (nb_want < 2 * n_occ) nb_want = 2 * n_occ;
-    int bb = 4;
-    while (bb < wa.bucket_bits && (1LL << bb) < nb_want) bb++;
-    r.bshift = 0;
-    while (r.bshift < 62 && ((u64)tw >> (r.bshift + bb)) != 0) r.bshift++;
+    int bb = nb_want > 16 ? 64 - __clzll(nb_want - 1) : 4;   // smallest with 2^bb >= nb_want
+    bb = bb < wa.bucket_bits ? bb : wa.bucket_bits;
+    r.bshift = max(0, 64 - __clzll(tw) - bb);                 // smallest with tw < 2^(bshift + bb)
     // key buckets for direct accumulation: about two per list entry over the
     // list's key range (up to eight for a short list: the keys cluster),
     // within the table's capacity.  Direct accumulation pays once the step
@@ -712,6 +716,7 @@ __device__ __forceinline__ ScanScalars d_scan_top(const ListView &L, DevStep *st
         i64 want = 8 * n_occ < (1LL << 18) ? 8 * n_occ : (1LL << 18);
         if (want < 2 * n_occ) want = 2 * n_occ;
         if (want > (1LL << wa.kbucket_bits)) want = 1LL << wa.kbucket_bits;
+        r.kshift = max(0, __clzll(want) - __clzll((i64)kmax) - 1);   // at most two below the smallest that fits
         while (r.kshift < 63 && (i64)(kmax >> r.kshift) + 1 > want) r.kshift++;
         r.nkb = (i64)(kmax >> r.kshift) + 1;
     }
@@ -1558,19 +1563,51 @@ __device__ __forceinline__ bool team_sort(const u64 *k0, const i64 *v0, u64 *con
         if (!team_sync(bar, t, st)) return false;
         {
             // offset of this block's run of each digit: the digits before, and
-            // the same digit's runs of the blocks before
-            const int d = threadIdx.x & (nd - 1), parts = SORT_THREADS / nd, part = threadIdx.x / nd;
-            unsigned before = 0, all = 0;
-#pragma unroll 8
-            for (int b = part; b < t.n; b += parts) {
-                const unsigned h = __ldcg(&hist[(size_t)b * nd + d]);
-                all += h;
-                if (b < t.id) before += h;
-            }
+            // the same digit's runs of the blocks before.  Every block reads
+            // all counts: of many blocks four digits a load (304 blocks' rows
+            // were 38 rounds of latency a pass: 9e5 records 148 -> 104 us), of
+            // a few one digit a load (ten blocks: 33 us, 38 with four; scanning
+            // the columns by blocks first was slower for all)
             for (int q = threadIdx.x; q < nd; q += SORT_THREADS) S.off[q] = S.all[q] = 0;
             __syncthreads();
-            atomicAdd(&S.off[d], before);
-            atomicAdd(&S.all[d], all);
+            const bool four = nd >= 4 && t.n > 32;
+            const int per = four ? nd / 4 : nd, parts = SORT_THREADS / per, part = threadIdx.x / per;
+            const int d = (threadIdx.x - part * per) * (four ? 4 : 1);
+            if (four) {
+                uint4 before = make_uint4(0, 0, 0, 0), all = before;
+#pragma unroll 8
+                for (int b = part; b < t.n; b += parts) {
+                    const uint4 h = __ldcg((const uint4 *)&hist[(size_t)b * nd + d]);
+                    all.x += h.x;
+                    all.y += h.y;
+                    all.z += h.z;
+                    all.w += h.w;
+                    if (b < t.id) {
+                        before.x += h.x;
+                        before.y += h.y;
+                        before.z += h.z;
+                        before.w += h.w;
+                    }
+                }
+                atomicAdd(&S.off[d], before.x);
+                atomicAdd(&S.off[d + 1], before.y);
+                atomicAdd(&S.off[d + 2], before.z);
+                atomicAdd(&S.off[d + 3], before.w);
+                atomicAdd(&S.all[d], all.x);
+                atomicAdd(&S.all[d + 1], all.y);
+                atomicAdd(&S.all[d + 2], all.z);
+                atomicAdd(&S.all[d + 3], all.w);
+            } else {
+                unsigned before = 0, all = 0;
+#pragma unroll 8
+                for (int b = part; b < t.n; b += parts) {
+                    const unsigned h = __ldcg(&hist[(size_t)b * nd + d]);
+                    all += h;
+                    if (b < t.id) before += h;
+                }
+                atomicAdd(&S.off[d], before);
+                atomicAdd(&S.all[d], all);
+            }
             __syncthreads();
             const unsigned v = threadIdx.x < nd ? S.all[threadIdx.x] : 0u;
             unsigned sum;

@@ -156,7 +156,7 @@ struct NoAllocResult {
 struct NoAllocScratch {
     u64 key[2][NOALLOC_MAX];
     i64 pop[2][NOALLOC_MAX];
-    unsigned hist[(1 << SORT_DIGIT_BITS) * NOALLOC_GRID];
+    __align__(16) unsigned hist[(1 << SORT_DIGIT_BITS) * NOALLOC_GRID];
     i64 part[4 * NOALLOC_GRID];
     unsigned bar[2];
     DevStep st;
