@@ -199,9 +199,11 @@ def read_profile(workload: str) -> dict:
     return out
 
 
+# (one kernel sorts, reduces, merges and writes the record: under ncu its
+# figures stand under the merge; older captures have a kernel per phase)
 PHASE_OF_KERNEL = [("k_scan", "scan"), ("k_local", "scan"), ("k_sample", "sample"), ("k_attempts", "attempts"), ("k_sort", "sort"),
                    ("k_seg", "reduce"), ("k_part_scan", "reduce"), ("k_merge", "merge"), ("k_keep", "merge"),
-                   ("k_scatter", "merge"), ("k_finalize", "finalize")]
+                   ("k_scatter", "merge"), ("k_annihilate", "merge"), ("k_finalize", "finalize")]
 UNIT_OF_PHASE = {"scan": "entry", "sample": "sample", "attempts": "attempt", "sort": "record", "reduce": "record",
                  "merge": "entry", "finalize": "step"}
 
@@ -318,7 +320,8 @@ def roofline_objects(name: str, pms: dict, nprof: int, precs_by_ctx: list, nw_by
     ph = ["scan", "sort", "reduce", "merge"]
     ta = sum(per.get(q, 0.0) for q in ph) * 1e-3
     ba = sum(alg(q) for q in ph)
-    tr = [traffic(q) for q in ph]
+    # sort and reduction have no kernel of their own in a capture of the fused annihilation
+    tr = [traffic(q) for q in ph if q in prof or not str(prof.get("merge", {}).get("kernel", "")).startswith("k_annihilate")]
     ann = {"bound": "hbm", "phases": ph, "achieved": ba / ta / 1e9 if ta else None, "peak": hbm, "unit": "GB/s",
            "frac": ba / ta / 1e9 / hbm if ta else None, "algorithmic_bytes_per_step": ba,
            "traffic": sum(tr) if all(x is not None for x in tr) else None, "peak_source": src}

@@ -164,7 +164,7 @@ __device__ __forceinline__ void chunk_of(Team t, i64 n, i64 &lo, i64 &hi)
     hi = lo + c < n ? lo + c : n;
 }
 
-constexpr unsigned TEAM_SPINS = 1u << 21;   // polls of a wait: a second or so
+constexpr unsigned TEAM_SPINS = 1u << 24;   // polls of a wait: some ten seconds
 
 // All threads of the team's blocks call.  bar[0] counts arrivals, bar[1] the
 // barrier's generation; both are left as found plus one generation.  False if
