@@ -163,10 +163,10 @@ def algorithmic_bytes(phase: str, recs: list, nw: int, lmax: int = 2, fnc: bool 
         if phase == "scan":
             b = n * 16
         elif phase == "sample":
-            # buffered clusters (multi-spawn, or the original sampler on a
-            # generic Hamiltonian): their records are the attempt kernel's
-            b = r["n_sel"] * sbar * be + (ncl * bc if ncl else sp * 16)
+            # multi-spawn buffers its clusters: their records are the attempt kernel's
+            b = r["n_sel"] * sbar * be + (ncl * bc if multispawn else sp * 16)
         elif phase == "attempts":
+            ncl = ncl if multispawn else 0
             b = r["n_visit"] * be + ncl * bc + (sp * 16 if (ncl or r["n_visit"]) else 0)
         elif phase == "sort":
             b = (sp - r.get("n_direct", 0)) * 32

@@ -31,7 +31,9 @@
  *   - Every function returns a ccmc_status; nothing traps or aborts.  Errors
  *     found by kernels (buffer overflow, numeric overflow, a runaway
  *     population) are recorded in a device status word and reported by the
- *     next synchronising call.  No kernel waits on another.
+ *     next synchronising call.  No kernel waits on another; the blocks of one
+ *     cooperative launch wait for each other with a limit
+ *     (CCMC_ERR_TIMEOUT).
  *   - One context per CUDA stream; calls on one context are not thread-safe.
  *   - Host pointers are read during the call only (the library copies what it
  *     keeps).  Device memory is owned by the context and released by ccmc_free.
