@@ -145,7 +145,7 @@ __device__ __forceinline__ Fix128 block_fix(Fix128 v, u64 *sm)
 // are handled by one block (its barriers are the block's own) and a long list
 // by all of them, without a launch per phase: 12 to 24 launches of a step,
 // most with nothing to do on small systems, became two (a step of the
-// 38-orbital gas, 289 excitors: 89 -> 50 us; of the 114-orbital gas with 90,000:
+// 38-orbital gas, 289 excitors: 85 -> 44 us; of the 114-orbital gas with 90,000:
 // 318 -> 307 us; of the 1.1e7-excitor molecule: the same).  A barrier costs 2 to
 // 4 us with tens to hundreds of blocks, less than a launch and its ramp.  The blocks of a team
 // wait for each other, so a launch with more than one block per replica is
@@ -977,13 +977,14 @@ struct SampWarp {
 // spawning attempt each (or the append to the multi-spawn buffer).  Both
 // kinds share the attempt's code, so that it is fetched once.
 //
-// What bounds it: instruction issue (55 % of the slots, 24 of 32 lanes; the
-// two Philox draws of a sample are a third of it).  With every size handled
-// where it was drawn and bit-string determinants, 15.7 (gas) and 8.7
-// (molecule) lanes of 32 were active, 320 bytes of local memory per thread.
-// 1.5e8 samples of the 162-orbital FP32 gas: 18.7 -> 7.6 ms; 2e7 of the
-// molecule: 5.5 ms (with the attempts of its clusters, which then went through
-// a buffer) -> 3.6 ms; 64 gas replicas: 3.2 -> 1.65 ms.
+// What bounds it: instruction issue on the gas (57 % of the slots, 25 of 32
+// lanes; the two Philox draws of a sample are a third of it), instruction
+// fetch on the molecule.  With every size handled where it was drawn and
+// bit-string determinants, 15.7 (gas) and 8.7 (molecule) lanes of 32 were
+// active, with 320 bytes of local memory per thread.  1.5e8 samples of the
+// 162-orbital FP32 gas: 18.7 -> 6.8 ms; 2e7 of the molecule: 5.5 ms (with the
+// attempts of its clusters, which then went through a buffer) -> 3.2 ms; 64 gas
+// replicas: 3.2 -> 1.45 ms.
 // DIST: the simulated distribution's restricted composite draw is compiled
 // in (a separate instantiation keeps it out of the plain sampler's loop)
 template <typename R, bool GAS, bool DIST>

