@@ -33,7 +33,7 @@
  *     population) are recorded in a device status word and reported by the
  *     next synchronising call.  No kernel waits on another; the blocks of one
  *     cooperative launch wait for each other with a limit
- *     (CCMC_ERR_TIMEOUT).
+ *     (CCMC_ERR_TIMEOUT, see ccmc_wait_limit).
  *   - One context per CUDA stream; calls on one context are not thread-safe.
  *   - Host pointers are read during the call only (the library copies what it
  *     keeps).  Device memory is owned by the context and released by ccmc_free.
@@ -220,6 +220,14 @@ ccmc_status ccmc_get_death(ccmc_ctx *ctx, int64_t *death, size_t cap, size_t *n)
  * shift boundary (checkpoint state besides the list). */
 ccmc_status ccmc_set_state(ccmc_ctx *ctx, uint64_t iter, double shift, int32_t vary, double nprev);
 ccmc_status ccmc_get_state(ccmc_ctx *ctx, uint64_t *iter, double *shift, int32_t *vary, double *nprev);
+
+/* Polls (some half a microsecond each) after which a wait between the blocks
+ * of a step gives up; 0: the default, some ten seconds.  A wait that ran out
+ * leaves the step unfinished: the context's kernels then do nothing and every
+ * call that reports errors returns CCMC_ERR_TIMEOUT until ccmc_set_list or
+ * ccmc_load gives the context a new list.  (ccmc_set_state sets the iteration
+ * that the list belongs to.)  Waits for work in flight. */
+ccmc_status ccmc_wait_limit(ccmc_ctx *ctx, uint32_t polls);
 
 /* Checkpoint to / restore from a file (state + list).  Because every random
  * number is a function of (seed, replica, iteration, index), a restored run

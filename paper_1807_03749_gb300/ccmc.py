@@ -8,8 +8,8 @@ from __future__ import annotations
 
 import ctypes
 import os
-from ctypes import (CFUNCTYPE, POINTER, c_char_p, c_double, c_int, c_int32, c_int64, c_size_t, c_uint64,
-                    c_void_p)
+from ctypes import (CFUNCTYPE, POINTER, c_char_p, c_double, c_int, c_int32, c_int64, c_size_t, c_uint32,
+                    c_uint64, c_void_p)
 
 import numpy as np
 
@@ -69,7 +69,7 @@ EXPORTS = [
     "ccmc_get_list", "ccmc_set_list", "ccmc_get_spawned", "ccmc_get_death", "ccmc_set_state", "ccmc_get_state",
     "ccmc_save", "ccmc_load", "ccmc_sync", "ccmc_last_error", "ccmc_free", "ccmc_profile", "ccmc_phase_times",
     "ccmc_reduce_records_noalloc", "ccmc_batch_create", "ccmc_step_batched", "ccmc_batch_info", "ccmc_batch_free",
-    "ccmc_batch_profile", "ccmc_batch_phase_times", "ccmc_colocation",
+    "ccmc_batch_profile", "ccmc_batch_phase_times", "ccmc_colocation", "ccmc_wait_limit",
 ]
 
 PHASES = ["scan", "sample", "attempts", "sort", "reduce", "merge", "finalize"]
@@ -97,6 +97,7 @@ def load(path: str | None = None):
         "ccmc_get_death": (c_int, [vp, i64p, c_size_t, POINTER(c_size_t)]),
         "ccmc_set_state": (c_int, [vp, c_uint64, c_double, c_int32, c_double]),
         "ccmc_get_state": (c_int, [vp, u64p, dp, i32p, dp]),
+        "ccmc_wait_limit": (c_int, [vp, c_uint32]),
         "ccmc_save": (c_int, [vp, c_char_p]),
         "ccmc_load": (c_int, [vp, c_char_p]),
         "ccmc_sync": (c_int, [vp]),
@@ -297,6 +298,10 @@ class Context:
         self._check(self._lib.ccmc_get_state(self._h, ctypes.byref(it), ctypes.byref(sh), ctypes.byref(vy),
                                              ctypes.byref(npv)))
         return int(it.value), sh.value, bool(vy.value), npv.value
+
+    def wait_limit(self, polls: int = 0):
+        """Polls after which a wait between a step's blocks gives up (0: the default)."""
+        self._check(self._lib.ccmc_wait_limit(self._h, polls))
 
     def save(self, path: str):
         self._check(self._lib.ccmc_save(self._h, os.fsencode(path)))

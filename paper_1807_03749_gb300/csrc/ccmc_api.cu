@@ -220,7 +220,7 @@ struct ccmc_ctx {
     double nprev = 0.0;
     u64 records_read = 0;
     bool stepped = false;
-    bool timed_out = false;       // a device wait gave up: the barriers are reset with the next list
+    unsigned wait_limit = 0;      // see DevStep
     // pinned staging
     DevStep *h_st = nullptr;
     double *h_shift = nullptr;
@@ -276,14 +276,12 @@ cudaError_t wait_batch(ccmc_ctx *ctx)
 
 ccmc_status status_from_bits(ccmc_ctx *ctx, unsigned bits)
 {
+    // the step was not finished, whatever else it found
+    if (bits & ERRB_TIMEOUT) return fail(ctx, CCMC_ERR_TIMEOUT, "a wait between the blocks of a step gave up");
     // a runaway population overflows the buffers too; it is the cause to report
     if (bits & ERRB_RUNAWAY)
         return fail(ctx, CCMC_ERR_RUNAWAY, "population runaway: a step needed more than max(64 x target_pop, 2^24) "
                                            "samples or spawning attempts");
-    if (bits & ERRB_TIMEOUT) {
-        ctx->timed_out = true;
-        return fail(ctx, CCMC_ERR_TIMEOUT, "a wait between the blocks of a step gave up");
-    }
     if (bits & ERRB_SPAWN_OVERFLOW) return fail(ctx, CCMC_ERR_SPAWN_OVERFLOW, "spawned particles exceeded spawn_capacity");
     if (bits & ERRB_CLUSTER_OVERFLOW) return fail(ctx, CCMC_ERR_SPAWN_OVERFLOW, "multi-spawn clusters exceeded capacity");
     if (bits & ERRB_LIST_OVERFLOW) return fail(ctx, CCMC_ERR_LIST_OVERFLOW, "occupied excitors exceeded list_capacity");
@@ -755,7 +753,6 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
         }
     }
 
-    ctx->timed_out = true;   // the barriers start at zero with the first list
     // initial state: d0_init on HF
     ctx->iter = 0;
     ctx->shift = 0.0;
@@ -836,9 +833,12 @@ ccmc_status ccmc_set_list(ccmc_ctx *ctx, const uint64_t *bits, const int64_t *po
     st.shift = ctx->shift;
     st.n_occ = (i64)n;
     st.cur = ctx->sc.cur;
+    st.wait_limit = ctx->wait_limit;
+    // the barriers with it: the error word that is overwritten here may tell,
+    // unread, of a wait that ran out and left them with a count
+    CK(cudaMemsetAsync(ctx->sc.wa.bar, 0, 64 * sizeof(unsigned), ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     CK(cudaMemcpy(ctx->sc.st, &st, sizeof(DevStep), cudaMemcpyHostToDevice));
-    if (ctx->timed_out) CK(cudaMemset(ctx->sc.wa.bar, 0, 64 * sizeof(unsigned)));
-    ctx->timed_out = false;
     ctx->stepped = false;
     return CCMC_OK;
 }
@@ -1091,6 +1091,16 @@ ccmc_status ccmc_set_state(ccmc_ctx *ctx, uint64_t iter, double shift, int32_t v
     CK(cudaStreamSynchronize(ctx->stream));
     CK(cudaMemcpy(&ctx->sc.st->iter, &iter, sizeof(u64), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(&ctx->sc.st->shift, &shift, sizeof(double), cudaMemcpyHostToDevice));
+    return CCMC_OK;
+}
+
+ccmc_status ccmc_wait_limit(ccmc_ctx *ctx, uint32_t polls)
+{
+    if (!ctx) return CCMC_ERR_ARG;
+    CK(wait_batch(ctx));
+    CK(cudaStreamSynchronize(ctx->stream));
+    ctx->wait_limit = polls;
+    CK(cudaMemcpy(&ctx->sc.st->wait_limit, &polls, sizeof(polls), cudaMemcpyHostToDevice));
     return CCMC_OK;
 }
 

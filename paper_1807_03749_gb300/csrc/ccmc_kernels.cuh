@@ -150,6 +150,14 @@ __device__ __forceinline__ Fix128 block_fix(Fix128 v, u64 *sm)
 // 4 us with tens to hundreds of blocks, less than a launch and its ramp.  The blocks of a team
 // wait for each other, so a launch with more than one block per replica is
 // cooperative (all resident), and every wait has a limit.
+//
+// A wait that runs out ends the step and every later one: the block sets
+// ERRB_TIMEOUT and returns, and a kernel that finds the bit set at its start
+// returns too, because the barrier words and the step's tables are then
+// unfinished.  Within the launch no barrier opens too soon: a block gives up
+// only after it has arrived, so the barrier it left still counts it, and the
+// next one lacks it and never opens.  The next list (ccmc_set_list) clears the
+// bit and the barrier words.
 // ---------------------------------------------------------------------------
 
 struct Team {
@@ -168,7 +176,8 @@ constexpr unsigned TEAM_SPINS = 1u << 24;   // polls of a wait: some ten seconds
 
 // All threads of the team's blocks call.  bar[0] counts arrivals, bar[1] the
 // barrier's generation; both are left as found plus one generation.  False if
-// the wait ran out: the caller reports it and returns.
+// the wait ran out (or another block's did, which will not come to the next
+// barrier): the bit is set, the caller returns.
 __device__ __forceinline__ bool team_sync(unsigned *bar, Team t, DevStep *st)
 {
     __shared__ int s_ok;
@@ -185,11 +194,12 @@ __device__ __forceinline__ bool team_sync(unsigned *bar, Team t, DevStep *st)
             asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gen) : "memory");
         } else {
-            for (unsigned spins = 0;; spins++) {
+            const unsigned limit = st->wait_limit ? st->wait_limit : TEAM_SPINS;
+            for (unsigned spins = 1;; spins++) {
                 unsigned now;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(gen) : "memory");
                 if (now != g) break;
-                if (spins > TEAM_SPINS) {
+                if (spins >= limit || ((spins & 1023u) == 0 && (__ldcg(&st->err) & ERRB_TIMEOUT))) {
                     atomicOr(&st->err, (unsigned)ERRB_TIMEOUT);
                     ok = 0;
                     break;
@@ -1980,19 +1990,26 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
 // arguments (one entry for a single context, many for a batch).
 // ---------------------------------------------------------------------------
 
+// (Both return if a team's wait ran out, in this step or an earlier one.  In
+// the launches with teams the bit can be set meanwhile, so one thread reads it
+// for its block.)
 #define REPLICA                               \
     const StepArgs &a = A[blockIdx.y];        \
+    if (a.st->err & ERRB_TIMEOUT) return;     \
     const int cur_ = a.st->cur
 
 // the replica's arguments copied to shared memory (hot kernels)
 #define REPLICA_SMEM                                                              \
     __shared__ StepArgs a_sm;                                                     \
+    __shared__ unsigned err_sm;                                                   \
     {                                                                             \
+        if (threadIdx.x == 0) err_sm = A[blockIdx.y].st->err;                     \
         const u64 *src_ = (const u64 *)&A[blockIdx.y];                            \
         u64 *dst_ = (u64 *)&a_sm;                                                 \
         for (int q_ = threadIdx.x; q_ < (int)(sizeof(StepArgs) / 8); q_ += blockDim.x) dst_[q_] = src_[q_]; \
     }                                                                             \
     __syncthreads();                                                              \
+    if (err_sm & ERRB_TIMEOUT) return;                                            \
     const StepArgs &a = a_sm;                                                     \
     const int cur_ = a.st->cur
 
@@ -2075,6 +2092,7 @@ __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_sample_f
             have = r;
         }
         const StepArgs &a = a_sm;
+        if (a.st->err & ERRB_TIMEOUT) continue;   // (no block sets it in this launch)
         const int v0 = fp.vstart[r];
         d_sample<R, GAS, DIST>(a.s, a.list[a.st->cur], a.st, a.p, a.wa, a.sp, a.cl, enum_base, v - v0,
                                fp.vstart[r + 1] - v0, ((SampWarp *)dyn_smem)[threadIdx.x >> 5]);

@@ -67,12 +67,15 @@ struct DevStep {
     u64 iter;
     double shift;
     i64 n_occ;          // list size at the start of the step
+    // (with n_occ: every kernel of a step reads the three first)
+    unsigned err;
+    int cur;            // list buffer holding the current list
     i64 ntot, n0, nex, n_sel, fnc_attempts;
     double mag[8];      // |A_s| of a cluster of size s
     double cmag[8];     // |A_s| / n_att(s): magnitude of one attempt's coefficient
     i64 natt_s[8];      // attempts of a cluster of size s
     int bucket_shift;   // selection buckets cover 2^bucket_shift positions each
-    int pad0;
+    unsigned wait_limit;   // polls after which a team's wait gives up (0: the default)
     i64 nbuckets;
     i64 n_sp;           // spawned records appended (may exceed capacity on overflow)
     u64 cl_packed;      // (clusters << CL_SHIFT) | attempts of buffered clusters
@@ -83,8 +86,6 @@ struct DevStep {
     i64 n_start;        // list size at the start of the latest finished step
     i64 n_step;         // list size at the start of the step under way (n_occ changes at its end)
     double cl_att;      // attempts of the buffered clusters (runaway check; exact below 2^53)
-    unsigned err;
-    int cur;            // list buffer holding the current list
     int kshift;         // key buckets cover 2^kshift keys each
     int scan_blocks;    // blocks of the step's list scan (E_num partials they wrote)
     i64 nkb;            // key buckets in use (0: no direct accumulation this step)
