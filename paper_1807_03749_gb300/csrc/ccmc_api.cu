@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -272,6 +273,17 @@ ccmc_status cuda_fail(ccmc_ctx *c, cudaError_t e, const char *where)
 cudaError_t wait_batch(ccmc_ctx *ctx)
 {
     return ctx->batch ? cudaStreamSynchronize(ctx->batch_stream) : cudaSuccess;
+}
+
+// Bytes [at, at + n) of the page-locked copy of the device scalars to the
+// device, on the context's stream: its kernels need not wait for the legacy
+// stream, and a copy from pageable memory may still be on its way when the call
+// returns.
+cudaError_t put_step(ccmc_ctx *ctx, size_t at, size_t n)
+{
+    const cudaError_t e = cudaMemcpyAsync((char *)ctx->sc.st + at, (const char *)ctx->h_st + at, n,
+                                          cudaMemcpyHostToDevice, ctx->stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->stream);
 }
 
 ccmc_status status_from_bits(ccmc_ctx *ctx, unsigned bits)
@@ -753,6 +765,11 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
         }
     }
 
+    // the tables' copies from pageable memory have arrived before the context's stream reads them
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        ccmc_free(ctx);
+        return CCMC_ERR_CUDA;
+    }
     // initial state: d0_init on HF
     ctx->iter = 0;
     ctx->shift = 0.0;
@@ -827,7 +844,7 @@ ccmc_status ccmc_set_list(ccmc_ctx *ctx, const uint64_t *bits, const int64_t *po
     if (bad & BAD_FIRST) return fail(ctx, CCMC_ERR_ARG, "first entry must be HF");
     if (bad & BAD_ORDER) return fail(ctx, CCMC_ERR_ARG, "list not sorted and unique");
     ctx->sc.cur = nb;
-    DevStep st;
+    DevStep &st = *ctx->h_st;
     memset(&st, 0, sizeof(st));
     st.iter = ctx->iter;
     st.shift = ctx->shift;
@@ -837,8 +854,7 @@ ccmc_status ccmc_set_list(ccmc_ctx *ctx, const uint64_t *bits, const int64_t *po
     // the barriers with it: the error word that is overwritten here may tell,
     // unread, of a wait that ran out and left them with a count
     CK(cudaMemsetAsync(ctx->sc.wa.bar, 0, 64 * sizeof(unsigned), ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaMemcpy(ctx->sc.st, &st, sizeof(DevStep), cudaMemcpyHostToDevice));
+    CK(put_step(ctx, 0, sizeof(DevStep)));
     ctx->stepped = false;
     return CCMC_OK;
 }
@@ -1089,8 +1105,10 @@ ccmc_status ccmc_set_state(ccmc_ctx *ctx, uint64_t iter, double shift, int32_t v
     ctx->records_read = iter;
     CK(wait_batch(ctx));
     CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaMemcpy(&ctx->sc.st->iter, &iter, sizeof(u64), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(&ctx->sc.st->shift, &shift, sizeof(double), cudaMemcpyHostToDevice));
+    static_assert(offsetof(DevStep, iter) == 0 && offsetof(DevStep, shift) == 8, "iteration and shift in one copy");
+    ctx->h_st->iter = iter;
+    ctx->h_st->shift = shift;
+    CK(put_step(ctx, 0, 16));
     return CCMC_OK;
 }
 
@@ -1100,7 +1118,8 @@ ccmc_status ccmc_wait_limit(ccmc_ctx *ctx, uint32_t polls)
     CK(wait_batch(ctx));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->wait_limit = polls;
-    CK(cudaMemcpy(&ctx->sc.st->wait_limit, &polls, sizeof(polls), cudaMemcpyHostToDevice));
+    ctx->h_st->wait_limit = polls;
+    CK(put_step(ctx, offsetof(DevStep, wait_limit), sizeof(polls)));
     return CCMC_OK;
 }
 
@@ -1469,6 +1488,8 @@ ccmc_status ccmc_batch_create(ccmc_ctx **ctxs, int32_t n, void *cuda_stream, ccm
         ok = ok && g.d_args && g.d_vstart && g.d_counter &&
              cudaMemcpy(g.d_args, ga.data(), sizeof(StepArgs) * ga.size(), cudaMemcpyHostToDevice) == cudaSuccess;
     }
+    // (as in ccmc_init: arrived before the batch's stream reads them)
+    ok = ok && cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess;
     // per-replica shapes may not exceed what every context allocated for
     Shapes lim = ctxs[0]->sc.sh;
     for (int r = 1; r < n; r++) {
