@@ -332,12 +332,16 @@ void ccmc_batch_free(ccmc_batch *b);
  * plus histograms, block partials and barriers), held by every GPU that
  * loads the library until the process exits.  n above
  * CCMC_NOALLOC_MAX_RECORDS is rejected with CCMC_ERR_ARG before any work.
- * The first call on a device looks up that array's device address (once per
- * device, with the device current); make that first call before any stream
+ * The first call on a device looks up that array's device address, sets the
+ * kernel's shared-memory size and allocates a page of page-locked host memory
+ * for the results (once per device, with the device current; another page for
+ * every 64 calls under way at a time); make that first call before any stream
  * capture.  The array is shared per device by every caller in the process
  * (other streams, other threads, other library contexts) and keeps the last
  * call's contents; calls that overlap on the GPU race and must be
- * serialised by the caller. */
+ * serialised by the caller.  Calls of several threads that the GPU runs one
+ * after another (on one stream, or on streams ordered by events) may overlap
+ * on the host. */
 ccmc_status ccmc_reduce_records_noalloc(const uint64_t *keys_in, const int64_t *pops_in, size_t n, int32_t key_bits,
                                         uint64_t *keys_out, int64_t *pops_out, size_t *n_out, void *cuda_stream);
 

@@ -151,7 +151,9 @@ constexpr size_t NOALLOC_MAX = (size_t)1 << 16;   // records per call
 constexpr int NOALLOC_GRID = (int)(NOALLOC_MAX / (2 * SORT_THREADS));   // blocks of the largest call
 
 struct NoAllocResult {
-    i64 n_keys;   // -1: a wait ran out
+    i64 n_keys;
+    int unfinished;        // a wait ran out (set by the block that gave up; n_keys may be written all the same)
+    NoAllocResult *next;   // of the free ones
 };
 
 struct NoAllocScratch {
@@ -165,9 +167,15 @@ struct NoAllocScratch {
 
 __device__ __align__(256) NoAllocScratch g_noalloc;
 
+constexpr int NOALLOC_SLOTS = 64;   // results allocated at a time
+
 std::mutex g_noalloc_mutex;
 NoAllocScratch *g_noalloc_ptr[256];
-NoAllocResult *g_noalloc_out[256];   // page-locked, mapped: the kernel writes a call's result there
+// Page-locked, mapped words, one per call under way: the kernel writes its
+// call's result there.  Calls of several threads can follow each other on the
+// GPU (one stream, or streams ordered by events) while their host parts
+// overlap, so a word belongs to one call from its launch until it is read.
+NoAllocResult *g_noalloc_free[256];
 
 // The whole call (its blocks wait for each other: a cooperative launch when
 // there are several).
@@ -177,21 +185,34 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_noalloc(const u64 *keys_in,
 {
     SortSmem &S = *(SortSmem *)dyn_smem;
     __shared__ i64 sm[64];
+    __shared__ unsigned err;
     const Team t = {(int)blockIdx.x, (int)gridDim.x};
+    if (t.n > 1) {
+        // a wait of an earlier call that has not cleared the barriers yet ran out
+        if (threadIdx.x == 0) err = N->st.err;
+        __syncthreads();
+        if (err & ERRB_TIMEOUT) {
+            res->unfinished = 1;
+            return;
+        }
+    }
     u64 *key[2] = {N->key[0], N->key[1]};
     i64 *pop[2] = {N->pop[0], N->pop[1]};
-    if (!team_sort(keys_in, pops_in, key, pop, n, key_bits, SORT_DIGIT_BITS, N->hist, N->bar, t, &N->st, S)) return;
-    const int src = ((key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS) & 1;
-    const i64 m = team_reduce(key[src], pop[src], n, keys_out, pops_out, N->part, N->bar, t, &N->st, sm);
-    if (t.id == 0 && threadIdx.x == 0) res->n_keys = m;
+    i64 m = -1;
+    if (team_sort(keys_in, pops_in, key, pop, n, key_bits, SORT_DIGIT_BITS, N->hist, N->bar, t, &N->st, S)) {
+        const int src = ((key_bits + SORT_DIGIT_BITS - 1) / SORT_DIGIT_BITS) & 1;
+        m = team_reduce(key[src], pop[src], n, keys_out, pops_out, N->part, N->bar, t, &N->st, sm);
+    }
+    if (m < 0) res->unfinished = 1;
+    else if (t.id == 0 && threadIdx.x == 0) res->n_keys = m;
 }
 
-// Device address of the scratch on the current device, looked up once per
+// Device address of the scratch on the current device dev, looked up once per
 // device (host code cannot use the symbol itself as a device address), with
-// the kernel's shared memory size set and a page-locked word for the result.
-cudaError_t noalloc_scratch(NoAllocScratch **out, NoAllocResult **res)
+// the kernel's shared memory size set, and a page-locked word for the result
+// that the caller gives back.
+cudaError_t noalloc_scratch(int &dev, NoAllocScratch **out, NoAllocResult **res)
 {
-    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
@@ -202,15 +223,26 @@ cudaError_t noalloc_scratch(NoAllocScratch **out, NoAllocResult **res)
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(k_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
         if (e != cudaSuccess) return e;
-        if (!g_noalloc_out[dev]) {
-            e = cudaHostAlloc((void **)&g_noalloc_out[dev], sizeof(NoAllocResult), cudaHostAllocMapped);
-            if (e != cudaSuccess) return e;
-        }
         g_noalloc_ptr[dev] = (NoAllocScratch *)p;
     }
+    if (!g_noalloc_free[dev]) {
+        NoAllocResult *r = nullptr;
+        e = cudaHostAlloc((void **)&r, NOALLOC_SLOTS * sizeof(NoAllocResult), cudaHostAllocMapped);
+        if (e != cudaSuccess) return e;
+        for (int q = 0; q < NOALLOC_SLOTS; q++) r[q].next = q + 1 < NOALLOC_SLOTS ? r + q + 1 : nullptr;
+        g_noalloc_free[dev] = r;
+    }
     *out = g_noalloc_ptr[dev];
-    *res = g_noalloc_out[dev];
+    *res = g_noalloc_free[dev];
+    g_noalloc_free[dev] = (*res)->next;
     return cudaSuccess;
+}
+
+void noalloc_done(int dev, NoAllocResult *res)
+{
+    std::lock_guard<std::mutex> lock(g_noalloc_mutex);
+    res->next = g_noalloc_free[dev];
+    g_noalloc_free[dev] = res;
 }
 
 }  // namespace
@@ -228,20 +260,25 @@ extern "C" ccmc_status ccmc_reduce_records_noalloc(const uint64_t *keys_in, cons
     if (n == 0) return CCMC_OK;
     if (!keys_in || !pops_in || !keys_out || !pops_out) return CCMC_ERR_ARG;
     cudaStream_t sm = (cudaStream_t)cuda_stream;
+    int dev = 0;
     NoAllocScratch *S = nullptr;
     NoAllocResult *res = nullptr;
-    if (noalloc_scratch(&S, &res) != cudaSuccess) return CCMC_ERR_CUDA;
-    res->n_keys = -1;
-    if (launch_blocks(k_noalloc, dim3((unsigned)sort_blocks((i64)n)), n > SORT_TILE, SORT_THREADS, sizeof(SortSmem), sm,
-                      (const u64 *)keys_in, (const i64 *)pops_in, (i64)n, (int)key_bits, (u64 *)keys_out, (i64 *)pops_out,
-                      S, res) != cudaSuccess)
-        return CCMC_ERR_CUDA;
-    if (cudaStreamSynchronize(sm) != cudaSuccess) return CCMC_ERR_CUDA;
+    if (noalloc_scratch(dev, &S, &res) != cudaSuccess) return CCMC_ERR_CUDA;
+    res->n_keys = 0;
+    res->unfinished = 0;
+    cudaError_t e = launch_blocks(k_noalloc, dim3((unsigned)sort_blocks((i64)n)), n > SORT_TILE, SORT_THREADS,
+                                  sizeof(SortSmem), sm, (const u64 *)keys_in, (const i64 *)pops_in, (i64)n, (int)key_bits,
+                                  (u64 *)keys_out, (i64 *)pops_out, S, res);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(sm);
     const i64 m = *(volatile i64 *)&res->n_keys;
-    if (m < 0) {   // a wait ran out: the next call starts clean
+    const bool unfinished = *(volatile int *)&res->unfinished != 0;
+    if (e == cudaSuccess && unfinished) {   // a wait ran out: the next call starts clean
         cudaMemsetAsync(S->bar, 0, sizeof(S->bar) + sizeof(S->st), sm);
-        return CCMC_ERR_TIMEOUT;
+        cudaStreamSynchronize(sm);
     }
+    noalloc_done(dev, res);
+    if (e != cudaSuccess) return CCMC_ERR_CUDA;
+    if (unfinished) return CCMC_ERR_TIMEOUT;
     *n_out = (size_t)m;
     return CCMC_OK;
 }
