@@ -14,6 +14,7 @@ constexpr int MAX_CHECKPOINTS = 64;
 constexpr int TILE_I = 32, TILE_J = 64;   // excitors per side of a pair tile
 constexpr int GROUP = 128;                // iterations in one 16-byte word of a plane
 constexpr int CHUNK = 1024;               // iterations whose owners a warp stages at a time
+constexpr int MAX_PLANES = 16;            // bits of an owner (n_ranks <= 65535)
 
 // The owners as bit planes over time: bit t of planes[(g nb + b) npad + i] is
 // bit b of excitor i's owner at iteration 128 g + t, so that two excitors'
@@ -216,10 +217,13 @@ extern "C" ccmc_status ccmc_colocation(const uint64_t *dets, size_t n, int32_t n
     u64 *d_dets = (u64 *)((unsigned char *)mem + planes_bytes), *d_s1 = d_dets + nn * nw, *d_s2 = d_s1 + nck;
     i64 *d_ck = (i64 *)(d_s2 + nck);
     const size_t smem = 2 * (size_t)nb * (TILE_I + TILE_J) * sizeof(uint4);
+    // the limit belongs to the kernel, not to the launch: every call sets the
+    // same one, so that a call of another thread cannot lower it in between
+    constexpr int PAIRS_SMEM_MAX = 2 * MAX_PLANES * (TILE_I + TILE_J) * (int)sizeof(uint4);
     if (cudaMemcpyAsync(d_dets, dets, nn * nw * 8, cudaMemcpyHostToDevice, sm) != cudaSuccess ||
         cudaMemcpyAsync(d_ck, checkpoints, nck * 8, cudaMemcpyHostToDevice, sm) != cudaSuccess ||
         cudaMemsetAsync(d_s1, 0, 2 * nck * 8, sm) != cudaSuccess ||
-        cudaFuncSetAttribute(k_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaFuncSetAttribute(k_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIRS_SMEM_MAX) != cudaSuccess) {
         st = CCMC_ERR_CUDA;
     } else {
         k_owner_planes<<<1216, 256, 0, sm>>>(d_dets, (i64)n, (i64)npad, n_words, t_max, nu_move, (u64)n_ranks, nb, planes);
@@ -231,6 +235,7 @@ extern "C" ccmc_status ccmc_colocation(const uint64_t *dets, size_t n, int32_t n
             cudaStreamSynchronize(sm) != cudaSuccess)
             st = CCMC_ERR_CUDA;
     }
+    if (st != CCMC_OK) cudaStreamSynchronize(sm);   // no copy may still use the caller's arrays
     cudaFreeAsync(mem, sm);
     return st;
 }
