@@ -262,9 +262,10 @@ ccmc_status ccmc_phase_times(ccmc_ctx *ctx, double *ms, int64_t *launches, int32
 
 /* ---- Batched form: many independent contexts stepped together ----------
  * Every phase of the step is one kernel launch over all replicas that share
- * a Hamiltonian kind and precision (a CUDA grid dimension indexes the
- * replica), and the whole step is captured once in a CUDA graph and replayed.
- * The cluster sampler, the bulk of the work, is one persistent launch whose
+ * a Hamiltonian kind and precision, and the whole step is captured once in a
+ * CUDA graph and replayed.  The scan and the annihilation share their blocks
+ * out in proportion to each replica's list and records.  The cluster sampler,
+ * the bulk of the work, is one persistent launch whose
  * blocks take shares of the replicas' samples from a plan written on the
  * device each step, so replicas of very different sizes keep the GPU busy.
  * Per-replica grid sizes, the sampler's samples per share and the radix digit

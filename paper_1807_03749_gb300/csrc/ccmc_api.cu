@@ -1250,7 +1250,7 @@ struct BatchGroup {
 
 // Shapes the tuner chooses between.
 struct BatchShape {
-    int work = 64;      // per-replica blocks of the list, merge and sort kernels
+    int work = 64;      // per-replica blocks of the attempt and owner-table kernels
     int tile = 1024;    // samples per share of the persistent sampler
     int digit = 8;      // radix digit bits
 };
@@ -1317,8 +1317,6 @@ Shapes shapes_for(const ccmc_batch *b, const BatchShape &c)
 {
     Shapes sh = b->lim;
     sh.work_grid = std::min(c.work, b->lim.work_grid);
-    sh.scan_grid = std::min(std::max(2, c.work / 2), b->lim.scan_grid);
-    sh.sort_grid = std::min(std::max(2, c.work / 2), b->lim.sort_grid);
     sh.digit_bits = c.digit;
     sh.enum_slots = sh.scan_grid + sh.work_grid;
     return sh;

@@ -627,11 +627,11 @@ __device__ __forceinline__ i64 threshold(const RunParams &p, u64 it, u64 key, i6
 // a1: scans over the list
 // ---------------------------------------------------------------------------
 
-// Blocks of the list scan: one per 512 entries (two rows of 32 per warp).
-__device__ __forceinline__ int scan_blocks(i64 n)
+// Blocks of the list scan: one per 512 entries (one row of 32 per warp).
+__device__ __forceinline__ i64 scan_blocks(i64 n)
 {
     const i64 b = (n + SCAN_THREADS - 1) / SCAN_THREADS;
-    return (int)(b < 1 ? 1 : (b > (i64)gridDim.x ? (i64)gridDim.x : b));
+    return b < 1 ? 1 : b;
 }
 
 // this warp's entries of the list: warp-granular chunks need no block barrier
@@ -1986,7 +1986,8 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
 
 
 // ---------------------------------------------------------------------------
-// Kernels: each block serves replica blockIdx.y of an array of per-replica
+// Kernels: each block serves replica blockIdx.y (the list kernels: the
+// replicas of its shares) of an array of per-replica
 // arguments (one entry for a single context, many for a batch).
 // ---------------------------------------------------------------------------
 
@@ -2020,16 +2021,174 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_local_scan(const StepArgs *__r
 // owners and position table of the simulated distribution, for K words
 void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm);
 
+// The blocks of a batch's launch shared out between its replicas, in
+// proportion to the blocks that each would use alone (units_of(r), which must
+// not change during the launch).  Every block works the same shares out: a
+// replica's team is a run of blocks if its share is two or more.  The blocks
+// left over take the other replicas, one block each, round after round; the
+// last, partly filled round has as many blocks for each as there are.  A block
+// takes its replicas in this order and only later ones wait for it, so every
+// wait ends.
+//
+// Equal shares (two blocks per SM over the replicas) left a list of 4.8e6
+// entries among 200 small ones to one block: 32.5 ms a step, now 1.06 (one of
+// 95,000 entries: 1.27 and 0.42 ms).  Where equal shares were right it costs
+// the working out, some 3 us a launch: 64 replicas of 18,000 entries 0.951 and
+// 0.959 ms a step, 700 of 280 entries 0.65 and 0.69 ms.
+//
+// (All that is kept between replicas is in shared memory: in registers it
+// would spill in the loops of the replica's own work.)
+struct Shares {
+    static constexpr int KEPT = 2 * SCAN_THREADS;   // replicas whose units are read once
+    i64 sm[32], want, give;       // units of the replicas that want several blocks, blocks for them
+    int smi[32], kept[KEPT], list[SCAN_THREADS];
+    int first, hands, full, per;  // blocks before those left over, these, rounds of these, blocks each in the last round
+    int stage, base, rank, q, count;
+    int rep, tail;                // the replica to do, the one of the last round
+    Team team, tail_team;
+};
+
+template <typename U>
+__device__ __forceinline__ i64 units_at(const Shares &S, int r, U units_of)
+{
+    return r < Shares::KEPT ? S.kept[r] : units_of(r);
+}
+
+// blocks of replica r's team, 0: done by the blocks left over
+__device__ __forceinline__ int share_at(i64 u, i64 want, i64 give, int most)
+{
+    const i64 n = u < 2 ? 0 : u * give / want;
+    return n < 2 ? 0 : (int)(n < most ? n : most);
+}
+
+template <typename U>
+__device__ __forceinline__ void shares_init(Shares &S, int nrep, int most, U units_of)
+{
+    const int B = (int)gridDim.x, id = (int)blockIdx.x, tid = threadIdx.x;
+    i64 v = 0;   // units of the replicas that want several blocks, and the other replicas
+#pragma unroll
+    for (int r = tid; r < Shares::KEPT; r += SCAN_THREADS) {
+        const i64 u = r < nrep ? units_of(r) : 0;
+        S.kept[r] = (int)u;
+        v += u > 1 ? u << 24 : u;
+    }
+    for (int r = Shares::KEPT + tid; r < nrep; r += SCAN_THREADS) {
+        const i64 u = units_of(r);
+        v += u > 1 ? u << 24 : 1;
+    }
+    v = block_sum(v, S.sm);
+    const i64 want = v >> 24, ones = v & ((1 << 24) - 1), give = want + ones <= B ? want : B * want / (want + ones);
+    if (tid == 0) {
+        S.stage = S.base = S.rank = S.q = S.count = 0;
+        S.tail = -1;
+        S.want = want;
+        S.give = give;
+    }
+    int taken = 0, teams = 0;
+    for (int base = 0; want > 0 && base < nrep; base += SCAN_THREADS) {
+        const int r = base + tid, n = r < nrep ? share_at(units_at(S, r, units_of), want, give, most) : 0;
+        int tot;   // blocks, teams << 16
+        const int at = taken + (block_incl_scan(n ? n | (1 << 16) : 0, S.smi, tot) & 0xFFFF) - n;
+        if (id >= at && id < at + n) {
+            S.rep = r;
+            S.team = Team{id - at, n};
+            S.count = 1;
+        }
+        taken += tot & 0xFFFF;
+        teams += tot >> 16;
+    }
+    if (tid == 0) {
+        const int first = taken < B ? taken : 0, hands = B - first, left = nrep - teams;
+        S.first = first;
+        S.hands = hands;
+        S.full = left / hands;
+        S.per = left % hands ? hands / (left % hands) : 0;
+    }
+}
+
+// The next replica of this block in S.rep, with S.team; false if there is none.
+template <typename U>
+__device__ __forceinline__ bool next_share(Shares &S, int nrep, int most, U units_of)
+{
+    const int id = (int)blockIdx.x, tid = threadIdx.x;
+    __syncthreads();
+    if (S.stage == 0) {
+        const int have = S.count;
+        __syncthreads();
+        if (tid == 0) {
+            S.stage = 1;
+            S.count = 0;
+        }
+        if (have) return true;
+        __syncthreads();
+    }
+    if (id < S.first) return false;
+    for (;;) {
+        const int q = S.q, count = S.count, base = S.base, rank = S.rank;
+        __syncthreads();
+        if (q < count) {
+            if (tid == 0) {
+                S.rep = S.list[q];
+                S.team = Team{0, 1};
+                S.q = q + 1;
+            }
+            __syncthreads();
+            return true;
+        }
+        if (base >= nrep) break;
+        const int r = base + tid, hands = S.hands;
+        const i64 u = r < nrep ? units_at(S, r, units_of) : 0;
+        const bool one = r < nrep && share_at(u, S.want, S.give, most) == 0;
+        if (tid == 0) {
+            S.base = base + SCAN_THREADS;
+            S.q = S.count = 0;
+        }
+        int tot;
+        const int at = rank + block_incl_scan(one ? 1 : 0, S.smi, tot) - 1, late = at - S.full * hands;
+        if (one && late < 0) {
+            if (at % hands == id - S.first) S.list[atomicAdd(&S.count, 1)] = r;
+        } else if (one) {
+            const i64 m = u < most ? u : most;
+            const int per = S.per, n = (int)(m < per ? m : per), b = id - S.first - late * per;
+            if (b >= 0 && b < n) {
+                S.tail = r;
+                S.tail_team = Team{b, n};
+            }
+        }
+        if (tid == 0) S.rank = rank + tot;
+        __syncthreads();
+    }
+    const int tail = S.tail;
+    __syncthreads();
+    if (tail < 0) return false;
+    if (tid == 0) {
+        S.rep = tail;
+        S.team = S.tail_team;
+        S.tail = -1;
+    }
+    __syncthreads();
+    return true;
+}
+
+// a replica's arguments copied to shared memory; false if a team's wait ran
+// out for it (as in REPLICA_SMEM).  All threads of the block call.
+__device__ __forceinline__ bool load_replica(StepArgs &a, const StepArgs &from, unsigned &err)
+{
+    __syncthreads();   // the replica before is done
+    if (threadIdx.x == 0) err = from.st->err;
+    const u64 *src = (const u64 *)&from;
+    u64 *dst = (u64 *)&a;
+    for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / 8); q += blockDim.x) dst[q] = src[q];
+    __syncthreads();
+    return !(err & ERRB_TIMEOUT);
+}
+
 // a1 in one launch: block sums, a barrier, then every block derives the
 // totals and its prefix itself and writes its entries' rows.
 template <typename R, bool GAS>
-__global__ void __launch_bounds__(SCAN_THREADS, 2) k_scan(const StepArgs *__restrict__ A)
+__device__ __forceinline__ void d_scan(const StepArgs &a, Team t, i64 *sm)
 {
-    REPLICA_SMEM;
-    __shared__ i64 sm[64];
-    const Team t = {(int)blockIdx.x, scan_blocks(a.st->n_occ)};
-    if (t.id >= t.n) return;
-    const ListView &L = a.list[cur_];
+    const ListView &L = a.list[a.st->cur];
     i64 bw, ba, cw, ca, tw, ta = 0;
     d_scan_partial(L, a.st, a.p, a.wa, t, bw, ba, sm);
     if (!team_sync(a.wa.bar, t, a.st)) return;
@@ -2041,6 +2200,27 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_scan(const StepArgs *__rest
     }
     const ScanScalars sc = d_scan_top(L, a.st, a.p, a.wa, tw, ta, a.s.lmax, t);
     d_scan_final<R, GAS>(a.s, L, a.st, a.p, a.wa, t, cw + bw, ca + ba, sc);
+}
+
+// MANY: nrep replicas share the launch's blocks, teams of most blocks at most
+template <typename R, bool GAS, bool MANY>
+__global__ void __launch_bounds__(SCAN_THREADS, 2) k_scan(const StepArgs *__restrict__ A, int nrep, int most)
+{
+    __shared__ i64 sm[64];
+    if constexpr (MANY) {
+        __shared__ Shares S;
+        __shared__ StepArgs a;
+        __shared__ unsigned err;
+        const auto units = [&](int r) { return scan_blocks(A[r].st->n_occ); };
+        shares_init(S, nrep, most, units);
+        while (next_share(S, nrep, most, units))
+            if (load_replica(a, A[S.rep], err)) d_scan<R, GAS>(a, S.team, sm);
+    } else {
+        REPLICA_SMEM;
+        const i64 b = scan_blocks(a.st->n_occ);
+        const Team t = {(int)blockIdx.x, (int)(b < most ? b : most)};
+        if (t.id < t.n) d_scan<R, GAS>(a, t, sm);
+    }
 }
 
 extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -2115,24 +2295,29 @@ struct AnnihilateShape {
     int enum_base, enum_slots;   // the sampler's E_num partials
 };
 
-template <typename R, bool GAS>
-__global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *__restrict__ A, AnnihilateShape as, int what)
+// records in the spawn buffer
+__device__ __forceinline__ i64 spawned_of(const StepArgs &a) { return a.st->n_sp < a.sp.cap ? a.st->n_sp : a.sp.cap; }
+
+// Blocks of the annihilation: up to a tile of records one block, else one per
+// 1,024; one per 1,024 list entries.  (n_step, not n_occ: a block that starts
+// after the last one has finished the step must see the same team.)
+__device__ __forceinline__ i64 annihilate_blocks(const StepArgs &a)
 {
-    REPLICA_SMEM;
-    __shared__ i64 sm[128];
-    __shared__ bool s_last;
-    SortSmem &S = *(SortSmem *)dyn_smem;
+    const i64 bs = sort_blocks(spawned_of(a)), bm = (a.st->n_step + 2 * SCAN_THREADS - 1) / (2 * SCAN_THREADS);
+    return bs > bm ? bs : (bm < 1 ? 1 : bm);
+}
+
+template <typename R, bool GAS>
+__device__ __forceinline__ void d_annihilate(const StepArgs &a, Team team, const AnnihilateShape &as, int what, SortSmem &S, i64 *sm,
+                                             bool &s_last)
+{
     DevStep *st = a.st;
+    const int cur_ = st->cur;
     const WorkArrays &wa = a.wa;
     const ListView &L = a.list[cur_], &O = a.list[cur_ ^ 1];
-    // (n_step: a block that starts after the last one has finished the step
-    // must see the same team)
-    const i64 nsp = st->n_sp < a.sp.cap ? st->n_sp : a.sp.cap, n = st->n_step;
-    // up to a tile of records one block, else one per 1,024; one per 1,024 list entries
-    const i64 G = gridDim.x, bs = sort_blocks(nsp), bm = (n + 2 * SCAN_THREADS - 1) / (2 * SCAN_THREADS);
-    const int ns = (int)(bs < 1 ? 1 : (bs > G ? G : bs)), nm = (int)(bm < 1 ? 1 : (bm > G ? G : bm));
-    const Team sort_team = {(int)blockIdx.x, ns}, team = {(int)blockIdx.x, ns > nm ? ns : nm};
-    if (team.id >= team.n) return;
+    const i64 nsp = spawned_of(a);
+    const i64 bs = sort_blocks(nsp);
+    const Team sort_team = {team.id, (int)(bs < team.n ? bs : team.n)};
     const int src = ((as.key_bits + as.digit_bits - 1) / as.digit_bits) & 1;   // the sorted pair
     if (nsp > 0 && sort_team.id < sort_team.n) {
         if (what & DO_SORT)
@@ -2179,6 +2364,29 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *
     }
 }
 
+template <typename R, bool GAS, bool MANY>
+__global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *__restrict__ A, int nrep, int most, AnnihilateShape as,
+                                                                int what)
+{
+    __shared__ i64 sm[128];
+    __shared__ bool s_last;
+    SortSmem &S = *(SortSmem *)dyn_smem;
+    if constexpr (MANY) {
+        __shared__ Shares W;
+        __shared__ StepArgs a;
+        __shared__ unsigned err;
+        const auto units = [&](int r) { return annihilate_blocks(A[r]); };
+        shares_init(W, nrep, most, units);
+        while (next_share(W, nrep, most, units))
+            if (load_replica(a, A[W.rep], err)) d_annihilate<R, GAS>(a, W.team, as, what, S, sm, s_last);
+    } else {
+        REPLICA_SMEM;
+        const i64 b = annihilate_blocks(a);
+        const Team t = {(int)blockIdx.x, (int)(b < most ? b : most)};
+        if (t.id < t.n) d_annihilate<R, GAS>(a, t, as, what, S, sm, s_last);
+    }
+}
+
 // Launches a grid, cooperatively (all blocks resident) if its blocks wait for
 // one another.
 template <typename... P, typename... Q>
@@ -2197,11 +2405,11 @@ cudaError_t launch_blocks(void (*k)(P...), dim3 grid, bool cooperative, int thre
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
-// Launches a kernel whose blocks wait for their replica's other blocks: as
-// many per replica as fit on the GPU with every replica's (at most want).
-// One block per replica waits for nobody.
+// Launches a kernel whose blocks wait for their replica's other blocks, teams
+// of most blocks at most: as many blocks as fit on the GPU, of a single
+// replica's at most those.
 template <typename... P, typename... Q>
-cudaError_t launch_team(void (*k)(P...), int want, int nrep, int threads, size_t smem, cudaStream_t sm, Q... args)
+cudaError_t launch_team(void (*k)(P...), const StepArgs *A, int nrep, int most, int threads, size_t smem, cudaStream_t sm, Q... args)
 {
     int dev = 0, sms = 0, per = 0;
     if (cudaError_t e = cudaGetDevice(&dev)) return e;
@@ -2209,10 +2417,11 @@ cudaError_t launch_team(void (*k)(P...), int want, int nrep, int threads, size_t
     if (smem)
         if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
     if (cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, smem)) return e;
-    int g = per * sms / nrep;
-    if (g > want) g = want;
-    if (g < 1) g = 1;
-    return launch_blocks(k, dim3(g, nrep), g > 1, threads, smem, sm, args...);
+    int g = per * sms;
+    if (most > g) most = g;
+    if (most < 1) most = 1;
+    if (nrep == 1) g = most;
+    return launch_blocks(k, dim3(g), g > 1, threads, smem, sm, A, nrep, most, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -2230,7 +2439,8 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, int K, const Shapes &sh, 
     const dim3 gwork(sh.work_grid, nrep);
     const int team = min(sh.scan_grid, sh.sort_grid);
     mark(0);
-    if (cudaError_t e = launch_team(k_scan<R, GAS>, team, nrep, SCAN_THREADS, 0, sm, A)) return e;
+    auto *scan = nrep > 1 ? k_scan<R, GAS, true> : k_scan<R, GAS, false>;
+    if (cudaError_t e = launch_team(scan, A, nrep, team, SCAN_THREADS, 0, sm)) return e;
     launches[0] += 1;
     if (sh.nranks > 1) {
         // simulated distribution: owners and per-processor position tables
@@ -2259,12 +2469,12 @@ cudaError_t launch_phases(const StepArgs *A, int nrep, int K, const Shapes &sh, 
         launches[2] += 1;
     }
     const AnnihilateShape as = {sh.key_bits, sh.digit_bits, sh.scan_grid, plan ? plan->wmax : sh.work_grid};
+    auto *annihilate = nrep > 1 ? k_annihilate<R, GAS, true> : k_annihilate<R, GAS, false>;
     // one launch, or with the phase timers one per phase (a7, a8, a9, a10)
     for (int ph = 0; ph < 4; ph++) {
         mark(3 + ph);
         if (!ev && ph > 0) continue;
-        if (cudaError_t e = launch_team(k_annihilate<R, GAS>, team, nrep, SCAN_THREADS, sizeof(SortSmem), sm, A, as,
-                                        ev ? 1 << ph : (int)DO_ALL))
+        if (cudaError_t e = launch_team(annihilate, A, nrep, team, SCAN_THREADS, sizeof(SortSmem), sm, as, ev ? 1 << ph : (int)DO_ALL))
             return e;
         launches[3 + ph] += 1;
     }

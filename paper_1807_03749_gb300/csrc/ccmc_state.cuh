@@ -178,7 +178,7 @@ struct Shapes {
 };
 
 // Per-replica arguments of the step kernels (device-resident; a single
-// context has one, a batch an array indexed by blockIdx.y).
+// context has one, a batch an array with one per replica).
 struct StepArgs {
     SysDev s;
     RunParams p;
