@@ -265,11 +265,12 @@ ccmc_status ccmc_phase_times(ccmc_ctx *ctx, double *ms, int64_t *launches, int32
  * a Hamiltonian kind and precision, and the whole step is captured once in a
  * CUDA graph and replayed.  The scan and the annihilation share their blocks
  * out in proportion to each replica's list and records.  The cluster sampler,
- * the bulk of the work, is one persistent launch whose
- * blocks take shares of the replicas' samples from a plan written on the
- * device each step, so replicas of very different sizes keep the GPU busy.
- * Per-replica grid sizes, the sampler's samples per share and the radix digit
- * width are chosen by timing candidates on real steps, again whenever the
+ * the bulk of the work, is one persistent launch whose blocks take shares of
+ * the replicas' samples from a plan written on the device each step, so
+ * replicas of very different sizes keep the GPU busy.
+ * The sampler's samples per share, the radix digit width and (where a member
+ * uses these kernels) the blocks per replica of the attempts and of the owner
+ * tables are chosen by timing candidates on real steps, again whenever the
  * batch's total population has changed by a factor of two since the last
  * choice (the trajectory does not depend on them).
  * Replicas keep their own Philox keys, shift control and checkpoints; results

@@ -1255,6 +1255,8 @@ struct BatchShape {
     int digit = 8;      // radix digit bits
 };
 
+// stages: blocks of the attempt and owner-table kernels (of batches that
+// launch them), samples per share, digit
 constexpr int TUNE_STAGES = 3;
 const int TUNE_WORK[] = {32, 64, 128, 256};
 const int TUNE_TILE[] = {256, 512, 1024, 2048, 4096};
@@ -1281,7 +1283,8 @@ struct ccmc_batch {
     BatchShape shape;                 // current choice
     int flat_grid = 0;                // blocks of the persistent sampler
     bool tuned = false;
-    int tune_stage = 0, tune_idx = 0, tunings = 0;
+    int first_stage = 1;              // 0 if a member uses the kernels of the first stage
+    int tune_stage = 1, tune_idx = 0, tunings = 0;
     BatchShape tune_best;
     float tune_best_ms = 0.0f;
     cudaEvent_t tune_ev[2] = {nullptr, nullptr};
@@ -1386,7 +1389,7 @@ ccmc_status batch_boundaries(ccmc_batch *b)
     // a population twice or half as large as at the last tuning: tune again
     if (b->tuned && (pop > 2.0 * b->pop_tuned || pop < 0.5 * b->pop_tuned)) {
         b->tuned = false;
-        b->tune_stage = 0;
+        b->tune_stage = b->first_stage;
         b->tune_idx = 0;
         b->tune_best = b->shape;
         b->tune_best_ms = 1e30f;
@@ -1498,6 +1501,8 @@ ccmc_status ccmc_batch_create(ccmc_ctx **ctxs, int32_t n, void *cuda_stream, ccm
     }
     lim.digit_bits = MAX_DIGIT_BITS;
     b->lim = lim;
+    for (const BatchGroup &g : b->groups)
+        if (g.multi || lim.nranks > 1) b->first_stage = b->tune_stage = 0;
     b->sh = shapes_for(b, b->shape);
     int dev = 0, sms = 0;
     ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
