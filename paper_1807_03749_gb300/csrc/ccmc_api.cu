@@ -687,7 +687,11 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     const i64 lc = ctx->list_cap;
     wa.picks = al.arr<PickEntry>(lc);
     wa.href = al.arr<double>(lc);
-    wa.bucket_bits = 18;
+    // up to 2^18 buckets for a short list: what the scan asks for at a full list
+    // and at twice the target population
+    wa.bucket_bits = 10;
+    while (wa.bucket_bits < 18 && (double)(1LL << wa.bucket_bits) < std::max(2.0 * (double)lc, params->target_pop / 16.0))
+        wa.bucket_bits++;
     while (wa.bucket_bits < 24 && (1LL << wa.bucket_bits) < lc / 2) wa.bucket_bits++;
     wa.bucket = al.arr<int>(((size_t)1 << wa.bucket_bits) + 1);
     wa.att_end = al.arr<i64>(lc);
@@ -706,7 +710,7 @@ ccmc_status ccmc_init(const ccmc_hamiltonian *ham, const ccmc_reference *ref, in
     wa.part = al.arr<i64>(4 * 2 * (size_t)std::max(sh.scan_grid, sh.work_grid));
     wa.bar = al.arr<unsigned>(64);
     wa.enum_part = al.arr<u64>(2 * (size_t)sh.enum_slots);
-    wa.hist = al.arr<unsigned>((size_t)(1 << SORT_DIGIT_BITS) * sh.sort_grid);
+    wa.hist = al.arr<unsigned>((size_t)(1 << SORT_DIGIT_BITS) * (size_t)std::min<i64>(sh.sort_grid, sort_blocks(sp.cap)));
     wa.ring = al.arr<Record>(RING);
     wa.owner = nullptr;
     wa.lcp = nullptr;

@@ -1415,15 +1415,6 @@ struct SortSmem {
     unsigned sc[32];
 };
 
-// Blocks that sort n records.  A pass of several blocks is latency (a tile,
-// two barriers and the reads between: 13 us a digit with 1,024 records per
-// block, 16 us with 4,096); one block's passes have no barriers, so it takes a
-// whole tile.
-__host__ __device__ __forceinline__ i64 sort_blocks(i64 n)
-{
-    return n <= SORT_TILE ? 1 : (n + 2 * SORT_THREADS - 1) / (2 * SORT_THREADS);
-}
-
 // Sorts a tile's items (ipt per thread; item j of lane l of warp w is number
 // 32 (ipt w + j) + l) by one digit into S.tk / S.tv, stably: digit, then warp, item, lane.  Leaves
 // the digits' counts in S.tot and their exclusive prefix in S.tpre.

@@ -15,6 +15,15 @@ constexpr int SORT_ITEMS = 8;
 constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;
 constexpr int MAX_DIGIT_BITS = 8;         // of a caller's choice
 constexpr int SORT_DIGIT_BITS = 9;        // default: one digit value per thread of a sorting block
+// Blocks that sort n records.  A pass of several blocks is latency (a tile,
+// two barriers and the reads between: 13 us a digit with 1,024 records per
+// block, 16 us with 4,096); one block's passes have no barriers, so it takes a
+// whole tile.
+__host__ __device__ __forceinline__ i64 sort_blocks(i64 n)
+{
+    return n <= SORT_TILE ? 1 : (n + 2 * SORT_THREADS - 1) / (2 * SORT_THREADS);
+}
+
 // resident blocks of the cluster sampler per SM (its register budget)
 #ifndef CCMC_SAMPLE_BLOCKS_PER_SM
 #define CCMC_SAMPLE_BLOCKS_PER_SM 3
@@ -157,7 +166,7 @@ struct WorkArrays {
     int *before;      // kept new keys inserted just before each list entry
     i64 *keep_s;      // keep flags of reduced spawns -> exclusive prefix
     i64 *ins;         // insertion position of a new key, -1 when matched
-    unsigned *hist;   // radix histograms (2^bits per sorting block)
+    unsigned *hist;   // radix histograms (2^bits per sorting block, of as many as the spawn buffer can have)
     Record *ring;     // per-step records
     // simulated distribution (Sec. III), allocated only with N_p > 1
     unsigned short *owner;  // processor of each list entry at this iteration
