@@ -112,7 +112,7 @@ __device__ __forceinline__ void count_equal(PairCount &c, unsigned d, const unsi
 // by integer logic: nb operations per 32 iterations of a pair, two more for
 // the carry-save columns that replace three of four population counts (8
 // issue slots each); the next group's planes are copied meanwhile.  3,813
-// excitors, 4,096 iterations, 32 processors: 0.72 ms (19.2 ms comparing and
+// excitors, 4,096 iterations, 32 processors: 0.71 ms (19.2 ms comparing and
 // adding one owner at a time).
 template <typename V>
 __global__ void __launch_bounds__(256) k_pairs(const V *planes, i64 n, i64 npad, int nb, i64 t_max, const i64 *ck,

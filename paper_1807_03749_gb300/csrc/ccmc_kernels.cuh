@@ -1016,7 +1016,7 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         double coef_hf, death_x;
         RoundCut hf_cut;
         int n, nbk, bshift;
-        bool n0_neg, n0_zero, hf_ok;
+        bool n0_neg, n0_zero, hf_ok, timed_out;
     } ss;
     if (threadIdx.x < 8) {
         smag[threadIdx.x] = st->mag[threadIdx.x];
@@ -1041,8 +1041,10 @@ __device__ __forceinline__ void d_sample(const SysDev &s, const ListView &L, Dev
         ss.death_x = st->hf_death;
         ss.hf_cut = st->hf_cut;
         ss.hf_ok = st->hf_ok != 0;
+        ss.timed_out = (st->err & ERRB_TIMEOUT) != 0;
     }
     __syncthreads();
+    if (ss.timed_out) return;
     AttQueue &q = sw.q;
     RecStage &rb = sw.rs;
     int wn = 0, hn = 0, qn = 0, rn = 0;   // warp-uniform queue fills
@@ -1317,7 +1319,9 @@ __device__ __forceinline__ void d_attempts(const SysDev &s, const ListView &L, D
 {
     // the cluster attempts of a runaway population are not run (their
     // packed count may have wrapped); the step reports the error instead
-    if ((st->err & ERRB_RUNAWAY) || st->cl_att > (double)p.work_cap) {
+    const unsigned before = st->err;
+    if (before & ERRB_TIMEOUT) return;
+    if ((before & ERRB_RUNAWAY) || st->cl_att > (double)p.work_cap) {
         if (threadIdx.x == 0 && blockIdx.x == 0) atomicOr(&st->err, (unsigned)ERRB_RUNAWAY);
         return;
     }
@@ -1972,19 +1976,17 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
 }
 
 // ---------------------------------------------------------------------------
-// Launcher
-// ---------------------------------------------------------------------------
-
-
-// ---------------------------------------------------------------------------
 // Kernels: each block serves replica blockIdx.y (the list kernels: the
 // replicas of its shares) of an array of per-replica
 // arguments (one entry for a single context, many for a batch).
 // ---------------------------------------------------------------------------
 
-// (Both return if a team's wait ran out, in this step or an earlier one.  In
-// the launches with teams the bit can be set meanwhile, so one thread reads it
-// for its block.)
+// Every kernel returns if a team's wait ran out, in this step or an earlier one.
+// Only the launches with teams can set the bit meanwhile: there one thread reads
+// it for its block (RETURN_IF_TIMED_OUT).  The bit is read along with what the
+// kernel reads first anyway; read ahead of it, it cost each kernel a memory
+// latency (50 steps of the 38-orbital gas between restore and read: 2.57 ms,
+// 2.63 with the bit read ahead).
 #define REPLICA                               \
     const StepArgs &a = A[blockIdx.y];        \
     if (a.st->err & ERRB_TIMEOUT) return;     \
@@ -1993,17 +1995,20 @@ __device__ __forceinline__ void d_finalize(DevStep *st, const RunParams &p, cons
 // the replica's arguments copied to shared memory (hot kernels)
 #define REPLICA_SMEM                                                              \
     __shared__ StepArgs a_sm;                                                     \
-    __shared__ unsigned err_sm;                                                   \
     {                                                                             \
-        if (threadIdx.x == 0) err_sm = A[blockIdx.y].st->err;                     \
         const u64 *src_ = (const u64 *)&A[blockIdx.y];                            \
         u64 *dst_ = (u64 *)&a_sm;                                                 \
         for (int q_ = threadIdx.x; q_ < (int)(sizeof(StepArgs) / 8); q_ += blockDim.x) dst_[q_] = src_[q_]; \
     }                                                                             \
     __syncthreads();                                                              \
-    if (err_sm & ERRB_TIMEOUT) return;                                            \
     const StepArgs &a = a_sm;                                                     \
     const int cur_ = a.st->cur
+
+#define RETURN_IF_TIMED_OUT                                                       \
+    __shared__ unsigned err_sm;                                                   \
+    if (threadIdx.x == 0) err_sm = a.st->err;                                     \
+    __syncthreads();                                                              \
+    if (err_sm & ERRB_TIMEOUT) return
 
 // Kernels that depend on neither kind nor precision (defined in ccmc_step.cu).
 __global__ void __launch_bounds__(1024) k_sample_plan(const StepArgs *__restrict__ A, int nrep, FlatPlan fp,
@@ -2162,14 +2167,15 @@ __device__ __forceinline__ bool next_share(Shares &S, int nrep, int most, U unit
 }
 
 // a replica's arguments copied to shared memory; false if a team's wait ran
-// out for it (as in REPLICA_SMEM).  All threads of the block call.
+// out for it.  All threads of the block call.
 __device__ __forceinline__ bool load_replica(StepArgs &a, const StepArgs &from, unsigned &err)
 {
     __syncthreads();   // the replica before is done
-    if (threadIdx.x == 0) err = from.st->err;
     const u64 *src = (const u64 *)&from;
     u64 *dst = (u64 *)&a;
     for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / 8); q += blockDim.x) dst[q] = src[q];
+    __syncthreads();
+    if (threadIdx.x == 0) err = a.st->err;
     __syncthreads();
     return !(err & ERRB_TIMEOUT);
 }
@@ -2209,6 +2215,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_scan(const StepArgs *__rest
     } else {
         REPLICA_SMEM;
         const i64 b = scan_blocks(a.st->n_occ);
+        RETURN_IF_TIMED_OUT;
         const Team t = {(int)blockIdx.x, (int)(b < most ? b : most)};
         if (t.id < t.n) d_scan<R, GAS>(a, t, sm);
     }
@@ -2263,7 +2270,6 @@ __global__ void __launch_bounds__(WORK_THREADS, SAMPLE_BLOCKS_PER_SM) k_sample_f
             have = r;
         }
         const StepArgs &a = a_sm;
-        if (a.st->err & ERRB_TIMEOUT) continue;   // (no block sets it in this launch)
         const int v0 = fp.vstart[r];
         d_sample<R, GAS, DIST>(a.s, a.list[a.st->cur], a.st, a.p, a.wa, a.sp, a.cl, enum_base, v - v0,
                                fp.vstart[r + 1] - v0, ((SampWarp *)dyn_smem)[threadIdx.x >> 5]);
@@ -2373,6 +2379,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *
     } else {
         REPLICA_SMEM;
         const i64 b = annihilate_blocks(a);
+        RETURN_IF_TIMED_OUT;
         const Team t = {(int)blockIdx.x, (int)(b < most ? b : most)};
         if (t.id < t.n) d_annihilate<R, GAS>(a, t, as, what, S, sm, s_last);
     }
