@@ -2030,7 +2030,7 @@ void launch_local_table(const StepArgs *A, int K, dim3 grid, cudaStream_t sm);
 // entries among 200 small ones to one block: 32.5 ms a step, now 1.06 (one of
 // 95,000 entries: 1.27 and 0.42 ms).  Where equal shares were right it costs
 // the working out, some 3 us a launch: 64 replicas of 18,000 entries 0.951 and
-// 0.959 ms a step, 700 of 280 entries 0.65 and 0.69 ms.
+// 0.956 ms a step, 700 of 280 entries 0.65 and 0.685 ms.
 //
 // (All that is kept between replicas is in shared memory: in registers it
 // would spill in the loops of the replica's own work.)
@@ -2039,7 +2039,7 @@ struct Shares {
     i64 sm[32], want, give;       // units of the replicas that want several blocks, blocks for them
     int smi[32], kept[KEPT], list[SCAN_THREADS];
     int first, hands, full, per;  // blocks before those left over, these, rounds of these, blocks each in the last round
-    int stage, base, rank, q, count;
+    int stage, base, rank, q, count;   // (stage 2: no replica wants several blocks)
     int rep, tail;                // the replica to do, the one of the last round
     Team team, tail_team;
 };
@@ -2075,13 +2075,15 @@ __device__ __forceinline__ void shares_init(Shares &S, int nrep, int most, U uni
     v = block_sum(v, S.sm);
     const i64 want = v >> 24, ones = v & ((1 << 24) - 1), give = want + ones <= B ? want : B * want / (want + ones);
     if (tid == 0) {
-        S.stage = S.base = S.rank = S.q = S.count = 0;
+        S.stage = want ? 0 : 2;
+        S.base = S.rank = S.q = S.count = 0;
         S.tail = -1;
         S.want = want;
         S.give = give;
     }
+    if (want == 0) return;
     int taken = 0, teams = 0;
-    for (int base = 0; want > 0 && base < nrep; base += SCAN_THREADS) {
+    for (int base = 0; base < nrep; base += SCAN_THREADS) {
         const int r = base + tid, n = r < nrep ? share_at(units_at(S, r, units_of), want, give, most) : 0;
         int tot;   // blocks, teams << 16
         const int at = taken + (block_incl_scan(n ? n | (1 << 16) : 0, S.smi, tot) & 0xFFFF) - n;
@@ -2108,6 +2110,17 @@ __device__ __forceinline__ bool next_share(Shares &S, int nrep, int most, U unit
 {
     const int id = (int)blockIdx.x, tid = threadIdx.x;
     __syncthreads();
+    if (S.stage == 2) {
+        const int r = S.q + id;
+        __syncthreads();
+        if (tid == 0) {
+            S.rep = r;
+            S.team = Team{0, 1};
+            S.q += (int)gridDim.x;
+        }
+        __syncthreads();
+        return r < nrep;
+    }
     if (S.stage == 0) {
         const int have = S.count;
         __syncthreads();
@@ -2295,12 +2308,12 @@ struct AnnihilateShape {
 // records in the spawn buffer
 __device__ __forceinline__ i64 spawned_of(const StepArgs &a) { return a.st->n_sp < a.sp.cap ? a.st->n_sp : a.sp.cap; }
 
-// Blocks of the annihilation: up to a tile of records one block, else one per
-// 1,024; one per 1,024 list entries.  (n_step, not n_occ: a block that starts
-// after the last one has finished the step must see the same team.)
-__device__ __forceinline__ i64 annihilate_blocks(const StepArgs &a)
+// Blocks of the annihilation of nsp records: up to a tile one block, else one
+// per 1,024; one per 1,024 list entries.  (n_step, not n_occ: a block that
+// starts after the last one has finished the step must see the same team.)
+__device__ __forceinline__ i64 annihilate_blocks(const DevStep *st, i64 nsp)
 {
-    const i64 bs = sort_blocks(spawned_of(a)), bm = (a.st->n_step + 2 * SCAN_THREADS - 1) / (2 * SCAN_THREADS);
+    const i64 bs = sort_blocks(nsp), bm = (st->n_step + 2 * SCAN_THREADS - 1) / (2 * SCAN_THREADS);
     return bs > bm ? bs : (bm < 1 ? 1 : bm);
 }
 
@@ -2372,13 +2385,14 @@ __global__ void __launch_bounds__(SCAN_THREADS, 2) k_annihilate(const StepArgs *
         __shared__ Shares W;
         __shared__ StepArgs a;
         __shared__ unsigned err;
-        const auto units = [&](int r) { return annihilate_blocks(A[r]); };
+        // (records past the buffer's capacity included: one read less)
+        const auto units = [&](int r) { return annihilate_blocks(A[r].st, A[r].st->n_sp); };
         shares_init(W, nrep, most, units);
         while (next_share(W, nrep, most, units))
             if (load_replica(a, A[W.rep], err)) d_annihilate<R, GAS>(a, W.team, as, what, S, sm, s_last);
     } else {
         REPLICA_SMEM;
-        const i64 b = annihilate_blocks(a);
+        const i64 b = annihilate_blocks(a.st, spawned_of(a));
         RETURN_IF_TIMED_OUT;
         const Team t = {(int)blockIdx.x, (int)(b < most ? b : most)};
         if (t.id < t.n) d_annihilate<R, GAS>(a, t, as, what, S, sm, s_last);

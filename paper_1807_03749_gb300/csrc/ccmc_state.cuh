@@ -76,9 +76,11 @@ struct DevStep {
     u64 iter;
     double shift;
     i64 n_occ;          // list size at the start of the step
-    // (with n_occ: every kernel of a step reads the three first)
+    // (in one cache line with n_occ: what the kernels of a step read first)
     unsigned err;
     int cur;            // list buffer holding the current list
+    i64 n_sp;           // spawned records appended (may exceed capacity on overflow)
+    i64 n_step;         // list size at the start of the step under way (n_occ changes at its end)
     i64 ntot, n0, nex, n_sel, fnc_attempts;
     double mag[8];      // |A_s| of a cluster of size s
     double cmag[8];     // |A_s| / n_att(s): magnitude of one attempt's coefficient
@@ -86,14 +88,12 @@ struct DevStep {
     int bucket_shift;   // selection buckets cover 2^bucket_shift positions each
     unsigned wait_limit;   // polls after which a team's wait gives up (0: the default)
     i64 nbuckets;
-    i64 n_sp;           // spawned records appended (may exceed capacity on overflow)
     u64 cl_packed;      // (clusters << CL_SHIFT) | attempts of buffered clusters
     i64 n_attempts;
     i64 n_keys;         // distinct keys after the reduction
     i64 kept_list, kept_new;
     i64 ntot_after;
     i64 n_start;        // list size at the start of the latest finished step
-    i64 n_step;         // list size at the start of the step under way (n_occ changes at its end)
     double cl_att;      // attempts of the buffered clusters (runaway check; exact below 2^53)
     int kshift;         // key buckets cover 2^kshift keys each
     int scan_blocks;    // blocks of the step's list scan (E_num partials they wrote)
